@@ -100,15 +100,24 @@ enum Epi : int {
   EPI_SILU_GRAD = 3,  // C = acc * silu'(aux)
 };
 
-// C[M,N] = A[M,K] * B[K,N]   (B row-major [K][N], e.g. a weight W[in][out])
+// Rows gathered into a product's sums before its epilogue: row m of the output
+// gets p[i0[m] * ld + n] + p[i1[m] * ld + off1 + n] added (p null: nothing).
+struct RowAdd {
+  const float* p = nullptr;
+  int64_t ld = 0, off1 = 0;
+  const int32_t *i0 = nullptr, *i1 = nullptr;
+};
+
+// C[M,N] = epi(A[M,K] * B[K,N] + bias + add)   (B row-major [K][N], e.g. a weight W[in][out])
 xmgn_status gemm_nn_f32(const RowSrc& A, int64_t M, const float* B, int N, const float* bias,
                         float* C, int64_t ldc, int epi, float* pre, const float* aux,
-                        cudaStream_t s);
+                        cudaStream_t s, const RowAdd& add = RowAdd{});
 // C[M,N] = A[M,K] * B^T      (B row-major [N][K]; dX = dZ W^T with W[in][out], N=in, K=out)
 xmgn_status gemm_nt_f32(const RowSrc& A, int64_t M, const float* B, int N, float* C, int64_t ldc,
                         int epi, const float* aux, cudaStream_t s);
 // G[K1,N] = A^T B over M rows, written (not added) into G (row-major, ld N);
-// deterministic two-level reduction through `part` scratch.
+// deterministic two-level reduction through `part` scratch (its size covers
+// every product of at most K1 x N).
 size_t gemm_tn_part_elems(int64_t M, int K1, int N);
 xmgn_status gemm_tn_f32(const RowSrc& A, int64_t M, const float* B, int64_t ldb, int N, float* G,
                         float* part, cudaStream_t s);

@@ -1,9 +1,16 @@
-// FP32 "plain" form of the model: eqs. (1)-(4) evaluated literally, layer by
-// layer, with CUDA-core fp32 GEMMs over gathered rows (the edge MLP input
-// [h_i, h_j, e_ij] is never materialised, rows are gathered inside the GEMM),
-// LayerNorm kernels (the edge one also forms the receiver sums of eq. (2)),
-// and CSR/CSC segmented sums in the backward.  Per-layer checkpoints hold
-// h^l, e^l and a^l; the backward recomputes each MLP's activations.
+// FP32 "plain" form of the model: eqs. (1)-(4) layer by layer with CUDA-core
+// fp32 GEMMs, LayerNorm kernels (the edge one also forms the receiver sums of
+// eq. (2)), and CSR/CSC segmented sums in the backward.  Per-layer checkpoints
+// hold h^l, e^l and a^l; the backward recomputes each MLP's activations.
+//
+// The first edge layer is split by its input blocks, [h_i, h_j, e_ij] W1 =
+// h_i W1_r + h_j W1_s + e_ij W1_e: the node blocks are applied once per node
+// (P = h [W1_r | W1_s], E/n = 7 times fewer rows than edges) and the edge
+// product gathers two rows of P in its epilogue.  The backward sums dZ1 over
+// every node's received and sent edges first (S = [S_r | S_s]) and applies the
+// transposed blocks per node: dh += S [W1_r | W1_s]^T, dW1_r = h^T S_r, dW1_s =
+// h^T S_s.  Per edge and layer that leaves 8 H^2 multiply-adds (forward and
+// backward) of the 16 H^2 that the unsplit form does.
 //
 // The same code is the wide BF16 path (hidden widths other than 128): with
 // Gemm::tc set, every product runs on the tensor cores with bf16 operands
@@ -33,6 +40,7 @@ struct F32Ws {
   float* nfeat;  // node-encoder inputs when Fourier features are appended
   float *feat, *Z1, *A1, *Z2, *dZ2, *dZ1, *elast;
   float *dy, *dh, *dagg, *de, *dhr, *dhs, *grad;
+  float *P, *S;  // node projections h [W1_r | W1_s] and per-node sums of dZ1 [received | sent], n x 2H
   float *tnpart, *cspart, *lnpart, *losspart;
   void* wide;  // tensor-core GEMM scratch (wide BF16 path only)
 };
@@ -68,10 +76,12 @@ void f32_ws_layout(Arena& A, const ParamPlan& p, int64_t n, int64_t E, F32Ws& w,
   w.dh = A.take<float>(size_t(n) * H);
   w.dagg = A.take<float>(size_t(n) * H);
   w.de = A.take<float>(size_t(E) * H);
-  w.dhr = A.take<float>(size_t(E) * H);
-  w.dhs = A.take<float>(size_t(E) * H);
+  w.dhr = tc ? A.take<float>(size_t(E) * H) : nullptr;
+  w.dhs = tc ? A.take<float>(size_t(E) * H) : nullptr;
+  w.P = tc ? nullptr : A.take<float>(size_t(n) * 2 * H);
+  w.S = tc ? nullptr : A.take<float>(size_t(n) * 2 * H);
   w.grad = A.take<float>(size_t(p.total));
-  size_t tn = gemm_tn_part_elems(R, 3 * H, H);
+  size_t tn = gemm_tn_part_elems(R, wide_kmax(p), H);
   w.tnpart = A.take<float>(tn);
   w.cspart = A.take<float>(colsum_part_elems(R, H));
   w.lnpart = A.take<float>(ln_bwd_part_elems(H));
@@ -108,9 +118,11 @@ xmgn_status mlp_fwd_wide(const WideScratch& x, const MlpOff& o, const float* P, 
 
 xmgn_status mlp_fwd(const Gemm& gm, const MlpOff& o, const float* P, const RowSrc& X, int64_t M, float* A1,
                     float* Z2, float* Y, const float* resid_in, float* resid_out, cudaStream_t s,
-                    const Agg& agg = Agg{}) {
+                    const Agg& agg = Agg{}, const RowAdd& add = RowAdd{}) {
   if (gm.tc) return mlp_fwd_wide(gm.w, o, P, X, M, Y, resid_in, resid_out, s, agg);
-  XMGN_TRY(gemm_nn_f32(X, M, P + o.W1, o.hid, P + o.b1, A1, o.hid, EPI_SILU, nullptr, nullptr, s));
+  // split edge form: X holds the edge states only, W1_e is the last row block of W1
+  const float* W1 = P + o.W1 + (add.p ? int64_t(o.in - X.K) * o.hid : 0);
+  XMGN_TRY(gemm_nn_f32(X, M, W1, o.hid, P + o.b1, A1, o.hid, EPI_SILU, nullptr, nullptr, s, add));
   if (!o.ln) {
     return gemm_nn_f32(rows1(A1, o.hid, o.hid), M, P + o.W2, o.out, P + o.b2, Y, o.out, EPI_STORE, nullptr,
                        nullptr, s);
@@ -152,11 +164,16 @@ xmgn_status mlp_bwd_wide(const WideScratch& x, const MlpOff& o, const float* P, 
 
 // Backward of Y = MLP(X) given dY = dY1 + dY2[idx2]; writes every gradient of
 // the MLP into g and leaves dZ1 (gradient at the first layer's output) in w.dZ1.
+// In the split edge form (add.p set: X the edge states, P_r and P_s rows gathered)
+// only the W1_e block of dW1 is written here, and not db1: the caller forms the
+// rest from the per-node sums of dZ1.
 xmgn_status mlp_bwd(const Gemm& gm, const MlpOff& o, const float* P, const RowSrc& X, int64_t M, const float* dY1,
-                    const float* dY2, const int32_t* idx2, float* g, F32Ws& w, cudaStream_t s) {
+                    const float* dY2, const int32_t* idx2, float* g, F32Ws& w, cudaStream_t s,
+                    const RowAdd& add = RowAdd{}) {
   if (gm.tc) return mlp_bwd_wide(gm.w, o, P, X, M, dY1, dY2, idx2, g, w, s);
   const int H = o.hid;
-  XMGN_TRY(gemm_nn_f32(X, M, P + o.W1, H, P + o.b1, w.A1, H, EPI_SILU, w.Z1, nullptr, s));
+  const int64_t w1 = o.W1 + (add.p ? int64_t(o.in - X.K) * H : 0);
+  XMGN_TRY(gemm_nn_f32(X, M, P + w1, H, P + o.b1, w.A1, H, EPI_SILU, w.Z1, nullptr, s, add));
   const float* dZ2 = dY1;
   if (o.ln) {
     XMGN_TRY(gemm_nn_f32(rows1(w.A1, H, H), M, P + o.W2, o.out, P + o.b2, w.Z2, o.out, EPI_STORE, nullptr, nullptr,
@@ -168,8 +185,24 @@ xmgn_status mlp_bwd(const Gemm& gm, const MlpOff& o, const float* P, const RowSr
   XMGN_TRY(gemm_tn_f32(rows1(w.A1, H, H), M, dZ2, o.out, o.out, g + o.W2, w.tnpart, s));
   XMGN_TRY(colsum_f32(dZ2, M, o.out, o.out, g + o.b2, w.cspart, s));
   XMGN_TRY(gemm_nt_f32(rows1(dZ2, o.out, o.out), M, P + o.W2, H, w.dZ1, H, EPI_SILU_GRAD, w.Z1, s));
-  XMGN_TRY(gemm_tn_f32(X, M, w.dZ1, H, H, g + o.W1, w.tnpart, s));
-  XMGN_TRY(colsum_f32(w.dZ1, M, H, H, g + o.b1, w.cspart, s));
+  XMGN_TRY(gemm_tn_f32(X, M, w.dZ1, H, H, g + w1, w.tnpart, s));
+  if (!add.p) XMGN_TRY(colsum_f32(w.dZ1, M, H, H, g + o.b1, w.cspart, s));
+  return XMGN_OK;
+}
+
+// P = h [W1_r | W1_s] of an edge MLP (n x 2H) and the row gather that adds
+// P_r[receiver] + P_s[sender] to the edge product.
+xmgn_status node_projections(const MlpOff& o, const float* P, const float* h, const xmgn_graph& g, float* out,
+                             RowAdd& add, cudaStream_t s) {
+  const int H = o.hid;
+  for (int b = 0; b < 2; ++b)
+    XMGN_TRY(gemm_nn_f32(rows1(h, H, H), g.n_nodes, P + o.W1 + int64_t(b) * H * H, H, nullptr, out + b * H, 2 * H,
+                         EPI_STORE, nullptr, nullptr, s));
+  add.p = out;
+  add.ld = 2 * H;
+  add.off1 = H;
+  add.i0 = g.recv;
+  add.i1 = g.col;
   return XMGN_OK;
 }
 
@@ -224,12 +257,19 @@ xmgn_status f32_forward(const ParamPlan& p, const float* P, const xmgn_graph& g,
     float* el = c.e + size_t(l) * E * H;
     float* en = (l + 1 < p.L) ? c.e + size_t(l + 1) * E * H : w.elast;
     float* agg = c.agg + size_t(l) * n * H;
-    RowSrc X = rows1(hl, H, H, g.recv);                          // eq. (1): [h_i, h_j, e_ij]
-    rows_add(X, hl, H, H, g.col);
-    rows_add(X, el, H, H);
+    RowSrc X;                                                     // eq. (1): [h_i, h_j, e_ij]
+    RowAdd add;
+    if (tc) {
+      X = rows1(hl, H, H, g.recv);
+      rows_add(X, hl, H, H, g.col);
+      rows_add(X, el, H, H);
+    } else {
+      X = rows1(el, H, H);
+      XMGN_TRY(node_projections(p.edge[l], P, hl, g, w.P, add, s));
+    }
     Agg ag;                                                       // eq. (2), fused
     ag.row_ptr = g.row_ptr, ag.n = n, ag.out = agg;
-    XMGN_TRY(mlp_fwd(gm, p.edge[l], P, X, E, w.A1, w.Z2, nullptr, el, en, s, ag));
+    XMGN_TRY(mlp_fwd(gm, p.edge[l], P, X, E, w.A1, w.Z2, nullptr, el, en, s, ag, add));
     RowSrc Xn = rows1(hl, H, H);                                  // eq. (3): [h_i, a_i]
     rows_add(Xn, agg, H, H);
     XMGN_TRY(mlp_fwd(gm, p.node[l], P, Xn, n, w.A1, w.Z2, nullptr, hl, hn, s));
@@ -297,10 +337,17 @@ xmgn_status f32_backward(const ParamPlan& p, const float* P, const xmgn_graph& g
       XMGN_TRY(gemm_nt_f32(rows1(w.dZ1, H, H), n, P + on.W1, H, w.dh, H, EPI_ACCUM, nullptr, s));
     }
     // edge update: e' = e + m, a_i = sum m_ij  ->  dm = de' + da[recv]
-    RowSrc X = rows1(hl, H, H, g.recv);
-    rows_add(X, hl, H, H, g.col);
-    rows_add(X, el, H, H);
-    XMGN_TRY(mlp_bwd(gm, oe, P, X, E, w.de, w.dagg, g.recv, G, w, s));
+    RowSrc X;
+    RowAdd add;
+    if (tc) {
+      X = rows1(hl, H, H, g.recv);
+      rows_add(X, hl, H, H, g.col);
+      rows_add(X, el, H, H);
+    } else {
+      X = rows1(el, H, H);
+      XMGN_TRY(node_projections(oe, P, hl, g, w.P, add, s));
+    }
+    XMGN_TRY(mlp_bwd(gm, oe, P, X, E, w.de, w.dagg, g.recv, G, w, s, add));
     if (gm.tc) {  // dZ1 [W1_r; W1_s; W1_e]^T, one product per block
       WideOut o;
       o.n = 3;
@@ -310,13 +357,23 @@ xmgn_status f32_backward(const ParamPlan& p, const float* P, const xmgn_graph& g
       o.C[2] = w.de, o.ldc[2] = H, o.accum[2] = 1;
       XMGN_TRY(dz1_w1t_wide(gm.w, E, H, o, s));
     } else {
-      XMGN_TRY(gemm_nt_f32(rows1(w.dZ1, H, H), E, P + oe.W1, H, w.dhr, H, EPI_STORE, nullptr, s));
-      XMGN_TRY(gemm_nt_f32(rows1(w.dZ1, H, H), E, P + oe.W1 + int64_t(H) * H, H, w.dhs, H, EPI_STORE, nullptr, s));
+      // S = per-node sums of dZ1 over received and sent edges, then per node and block b of W1:
+      // dh += S_b W1_b^T, dW1_b = h^T S_b; db1 = column sums of S_r (every edge has one receiver)
+      XMGN_TRY(seg_sum_rows_f32(w.dZ1, H, g.row_ptr, n, H, w.S, 2 * H, false, s));
+      XMGN_TRY(seg_sum_cols_f32(w.dZ1, H, g.row_ptr, g.csc_perm, n, H, w.S + H, 2 * H, false, s));
+      for (int b = 0; b < 2; ++b) {
+        const int64_t wb = oe.W1 + int64_t(b) * H * H;
+        XMGN_TRY(gemm_nt_f32(rows1(w.S + b * H, 2 * H, H), n, P + wb, H, w.dh, H, EPI_ACCUM, nullptr, s));
+        XMGN_TRY(gemm_tn_f32(rows1(hl, H, H), n, w.S + b * H, 2 * H, H, G + wb, w.tnpart, s));
+      }
+      XMGN_TRY(colsum_f32(w.S, n, H, 2 * H, G + oe.b1, w.cspart, s));
       XMGN_TRY(gemm_nt_f32(rows1(w.dZ1, H, H), E, P + oe.W1 + 2 * int64_t(H) * H, H, w.de, H, EPI_ACCUM, nullptr,
                            s));
     }
-    XMGN_TRY(seg_sum_rows_f32(w.dhr, H, g.row_ptr, n, H, w.dh, H, true, s));
-    XMGN_TRY(seg_sum_cols_f32(w.dhs, H, g.row_ptr, g.csc_perm, n, H, w.dh, H, true, s));
+    if (tc) {
+      XMGN_TRY(seg_sum_rows_f32(w.dhr, H, g.row_ptr, n, H, w.dh, H, true, s));
+      XMGN_TRY(seg_sum_cols_f32(w.dhs, H, g.row_ptr, g.csc_perm, n, H, w.dh, H, true, s));
+    }
   }
   XMGN_TRY(edge_features(xyz, g.gid, g.recv, g.col, E, w.feat, s));
   XMGN_TRY(mlp_bwd(gm, p.ee, P, rows1(w.feat, kInEdge, kInEdge), E, w.de, nullptr, nullptr, G, w, s));

@@ -1,7 +1,7 @@
-// SIMT (CUDA-core, fp32) building blocks: tiled GEMMs over gathered row
-// sources, LayerNorm forward/backward, segmented sums over CSR/CSC, edge
-// features, masked MSE.  All reductions use fixed work assignment and fixed
-// summation order, so results are bit-reproducible.
+// SIMT (CUDA-core, fp32) building blocks beside the GEMMs (sgemm.cu):
+// LayerNorm forward/backward, segmented sums over CSR/CSC, edge features,
+// masked MSE.  All reductions use fixed work assignment and fixed summation
+// order, so results are bit-reproducible.
 #include <math.h>
 
 #include <initializer_list>
@@ -11,24 +11,7 @@
 namespace xmgn {
 
 namespace {
-constexpr int BT = 64;   // output tile edge
-constexpr int BK = 16;   // reduction step
 constexpr int kLnBlocksMax = 1024;  // LayerNorm-backward blocks, each writing one partial of dgamma, dbeta
-
-__device__ __forceinline__ float src_get(const RowSrc& A, int64_t r, int k) {
-#pragma unroll
-  for (int s = 0; s < 3; ++s) {
-    if (s < A.nseg) {
-      const RowSeg& g = A.s[s];
-      if (k < g.width) {
-        int64_t row = g.idx ? int64_t(g.idx[r]) : r;
-        return g.p[row * g.ld + k];
-      }
-      k -= g.width;
-    }
-  }
-  return 0.f;
-}
 
 // sum_{p < n} x[p * stride] as eight independent partial sums (p mod 8)
 // combined in a fixed order: deterministic, and eight loads in flight.
@@ -40,144 +23,6 @@ __device__ __forceinline__ float sum_strided(const float* __restrict__ x, int n,
     for (int q = 0; q < 8; ++q) s[q] += x[int64_t(p + q) * stride];
   for (int q = 0; p < n; ++p, ++q) s[q] += x[int64_t(p) * stride];
   return ((s[0] + s[1]) + (s[2] + s[3])) + ((s[4] + s[5]) + (s[6] + s[7]));
-}
-
-__device__ __forceinline__ float silu_f(float z) { return z / (1.f + __expf(-z)); }
-__device__ __forceinline__ float silu_grad_f(float z) {
-  float s = 1.f / (1.f + __expf(-z));
-  return s * (1.f + z * (1.f - s));
-}
-
-template <bool NT>
-__global__ void __launch_bounds__(256) gemm_nnt_kernel(RowSrc A, int64_t M, const float* __restrict__ B,
-                                                       int N, const float* __restrict__ bias,
-                                                       float* __restrict__ C, int64_t ldc, int epi,
-                                                       float* __restrict__ pre,
-                                                       const float* __restrict__ aux) {
-  __shared__ float As[BK][BT + 4];
-  __shared__ float Bs[BK][BT + 4];
-  const int K = A.K;
-  const int t = threadIdx.x, tx = t & 15, ty = t >> 4;
-  const int64_t m0 = int64_t(blockIdx.x) * BT;
-  const int n0 = blockIdx.y * BT;
-  float acc[4][4] = {};
-  for (int k0 = 0; k0 < K; k0 += BK) {
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      int idx = t + 256 * i;
-      int mm = idx >> 4, kk = idx & 15;
-      int64_t m = m0 + mm;
-      int k = k0 + kk;
-      As[kk][mm] = (m < M && k < K) ? src_get(A, m, k) : 0.f;
-      int nn = idx & 63, kb = idx >> 6;
-      int n = n0 + nn, kq = k0 + kb;
-      float bv = 0.f;
-      if (n < N && kq < K) bv = NT ? B[int64_t(n) * K + kq] : B[int64_t(kq) * N + n];
-      Bs[kb][nn] = bv;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int kk = 0; kk < BK; ++kk) {
-      float a[4], b[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) a[i] = As[kk][ty * 4 + i];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) b[j] = Bs[kk][tx * 4 + j];
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
-    }
-    __syncthreads();
-  }
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    int64_t m = m0 + ty * 4 + i;
-    if (m >= M) continue;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      int n = n0 + tx * 4 + j;
-      if (n >= N) continue;
-      float v = acc[i][j] + (bias ? bias[n] : 0.f);
-      float* c = C + m * ldc + n;
-      switch (epi) {
-        case EPI_STORE: *c = v; break;
-        case EPI_SILU:
-          if (pre) pre[m * ldc + n] = v;
-          *c = silu_f(v);
-          break;
-        case EPI_ACCUM: *c += v; break;
-        case EPI_SILU_GRAD: *c = acc[i][j] * silu_grad_f(aux[m * ldc + n]); break;
-      }
-    }
-  }
-}
-
-__global__ void __launch_bounds__(256) gemm_tn_kernel(RowSrc A, int64_t M, const float* __restrict__ B,
-                                                      int64_t ldb, int N, int64_t rows_per_chunk,
-                                                      float* __restrict__ part) {
-  __shared__ float As[BK][BT + 4];
-  __shared__ float Bs[BK][BT + 4];
-  const int K1 = A.K;
-  const int t = threadIdx.x, tx = t & 15, ty = t >> 4;
-  const int ntn = (N + BT - 1) / BT;
-  const int k10 = (blockIdx.x / ntn) * BT;
-  const int n0 = (blockIdx.x % ntn) * BT;
-  const int64_t r_begin = int64_t(blockIdx.y) * rows_per_chunk;
-  const int64_t r_end = min(M, r_begin + rows_per_chunk);
-  float acc[4][4] = {};
-  for (int64_t r0 = r_begin; r0 < r_end; r0 += BK) {
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      int idx = t + 256 * i;
-      int rr = idx >> 6, cc = idx & 63;
-      int64_t r = r0 + rr;
-      int k1 = k10 + cc, n = n0 + cc;
-      bool rv = r < r_end;
-      As[rr][cc] = (rv && k1 < K1) ? src_get(A, r, k1) : 0.f;
-      Bs[rr][cc] = (rv && n < N) ? B[r * ldb + n] : 0.f;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int rr = 0; rr < BK; ++rr) {
-      float a[4], b[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) a[i] = As[rr][ty * 4 + i];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) b[j] = Bs[rr][tx * 4 + j];
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
-    }
-    __syncthreads();
-  }
-  float* P = part + int64_t(blockIdx.y) * K1 * N;
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    int k1 = k10 + ty * 4 + i;
-    if (k1 >= K1) continue;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      int n = n0 + tx * 4 + j;
-      if (n < N) P[int64_t(k1) * N + n] = acc[i][j];
-    }
-  }
-}
-
-__global__ void reduce_chunks_kernel(const float* __restrict__ part, int nchunk, int64_t len,
-                                     float* __restrict__ out) {
-  for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < len;
-       i += int64_t(gridDim.x) * blockDim.x) {
-    out[i] = sum_strided(part + i, nchunk, len);
-  }
-}
-
-int tn_chunks(int64_t M) {
-  int64_t c = (M + 4095) / 4096;
-  if (c > 128) c = 128;
-  if (c < 1) c = 1;
-  return int(c);
 }
 
 // Column sums of one chunk of rows (eight loads in flight per thread).
@@ -729,45 +574,6 @@ __global__ void accum_kernel(float* __restrict__ dst, float* __restrict__ comp,
 }
 
 }  // namespace
-
-xmgn_status gemm_nn_f32(const RowSrc& A, int64_t M, const float* B, int N, const float* bias,
-                        float* C, int64_t ldc, int epi, float* pre, const float* aux,
-                        cudaStream_t s) {
-  if (M <= 0) return XMGN_OK;
-  dim3 grid(unsigned((M + BT - 1) / BT), unsigned((N + BT - 1) / BT));
-  gemm_nnt_kernel<false><<<grid, 256, 0, s>>>(A, M, B, N, bias, C, ldc, epi, pre, aux);
-  XMGN_LAUNCH_CHECK();
-  return XMGN_OK;
-}
-
-xmgn_status gemm_nt_f32(const RowSrc& A, int64_t M, const float* B, int N, float* C, int64_t ldc,
-                        int epi, const float* aux, cudaStream_t s) {
-  if (M <= 0) return XMGN_OK;
-  dim3 grid(unsigned((M + BT - 1) / BT), unsigned((N + BT - 1) / BT));
-  gemm_nnt_kernel<true><<<grid, 256, 0, s>>>(A, M, B, N, nullptr, C, ldc, epi, nullptr, aux);
-  XMGN_LAUNCH_CHECK();
-  return XMGN_OK;
-}
-
-size_t gemm_tn_part_elems(int64_t M, int K1, int N) {
-  return size_t(tn_chunks(M)) * size_t(K1) * size_t(N);
-}
-
-xmgn_status gemm_tn_f32(const RowSrc& A, int64_t M, const float* B, int64_t ldb, int N, float* G,
-                        float* part, cudaStream_t s) {
-  const int K1 = A.K;
-  const int nc = tn_chunks(M);
-  int64_t rpc = (M + nc - 1) / nc;
-  rpc = (rpc + BK - 1) / BK * BK;
-  if (rpc < BK) rpc = BK;
-  const int tiles = ((K1 + BT - 1) / BT) * ((N + BT - 1) / BT);
-  gemm_tn_kernel<<<dim3(tiles, nc), 256, 0, s>>>(A, M, B, ldb, N, rpc, part);
-  XMGN_LAUNCH_CHECK();
-  const int64_t len = int64_t(K1) * N;
-  reduce_chunks_kernel<<<grid_for(len, 256), 256, 0, s>>>(part, nc, len, G);
-  XMGN_LAUNCH_CHECK();
-  return XMGN_OK;
-}
 
 size_t colsum_part_elems(int64_t M, int N) { return size_t(colsum_chunks(M)) * size_t(N); }
 
