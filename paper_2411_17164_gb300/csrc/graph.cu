@@ -8,10 +8,16 @@
 // independent of thread scheduling.
 //
 // Search: uniform grid over the lattice bounding box, points counting-sorted
-// into cells, then for each point rings of cells at Chebyshev distance
-// r = 0, 1, 2, ... are scanned.  Any point outside rings 0..r differs by at
-// least r*c + 1 lattice units along some axis (c = cell edge), so the search
-// stops once the k-th best d^2 < (r*c + 1)^2.
+// into cells with their coordinates (16 bytes each), then for each point the
+// block of cells at Chebyshev distance <= 1 and after it rings r = 2, 3, ... are
+// scanned.  Any point outside the scanned block differs along some axis by at
+// least the distance from the point to that face of the block, so the search
+// stops once k candidates are nearer than the nearest face that has cells
+// behind it.
+//
+// The whole build runs on the stream with one host wait at its end: the grid
+// is laid out on the device from the bounding box, and the rows are emitted
+// only if they fit the caller's capacity, which the host reports afterwards.
 #include <math.h>
 
 #include "common.cuh"
@@ -66,203 +72,407 @@ __global__ void bbox_init_kernel(int32_t* bbox) {
   }
 }
 
+// Uniform grid of one reference set.
 struct Grid {
   int32_t lo[3];
-  int64_t c;      // cell edge in lattice units
-  int64_t g[3];   // cells per axis
+  int32_t c;     // cell edge in lattice units
+  int32_t g[3];  // cells per axis
+};
+constexpr int kMaxLevels = 16;
+struct LevelSizes {
+  int64_t n[kMaxLevels];
 };
 
-__device__ __forceinline__ int64_t cell_coord(int32_t q, int32_t lo, int64_t c) {
-  return (int64_t(q) - lo) / c;
+// Cells of a grid over n points.  On a surface the points of an occupied cell
+// grow as (n / cells)^(2/3) n^(1/3): two cells per point leave 2.5 points in an
+// occupied cell at 2k points but 10 at 200k and 18 at 1.25M, so the cells per
+// point grow with the square root of n up to six.  (Of the 6 n counters, the
+// scan and the clearing cost 20 us at 1.25M points; the search there reads 9
+// occupied cells per point.)
+__host__ __device__ inline int64_t cell_budget(int64_t n) {
+  double per = 2.0 * sqrt(double(n) / 8000.0);
+  if (per < 2.0) per = 2.0;
+  if (per > 6.0) per = 6.0;
+  const int64_t b = int64_t(per * double(n)) + 1024;
+  return b < (int64_t(1) << 30) ? b : (int64_t(1) << 30);
 }
 
-__global__ void cell_count_kernel(const int32_t* __restrict__ q, int64_t n, Grid G,
-                                  int64_t* __restrict__ cell_of, int32_t* __restrict__ cnt) {
+// The grid of every level (thread l: the first sizes.n[l] points) over the box
+// of all points: at most cell_budget cells.
+__global__ void grid_layout_kernel(const int32_t* __restrict__ bbox, LevelSizes sizes, int levels, Grid* __restrict__ out) {
+  const int l = threadIdx.x;
+  if (l >= levels) return;
+  const int64_t budget = cell_budget(sizes.n[l]);
+  double vol = 1.0;
+  Grid G;
+  for (int a = 0; a < 3; ++a) {
+    G.lo[a] = bbox[a];
+    vol *= double(int64_t(bbox[3 + a]) - bbox[a] + 1);
+  }
+  double c = cbrt(vol / double(budget - 1024));
+  if (c < 1) c = 1;
+  int64_t e = int64_t(ceil(c));
+  for (;;) {
+    int64_t tot = 1;
+    for (int a = 0; a < 3; ++a) {
+      const int64_t g = (int64_t(bbox[3 + a]) - bbox[a]) / e + 1;
+      G.g[a] = int32_t(g);
+      tot *= g;
+    }
+    if (tot <= budget) break;
+    e = e + e / 4 + 1;
+  }
+  G.c = int32_t(e);
+  out[l] = G;
+}
+
+__device__ __forceinline__ int cell_coord(int32_t q, int32_t lo, int32_t c) { return int(uint32_t(q - lo) / uint32_t(c)); }
+
+// Cell of every reference point, and its place among the cell's points.
+__global__ void cell_count_kernel(const int32_t* __restrict__ q, int64_t n, const Grid* __restrict__ grid,
+                                  int32_t* __restrict__ cell_of, int32_t* __restrict__ at, int32_t* __restrict__ cnt) {
+  const Grid G = *grid;
   for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n;
        i += int64_t(gridDim.x) * blockDim.x) {
-    int64_t cx = cell_coord(q[3 * i], G.lo[0], G.c);
-    int64_t cy = cell_coord(q[3 * i + 1], G.lo[1], G.c);
-    int64_t cz = cell_coord(q[3 * i + 2], G.lo[2], G.c);
-    int64_t cell = (cz * G.g[1] + cy) * G.g[0] + cx;
+    const int cx = cell_coord(q[3 * i], G.lo[0], G.c);
+    const int cy = cell_coord(q[3 * i + 1], G.lo[1], G.c);
+    const int cz = cell_coord(q[3 * i + 2], G.lo[2], G.c);
+    const int32_t cell = (cz * G.g[1] + cy) * G.g[0] + cx;
     cell_of[i] = cell;
-    atomicAdd(&cnt[cell], 1);
+    at[i] = atomicAdd(&cnt[cell], 1);
   }
 }
 
-__global__ void cell_scatter_kernel(const int64_t* __restrict__ cell_of, int64_t n,
-                                    const int64_t* __restrict__ start, int32_t* __restrict__ fill,
-                                    int32_t* __restrict__ sorted) {
+__global__ void cell_scatter_kernel(const int32_t* __restrict__ q, const int32_t* __restrict__ cell_of,
+                                    const int32_t* __restrict__ at, int64_t n, const int32_t* __restrict__ start,
+                                    int4* __restrict__ pts) {
   for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n;
-       i += int64_t(gridDim.x) * blockDim.x) {
-    int64_t c = cell_of[i];
-    int32_t off = atomicAdd(&fill[c], 1);
-    sorted[start[c] + off] = int32_t(i);
-  }
+       i += int64_t(gridDim.x) * blockDim.x)
+    pts[start[cell_of[i]] + at[i]] = make_int4(q[3 * i], q[3 * i + 1], q[3 * i + 2], int32_t(i));
 }
 
 __device__ __forceinline__ bool key_less(int64_t d1, int32_t j1, int64_t d2, int32_t j2) {
   return d1 < d2 || (d1 == d2 && j1 < j2);
 }
 
-// The k nearest reference points of lattice point i (excluding i itself),
-// ranked by (d^2, index), from the cell-sorted reference set; returns how
-// many were found (k unless the reference set is smaller).
-__device__ __forceinline__ int knn_point(const int32_t* __restrict__ q, const int32_t* __restrict__ sorted,
-                                         const int64_t* __restrict__ start, int k, const Grid& G, int32_t i,
-                                         int64_t* bd, int32_t* bj) {
-  const int64_t px = q[3 * i], py = q[3 * i + 1], pz = q[3 * i + 2];
-  const int64_t cx = (px - G.lo[0]) / G.c, cy = (py - G.lo[1]) / G.c, cz = (pz - G.lo[2]) / G.c;
-  int have = 0;
-  const int64_t rmax = max(G.g[0], max(G.g[1], G.g[2]));
-  for (int64_t r = 0; r <= rmax; ++r) {
-    for (int64_t dz = -r; dz <= r; ++dz) {
-      int64_t z = cz + dz;
-      if (z < 0 || z >= G.g[2]) continue;
-      for (int64_t dy = -r; dy <= r; ++dy) {
-        int64_t y = cy + dy;
-        if (y < 0 || y >= G.g[1]) continue;
-        bool face = (dz == -r || dz == r || dy == -r || dy == r);
-        int64_t step = face ? 1 : 2 * r;  // interior rows only touch the two x faces
-        for (int64_t dx = -r; dx <= r; dx += (step > 0 ? step : 1)) {
-          int64_t x = cx + dx;
-          if (x < 0 || x >= G.g[0]) continue;
-          int64_t cell = (z * G.g[1] + y) * G.g[0] + x;
-          for (int64_t s = start[cell], e = start[cell + 1]; s < e; ++s) {
-            int32_t j = sorted[s];
-            if (j == i) continue;
-            int64_t ddx = q[3 * j] - px, ddy = q[3 * j + 1] - py, ddz = q[3 * j + 2] - pz;
-            int64_t d = ddx * ddx + ddy * ddy + ddz * ddz;
-            if (have == k && !key_less(d, j, bd[k - 1], bj[k - 1])) continue;
-            int pos = have < k ? have : k - 1;
-            while (pos > 0 && key_less(d, j, bd[pos - 1], bj[pos - 1])) {
-              bd[pos] = bd[pos - 1];
-              bj[pos] = bj[pos - 1];
-              --pos;
-            }
-            bd[pos] = d;
-            bj[pos] = j;
-            if (have < k) ++have;
+// The KC best candidates of one lane, ascending by (d^2, index), in registers.
+template <int KC>
+struct Best {
+  int64_t d[KC];
+  int32_t j[KC];
+  __device__ __forceinline__ void clear() {
+#pragma unroll
+    for (int a = 0; a < KC; ++a) d[a] = INT64_MAX, j[a] = INT32_MAX;
+  }
+  __device__ __forceinline__ void insert(int64_t dn, int32_t jn) {
+    if (!key_less(dn, jn, d[KC - 1], j[KC - 1])) return;
+    bool lt = true;  // new key < slot a
+#pragma unroll
+    for (int a = KC - 1; a > 0; --a) {
+      const bool below = key_less(dn, jn, d[a - 1], j[a - 1]);
+      d[a] = below ? d[a - 1] : (lt ? dn : d[a]);
+      j[a] = below ? j[a - 1] : (lt ? jn : j[a]);
+      lt = below;
+    }
+    if (lt) d[0] = dn, j[0] = jn;
+  }
+  __device__ __forceinline__ void pop() {
+#pragma unroll
+    for (int a = 0; a + 1 < KC; ++a) d[a] = d[a + 1], j[a] = j[a + 1];
+    d[KC - 1] = INT64_MAX;
+    j[KC - 1] = INT32_MAX;
+  }
+};
+
+template <int G>
+__device__ __forceinline__ int group_get(uint32_t mask, int v, int l) {
+  if constexpr (G == 1) return v;
+  return __shfl_sync(mask, v, l, G);
+}
+
+// kNN among n_ref cell-sorted reference points.  QUERY false: of every
+// reference point, in cell order (itself excluded); true: of the points
+// q0..q1-1, which are not reference points but lie inside the grid.  A group
+// of G lanes serves a point: each lane finds the cell ranges of one (y, z) row of
+// the block (the cells of a row are neighbours in memory), then the lanes read
+// every range together, each keeping the best of what it read; the lists are
+// merged at the end.  Row i of the output is nbr[i*stride + off .. + k), -1 if
+// missing.  rcnt[j] counts the rows that list j; rank[slot] is the slot's place
+// among them (for the reverse edges).
+//
+// Bound by the latency of the dependent reads (range, then points).  Against a
+// thread per point with its candidate list in local memory, the cell ids read
+// first and the coordinates gathered: 114 -> 23 us at 2k points (eight lanes
+// per point), 185 -> 93 us at 200k, and 1.43 -> 0.77 ms for the three levels up
+// to 1.25M points.
+template <int KC, int G, bool QUERY>
+__global__ void __launch_bounds__(128) knn_kernel(const int32_t* __restrict__ q, const int4* __restrict__ pts,
+                                                  const int32_t* __restrict__ start, int64_t q0, int64_t q1, int k,
+                                                  const Grid* __restrict__ grid, int32_t* __restrict__ nbr,
+                                                  int64_t stride, int off, int32_t* __restrict__ rcnt,
+                                                  int32_t* __restrict__ rank) {
+  const Grid gr = *grid;
+  const int lane = threadIdx.x & 31, gl = lane % G;
+  const uint32_t mask = G == 1 ? 0u : ((G == 32 ? 0xffffffffu : ((1u << G) - 1u)) << (lane - gl));
+  for (int64_t t = q0 + (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) / G; t < q1;
+       t += int64_t(gridDim.x) * blockDim.x / G) {
+    int4 p;
+    if (QUERY)
+      p = make_int4(q[3 * t], q[3 * t + 1], q[3 * t + 2], int32_t(t));
+    else
+      p = pts[t];
+    const int cx = cell_coord(p.x, gr.lo[0], gr.c), cy = cell_coord(p.y, gr.lo[1], gr.c),
+              cz = cell_coord(p.z, gr.lo[2], gr.c);
+    Best<KC> best;
+    best.clear();
+    auto scan = [&](int s, int e) {
+      for (s += gl; s < e; s += G) {
+        const int4 c = pts[s];
+        const int32_t dx = c.x - p.x, dy = c.y - p.y, dz = c.z - p.z;
+        const int64_t d = int64_t(dx) * dx + int64_t(dy) * dy + int64_t(dz) * dz;
+        if (QUERY || c.w != p.w) best.insert(d, c.w);
+      }
+    };
+    for (int r = 1;; ++r) {
+      const int side = 2 * r + 1, rows = side * side;
+      const int x0 = max(cx - r, 0), x1 = min(cx + r, gr.g[0] - 1);
+      // this lane's row of the G rows from `base` on: one range, or the two end cells of an inner row
+      auto ranges = [&](int base) {
+        int4 v = make_int4(0, 0, 0, 0);
+        const int id = base + gl;
+        const int dy = id % side - r, dz = id / side - r;
+        const int y = cy + dy, z = cz + dz;
+        if (id < rows && y >= 0 && y < gr.g[1] && z >= 0 && z < gr.g[2]) {
+          const int32_t* row = start + (int64_t(z) * gr.g[1] + y) * gr.g[0];
+          if (r == 1 || dy == -r || dy == r || dz == -r || dz == r) {
+            v.x = row[x0];
+            v.y = row[x1 + 1];
+          } else {
+            if (cx - r >= 0) v.x = row[cx - r], v.y = row[cx - r + 1];
+            if (cx + r < gr.g[0]) v.z = row[cx + r], v.w = row[cx + r + 1];
           }
         }
+        return v;
+      };
+      int4 next = ranges(0);
+      for (int base = 0; base < rows; base += G) {
+        const int4 v = next;
+        if (base + G < rows) next = ranges(base + G);  // its loads are in flight while these rows are read
+#pragma unroll 1
+        for (int l = 0; l < G && base + l < rows; ++l) {
+          scan(group_get<G>(mask, v.x, l), group_get<G>(mask, v.y, l));
+          if (r > 1) scan(group_get<G>(mask, v.z, l), group_get<G>(mask, v.w, l));
+        }
+      }
+      // distance to the nearest face of the scanned block that has cells behind it
+      int64_t lim = INT64_MAX;
+      bool more = false;
+      const int cc[3] = {cx, cy, cz}, pp[3] = {p.x, p.y, p.z};
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        const int64_t rel = int64_t(pp[a]) - gr.lo[a];
+        if (cc[a] - r > 0) {
+          lim = min(lim, rel - int64_t(cc[a] - r) * gr.c + 1);
+          more = true;
+        }
+        if (cc[a] + r < gr.g[a] - 1) {
+          lim = min(lim, int64_t(cc[a] + r + 1) * gr.c - rel);
+          more = true;
+        }
+      }
+      if (!more) break;
+      int near = 0;
+#pragma unroll
+      for (int a = 0; a < KC; ++a) near += best.d[a] < lim * lim;
+#pragma unroll
+      for (int o = G / 2; o; o >>= 1) near += __shfl_xor_sync(mask, near, o, G);
+      if (near >= k) break;
+    }
+    for (int a = 0; a < k; ++a) {  // merge: the least head of the group's lists, k times
+      int64_t d = best.d[0];
+      int32_t j = best.j[0];
+#pragma unroll
+      for (int o = G / 2; o; o >>= 1) {
+        const int64_t d2 = __shfl_xor_sync(mask, d, o, G);
+        const int32_t j2 = __shfl_xor_sync(mask, j, o, G);
+        if (key_less(d2, j2, d, j)) d = d2, j = j2;
+      }
+      if (best.j[0] == j) best.pop();
+      if (gl == a % G) {
+        const int64_t slot = int64_t(p.w) * stride + off + a;
+        const bool found = j != INT32_MAX;
+        nbr[slot] = found ? j : -1;
+        if (found) rank[slot] = atomicAdd(&rcnt[j], 1);
       }
     }
-    if (have == k) {
-      int64_t lim = r * G.c + 1;
-      if (bd[k - 1] < lim * lim) break;
-    }
-  }
-  return have;
-}
-
-// kNN of every reference point among the reference points (visited in cell
-// order); row i of the output is nbr[i*stride + off .. + k), -1 if missing.
-__global__ void knn_search_kernel(const int32_t* __restrict__ q, const int32_t* __restrict__ sorted,
-                                  const int64_t* __restrict__ start, int64_t n, int k, Grid G,
-                                  int32_t* __restrict__ nbr, int64_t stride, int off) {
-  for (int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; t < n;
-       t += int64_t(gridDim.x) * blockDim.x) {
-    const int32_t i = sorted[t];
-    int64_t bd[kMaxK];
-    int32_t bj[kMaxK];
-    const int have = knn_point(q, sorted, start, k, G, i, bd, bj);
-    for (int a = 0; a < k; ++a) nbr[int64_t(i) * stride + off + a] = a < have ? bj[a] : -1;
   }
 }
 
-// kNN among the reference points of the query points q0..q1-1 (not in the
-// reference set; they must lie inside the grid).
-__global__ void knn_query_kernel(const int32_t* __restrict__ q, const int32_t* __restrict__ sorted,
-                                 const int64_t* __restrict__ start, int64_t q0, int64_t q1, int k, Grid G,
-                                 int32_t* __restrict__ nbr, int64_t stride, int off) {
-  for (int64_t i = q0 + int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < q1;
-       i += int64_t(gridDim.x) * blockDim.x) {
-    int64_t bd[kMaxK];
-    int32_t bj[kMaxK];
-    const int have = knn_point(q, sorted, start, k, G, int32_t(i), bd, bj);
-    for (int a = 0; a < k; ++a) nbr[i * stride + off + a] = a < have ? bj[a] : -1;
-  }
+template <bool QUERY, int G>
+void knn_launch_g(unsigned grid, cudaStream_t s, const int32_t* q, const int4* pts, const int32_t* start, int64_t q0,
+                  int64_t q1, int k, const Grid* gr, int32_t* nbr, int64_t stride, int off, int32_t* rcnt,
+                  int32_t* rank) {
+  if (k <= 3)
+    knn_kernel<3, G, QUERY><<<grid, 128, 0, s>>>(q, pts, start, q0, q1, k, gr, nbr, stride, off, rcnt, rank);
+  else if (k <= 6)
+    knn_kernel<6, G, QUERY><<<grid, 128, 0, s>>>(q, pts, start, q0, q1, k, gr, nbr, stride, off, rcnt, rank);
+  else if (k <= 8)
+    knn_kernel<8, G, QUERY><<<grid, 128, 0, s>>>(q, pts, start, q0, q1, k, gr, nbr, stride, off, rcnt, rank);
+  else if (k <= 16)
+    knn_kernel<16, G, QUERY><<<grid, 128, 0, s>>>(q, pts, start, q0, q1, k, gr, nbr, stride, off, rcnt, rank);
+  else
+    knn_kernel<kMaxK, G, QUERY><<<grid, 128, 0, s>>>(q, pts, start, q0, q1, k, gr, nbr, stride, off, rcnt, rank);
+}
+
+// Lanes per point: eight while that still leaves at most one wave of resident
+// threads (2k points: 47 us with one lane, 22 us with eight; beyond it the
+// merge and the lanes idle at the ends of short ranges cost more than the
+// parallel reads give: 200k points 97 against 130 us).
+template <bool QUERY>
+xmgn_status knn_launch(const int32_t* q, const int4* pts, const int32_t* start, int64_t q0, int64_t q1, int k,
+                       const Grid* gr, int32_t* nbr, int64_t stride, int off, int32_t* rcnt, int32_t* rank,
+                       cudaStream_t s) {
+  const int64_t n = q1 - q0;
+  if (n * 8 <= int64_t(num_sms()) * 2048)
+    knn_launch_g<QUERY, 8>(grid_for(n * 8, 128, 1 << 30), s, q, pts, start, q0, q1, k, gr, nbr, stride, off, rcnt, rank);
+  else
+    knn_launch_g<QUERY, 1>(grid_for(n, 128, 1 << 30), s, q, pts, start, q0, q1, k, gr, nbr, stride, off, rcnt, rank);
+  XMGN_LAUNCH_CHECK();
+  return XMGN_OK;
 }
 
 // ---- symmetrisation
-__global__ void sym_count_kernel(const int32_t* __restrict__ nbr, int64_t n, int k,
-                                 int32_t* __restrict__ cnt, uint32_t* err) {
+// Row i of the undirected graph = its own K slots and every j that lists i.
+// Reverse entries: slot t of point i names j = nbr[t]; i goes to place rank[t]
+// of j's list.
+__global__ void sym_rev_kernel(const int32_t* __restrict__ nbr, int64_t n, int k, const int64_t* __restrict__ rstart,
+                               const int32_t* __restrict__ rank, int32_t* __restrict__ rev) {
   for (int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; t < n * k;
        t += int64_t(gridDim.x) * blockDim.x) {
-    int32_t j = nbr[t];
-    if (j == -1) continue;  // empty slot
-    if (j < 0 || j >= n) {
-      dev_flag(err, DEV_ERR_GRAPH);
-      continue;
+    const int32_t j = nbr[t];
+    if (j >= 0) rev[rstart[j] + rank[t]] = int32_t(t / k);
+  }
+}
+
+// Sorts row i (ascending ids) and drops repeats: 16 lanes per row collect its
+// entries, every lane counts how many entries are less than its own and writes
+// it to that place (equal entries meet there and leave holes behind them), and
+// the filled places are closed up.  Rows of up to kRow entries stay in shared
+// memory, the two rows of a warp in step (their loops run to the longer one's
+// end: apart, the halves would take turns); longer ones, points that many
+// others list, are sorted on the global arrays.  out row i starts at rstart[i]
+// + K i.  Bound by the latency of the row's reads; 1.25M rows of 21 slots: 1216
+// us (a thread per row, insertion sort in global memory) -> 415 us.
+constexpr int kRow = 64;
+__global__ void __launch_bounds__(256) sym_sort_kernel(const int32_t* __restrict__ nbr, int64_t n, int k,
+                                                       const int64_t* __restrict__ rstart,
+                                                       const int32_t* __restrict__ rev, int32_t* __restrict__ out,
+                                                       int32_t* __restrict__ deg) {
+  __shared__ __align__(16) int32_t raw[16][kRow], srt[16][kRow];
+  const int lane = threadIdx.x & 31, l = lane & 15, gi = threadIdx.x >> 4, hs = lane & 16;
+  constexpr uint32_t kAll = 0xffffffffu;
+  auto half = [&](uint32_t m) { return (m >> hs) & 0xffffu; };  // this half's bits
+  for (int64_t i0 = int64_t(blockIdx.x) * 16 + (gi & ~1); i0 < n; i0 += int64_t(gridDim.x) * 16) {
+    const int64_t i = i0 + (gi & 1);
+    const bool in = i < n;
+    const int64_t r0 = in ? rstart[i] : 0, nr = in ? rstart[i + 1] - r0 : 0;
+    int32_t* const row = out + r0 + int64_t(k) * i;
+    int m = 0;
+    for (int a0 = 0; a0 < k; a0 += 16) {
+      const int32_t v = in && a0 + l < k ? nbr[i * k + a0 + l] : -1;
+      const uint32_t b = half(__ballot_sync(kAll, v >= 0));
+      const int at = m + __popc(b & ((1u << l) - 1u));
+      if (v >= 0 && at < kRow) raw[gi][at] = v;
+      m += __popc(b);
     }
-    atomicAdd(&cnt[j], 1);
-  }
-}
-
-__global__ void sym_own_kernel(const int32_t* __restrict__ nbr, int64_t n, int k,
-                               const int64_t* __restrict__ cstart, int32_t* __restrict__ cand,
-                               unsigned long long* __restrict__ fill) {
-  for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n;
-       i += int64_t(gridDim.x) * blockDim.x) {
-    for (int a = 0; a < k; ++a) cand[cstart[i] + a] = nbr[i * k + a];
-    fill[i] = (unsigned long long)(cstart[i] + k);
-  }
-}
-
-__global__ void sym_rev_kernel(const int32_t* __restrict__ nbr, int64_t n, int k,
-                               int32_t* __restrict__ cand, unsigned long long* __restrict__ fill) {
-  for (int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; t < n * k;
-       t += int64_t(gridDim.x) * blockDim.x) {
-    int32_t j = nbr[t];
-    if (j < 0 || j >= n) continue;
-    unsigned long long pos = atomicAdd(&fill[j], 1ull);
-    cand[pos] = int32_t(t / k);
-  }
-}
-
-__global__ void sym_sort_kernel(int32_t* __restrict__ cand, const int64_t* __restrict__ cstart,
-                                int64_t n, int32_t* __restrict__ deg) {
-  for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n;
-       i += int64_t(gridDim.x) * blockDim.x) {
-    int32_t* c = cand + cstart[i];
-    int64_t m = cstart[i + 1] - cstart[i];
-    for (int64_t a = 1; a < m; ++a) {  // insertion sort (rows are short)
-      int32_t v = c[a];
-      int64_t b = a - 1;
-      while (b >= 0 && c[b] > v) {
-        c[b + 1] = c[b];
-        --b;
+    const bool brief = m + nr <= kRow;
+    if (brief) {
+      for (int a = l; a < int(nr); a += 16) raw[gi][m + a] = rev[r0 + a];
+      m += int(nr);
+    } else {
+      m = 0;
+    }
+    const int mw = max(m, __shfl_xor_sync(kAll, m, 16));
+    for (int a = m + l; a < ((mw + 3) & ~3); a += 16) raw[gi][a] = INT32_MAX;  // less than nothing
+    for (int a = l; a < mw; a += 16) srt[gi][a] = -1;
+    __syncwarp();
+    for (int a0 = 0; a0 < mw; a0 += 16) {
+      const int a = a0 + l;
+      const int32_t x = a < m ? raw[gi][a] : -1;
+      int c = 0;
+      for (int b = 0; b < mw; b += 4) {
+        const int4 y = *reinterpret_cast<const int4*>(&raw[gi][b]);
+        c += (y.x < x) + (y.y < x) + (y.z < x) + (y.w < x);
       }
-      c[b + 1] = v;
+      if (a < m) srt[gi][c] = x;
     }
-    int32_t u = 0;
-    for (int64_t a = 0; a < m; ++a)
-      if (c[a] >= 0 && c[a] != int32_t(i) && (a == 0 || c[a] != c[a - 1])) ++u;
-    deg[i] = u;
-  }
-}
-
-__global__ void sym_emit_kernel(const int32_t* __restrict__ cand, const int64_t* __restrict__ cstart,
-                                const int64_t* __restrict__ row_ptr, int64_t n,
-                                int32_t* __restrict__ col, int32_t* __restrict__ recv) {
-  for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n;
-       i += int64_t(gridDim.x) * blockDim.x) {
-    const int32_t* c = cand + cstart[i];
-    int64_t m = cstart[i + 1] - cstart[i];
-    int64_t o = row_ptr[i];
-    for (int64_t a = 0; a < m; ++a) {
-      if (c[a] >= 0 && c[a] != int32_t(i) && (a == 0 || c[a] != c[a - 1])) {
-        col[o] = c[a];
-        if (recv) recv[o] = int32_t(i);
-        ++o;
+    __syncwarp();
+    int u = 0;
+    for (int a0 = 0; a0 < mw; a0 += 16) {
+      const int32_t x = a0 + l < m ? srt[gi][a0 + l] : -1;
+      const bool keep = x >= 0 && x != int32_t(i);
+      const uint32_t b = half(__ballot_sync(kAll, keep));
+      if (keep) row[u + __popc(b & ((1u << l) - 1u))] = x;
+      u += __popc(b);
+    }
+    if (in && brief && l == 0) deg[i] = u;
+    __syncwarp();
+    if (!in || brief) continue;
+    // long row, by its half-warp: entries a < k the own slots (empty ones rank last), then the reverse entries
+    const uint32_t mask = 0xffffu << hs;
+    const int64_t all = k + nr;
+    auto get = [&](int64_t a) {
+      const int32_t v = a < k ? nbr[i * k + a] : rev[r0 + a - k];
+      return v < 0 ? INT32_MAX : v;
+    };
+    for (int64_t a = l; a < all; a += 16) {
+      const int32_t x = get(a);
+      int64_t c = 0;
+      for (int64_t b = 0; b < all; ++b) {
+        const int32_t y = get(b);
+        c += y < x || (y == x && b < a);
       }
+      row[c] = x;
     }
+    __syncwarp(mask);
+    int32_t last = -1;  // the entry before this chunk
+    for (int64_t a0 = 0; a0 < all; a0 += 16) {
+      const int64_t a = a0 + l;
+      const int32_t x = a < all ? row[a] : INT32_MAX;
+      int32_t prev = __shfl_up_sync(mask, x, 1, 16);
+      if (l == 0) prev = last;
+      last = __shfl_sync(mask, x, 15, 16);
+      const bool keep = x != INT32_MAX && x != int32_t(i) && x != prev;
+      const uint32_t b = half(__ballot_sync(mask, keep));
+      if (keep) row[u + __popc(b & ((1u << l) - 1u))] = x;  // at or before the places already read
+      u += __popc(b);
+      __syncwarp(mask);
+    }
+    if (l == 0) deg[i] = u;
   }
 }
 
-__global__ void add_ramp_kernel(int64_t* cs, int64_t n, int k) {
-  for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i <= n;
-       i += int64_t(gridDim.x) * blockDim.x)
-    cs[i] += int64_t(k) * i;
+// Copies the sorted rows to their CSR places, 8 lanes per row; nothing is
+// written when the edges exceed the caller's capacity.
+__global__ void sym_emit_kernel(const int32_t* __restrict__ rows, const int64_t* __restrict__ rstart, int k,
+                                const int64_t* __restrict__ row_ptr, int64_t n, int64_t cap,
+                                int32_t* __restrict__ col, int32_t* __restrict__ recv,
+                                const uint32_t* __restrict__ err, int64_t* __restrict__ info) {
+  if (blockIdx.x == 0 && threadIdx.x == 0) {  // what the host reads at the end, in one copy
+    info[0] = row_ptr[n];
+    info[1] = int64_t(*err);
+  }
+  if (row_ptr[n] > cap) return;
+  const int l = threadIdx.x & 7;
+  for (int64_t i = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 3; i < n;
+       i += (int64_t(gridDim.x) * blockDim.x) >> 3) {
+    const int32_t* c = rows + rstart[i] + int64_t(k) * i;
+    const int64_t o = row_ptr[i], m = row_ptr[i + 1] - o;
+    for (int64_t a = l; a < m; a += 8) {
+      col[o + a] = c[a];
+      if (recv) recv[o + a] = int32_t(i);
+    }
+  }
 }
 
 }  // namespace
@@ -282,12 +492,17 @@ xmgn_status quantize_launch(const float* xyz, int64_t n, double scale, int32_t* 
 // keeps four edges in flight and reads rows of up to 8 edges whole; longer
 // rows are searched by key (their senders' ids, or global ids, ascend).  17.2M
 // edges of a 2M-point batch: 123 us (a binary search by key per thread) -> 98 us.
+// e < 0: the edge count is row_ptr[n], and nothing is written if it exceeds cap.
 constexpr int kPermEdges = 4;
 __global__ void __launch_bounds__(256) csc_perm_kernel(const int64_t* __restrict__ row_ptr,
                                                        const int32_t* __restrict__ col,
                                                        const int32_t* __restrict__ recv,
                                                        const int32_t* __restrict__ key, int64_t n, int64_t e,
-                                                       int32_t* __restrict__ perm, uint32_t* err) {
+                                                       int64_t cap, int32_t* __restrict__ perm, uint32_t* err) {
+  if (e < 0) {
+    e = row_ptr[n];
+    if (e > cap) return;
+  }
   const int64_t step = int64_t(gridDim.x) * blockDim.x * kPermEdges;
   for (int64_t p0 = int64_t(blockIdx.x) * blockDim.x * kPermEdges + threadIdx.x; p0 < e; p0 += step) {
     int32_t j[kPermEdges], r[kPermEdges];
@@ -339,111 +554,86 @@ __global__ void __launch_bounds__(256) csc_perm_kernel(const int64_t* __restrict
 }
 
 struct KnnWs {
-  int32_t *q, *bbox, *sorted, *nbr, *cnt, *cand, *deg;
-  int64_t *cell_of, *cstart, *scan_tmp;
-  unsigned long long* fill;
+  int32_t *q, *bbox, *nbr, *cnt, *rcnt, *rev, *rows, *rank, *deg, *cell_of, *at, *cstart;
+  int4* pts;
+  Grid* grid;
+  int64_t *rstart, *info, *scan_tmp;
 };
-
-static int64_t knn_max_cells(int64_t N) { return 2 * N + 1024; }
 
 // Workspace for N points with K directed slots per point.
 static void knn_layout(int64_t N, int32_t K, Arena& A, KnnWs& w) {
-  const int64_t cnt_n = knn_max_cells(N) > N ? knn_max_cells(N) : N;
+  const int64_t cells = cell_budget(N);
   w.q = A.take<int32_t>(size_t(3 * N));
   w.bbox = A.take<int32_t>(8);
-  w.cell_of = A.take<int64_t>(size_t(N));
-  w.sorted = A.take<int32_t>(size_t(N));
+  w.grid = A.take<Grid>(kMaxLevels);
+  w.info = A.take<int64_t>(2);
+  w.cell_of = A.take<int32_t>(size_t(N));
+  w.at = A.take<int32_t>(size_t(N));
+  w.pts = A.take<int4>(size_t(N));
   w.nbr = A.take<int32_t>(size_t(N * K));
-  w.cnt = A.take<int32_t>(size_t(cnt_n + 1));
-  w.cstart = A.take<int64_t>(size_t(cnt_n + 1));
-  w.cand = A.take<int32_t>(size_t(2 * N * K));
-  w.fill = A.take<unsigned long long>(size_t(N));
+  w.cnt = A.take<int32_t>(size_t(cells + 1));
+  w.cstart = A.take<int32_t>(size_t(cells + 1));
+  w.rcnt = A.take<int32_t>(size_t(N));
+  w.rstart = A.take<int64_t>(size_t(N + 1));
+  w.rev = A.take<int32_t>(size_t(N * K));
+  w.rows = A.take<int32_t>(size_t(2 * N * K));
+  w.rank = w.rows;  // the places of the reverse entries are used up before the rows are written
   w.deg = A.take<int32_t>(size_t(N));
-  w.scan_tmp = A.take<int64_t>(scan_tmp_elems(cnt_n + 1) + 16);
+  w.scan_tmp = A.take<int64_t>(scan_tmp_elems((cells > N ? cells : N) + 1) + 16);
 }
 
-// Lattice coordinates of all N points and their bounding box (host).
-static xmgn_status quantize_all(const float* xyz, int64_t N, double scale, KnnWs& w, int32_t hb[6],
-                                uint32_t* err, cudaStream_t s) {
-  bbox_init_kernel<<<1, 32, 0, s>>>(w.bbox);
+// Lattice coordinates of all N points, their bounding box and the levels' grids.
+static xmgn_status quantize_all(const float* xyz, int64_t N, double scale, const LevelSizes& sizes, int levels,
+                                KnnWs& w, uint32_t* err, cudaStream_t s) {
+  XMGN_TRY(quantize_launch(xyz, N, scale, w.q, w.bbox, err, s));
+  grid_layout_kernel<<<1, 32, 0, s>>>(w.bbox, sizes, levels, w.grid);
   XMGN_LAUNCH_CHECK();
-  quantize_kernel<<<grid_for(N, 256, int64_t(num_sms()) * 8), 256, 0, s>>>(xyz, N, float(scale), w.q, w.bbox, err);
-  XMGN_LAUNCH_CHECK();
-  uint32_t herr = 0;
-  XMGN_CUDA(cudaMemcpyAsync(hb, w.bbox, sizeof(int32_t) * 6, cudaMemcpyDeviceToHost, s));
-  XMGN_CUDA(cudaMemcpyAsync(&herr, err, sizeof(herr), cudaMemcpyDeviceToHost, s));
-  XMGN_CUDA(cudaStreamSynchronize(s));
-  if (herr & DEV_ERR_RANGE) {
-    XMGN_CUDA(cudaMemsetAsync(err, 0, sizeof(uint32_t), s));
-    return fail(XMGN_ERR_RANGE, "coordinate outside the lattice range (|x*scale| >= 2^24 or not finite)");
-  }
+  XMGN_CUDA(cudaMemsetAsync(w.rcnt, 0, sizeof(int32_t) * size_t(N), s));
   return XMGN_OK;
 }
 
-// Counting sort of the reference points 0..n_ref-1 into a uniform grid over
-// the bounding box hb of all points (about two cells per reference point).
-static xmgn_status grid_sort(int64_t n_ref, const int32_t hb[6], int64_t max_cells, KnnWs& w, Grid* Gout,
-                             cudaStream_t s) {
-  Grid G;
-  double vol = 1.0;
-  for (int a = 0; a < 3; ++a) {
-    G.lo[a] = hb[a];
-    vol *= double(int64_t(hb[3 + a]) - hb[a] + 1);
-  }
-  double c = cbrt(vol / (2.0 * double(n_ref)));
-  if (c < 1) c = 1;
-  G.c = int64_t(ceil(c));
-  for (;;) {
-    int64_t tot = 1;
-    for (int a = 0; a < 3; ++a) {
-      G.g[a] = (int64_t(hb[3 + a]) - hb[a]) / G.c + 1;
-      tot *= G.g[a];
-    }
-    if (tot <= max_cells) break;
-    G.c = G.c + G.c / 4 + 1;
-  }
-  const int64_t ncell = G.g[0] * G.g[1] * G.g[2];
-  XMGN_CUDA(cudaMemsetAsync(w.cnt, 0, sizeof(int32_t) * size_t(ncell), s));
-  cell_count_kernel<<<grid_for(n_ref, 256), 256, 0, s>>>(w.q, n_ref, G, w.cell_of, w.cnt);
+// Counting sort of the reference points 0..n_ref-1 into their grid.
+static xmgn_status grid_sort(int64_t n_ref, const Grid* grid, KnnWs& w, cudaStream_t s) {
+  const int64_t cells = cell_budget(n_ref);
+  XMGN_CUDA(cudaMemsetAsync(w.cnt, 0, sizeof(int32_t) * size_t(cells), s));
+  cell_count_kernel<<<grid_for(n_ref, 256), 256, 0, s>>>(w.q, n_ref, grid, w.cell_of, w.at, w.cnt);
   XMGN_LAUNCH_CHECK();
-  XMGN_TRY(exclusive_scan_i32(w.cnt, w.cstart, ncell, w.scan_tmp, s));
-  XMGN_CUDA(cudaMemsetAsync(w.cnt, 0, sizeof(int32_t) * size_t(ncell), s));
-  cell_scatter_kernel<<<grid_for(n_ref, 256), 256, 0, s>>>(w.cell_of, n_ref, w.cstart, w.cnt, w.sorted);
+  XMGN_TRY(exclusive_scan_i32(w.cnt, w.cstart, cells, w.scan_tmp, s));
+  cell_scatter_kernel<<<grid_for(n_ref, 256), 256, 0, s>>>(w.q, w.cell_of, w.at, n_ref, w.cstart, w.pts);
   XMGN_LAUNCH_CHECK();
-  *Gout = G;
   return XMGN_OK;
 }
 
 // Undirected receiver-major CSR from K directed slots per point (w.nbr,
-// -1 = empty): candidates of i = its own slots + every j listing i; the
-// candidate offsets are the scan of the reverse counts shifted by K*i.
+// -1 = empty; w.rcnt and w.rank as knn_kernel leaves them), and the one host
+// wait of a build: the edge count and the range error of the coordinates.
 static xmgn_status symmetrise_slots(int64_t N, int32_t K, KnnWs& w, int64_t* row_ptr, int32_t* col,
                                     int32_t* recv, int32_t* csc_perm, int64_t E_cap, int64_t* E_out,
                                     uint32_t* err, cudaStream_t s) {
-  XMGN_CUDA(cudaMemsetAsync(w.cnt, 0, sizeof(int32_t) * size_t(N), s));
-  sym_count_kernel<<<grid_for(N * K, 256), 256, 0, s>>>(w.nbr, N, K, w.cnt, err);
+  XMGN_TRY(exclusive_scan_i32(w.rcnt, w.rstart, N, w.scan_tmp, s));
+  sym_rev_kernel<<<grid_for(N * K, 256), 256, 0, s>>>(w.nbr, N, K, w.rstart, w.rank, w.rev);
   XMGN_LAUNCH_CHECK();
-  XMGN_TRY(exclusive_scan_i32(w.cnt, w.cstart, N, w.scan_tmp, s));
-  add_ramp_kernel<<<grid_for(N + 1, 256), 256, 0, s>>>(w.cstart, N, K);
-  XMGN_LAUNCH_CHECK();
-  sym_own_kernel<<<grid_for(N, 256), 256, 0, s>>>(w.nbr, N, K, w.cstart, w.cand, w.fill);
-  XMGN_LAUNCH_CHECK();
-  sym_rev_kernel<<<grid_for(N * K, 256), 256, 0, s>>>(w.nbr, N, K, w.cand, w.fill);
-  XMGN_LAUNCH_CHECK();
-  sym_sort_kernel<<<grid_for(N, 128), 128, 0, s>>>(w.cand, w.cstart, N, w.deg);
+  sym_sort_kernel<<<grid_for(N * 16, 256), 256, 0, s>>>(w.nbr, N, K, w.rstart, w.rev, w.rows, w.deg);
   XMGN_LAUNCH_CHECK();
   XMGN_TRY(exclusive_scan_i32(w.deg, row_ptr, N, w.scan_tmp, s));
-  int64_t E = 0;
-  XMGN_CUDA(cudaMemcpyAsync(&E, row_ptr + N, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-  XMGN_CUDA(cudaStreamSynchronize(s));
-  *E_out = E;
-  if (E > E_cap) return fail(XMGN_ERR_WORKSPACE, "E=%lld exceeds E_cap=%lld", (long long)E, (long long)E_cap);
-  sym_emit_kernel<<<grid_for(N, 128), 128, 0, s>>>(w.cand, w.cstart, row_ptr, N, col, recv);
+  sym_emit_kernel<<<grid_for(N * 8, 256), 256, 0, s>>>(w.rows, w.rstart, K, row_ptr, N, E_cap, col, recv, err, w.info);
   XMGN_LAUNCH_CHECK();
   if (csc_perm) {
-    csc_perm_kernel<<<grid_for((E + kPermEdges - 1) / kPermEdges, 256), 256, 0, s>>>(row_ptr, col, recv, nullptr, N, E, csc_perm, err);
+    const int64_t most = 2 * N * K < E_cap ? 2 * N * K : E_cap;
+    csc_perm_kernel<<<grid_for((most + kPermEdges - 1) / kPermEdges, 256), 256, 0, s>>>(row_ptr, col, recv, nullptr, N,
+                                                                                        -1, E_cap, csc_perm, err);
     XMGN_LAUNCH_CHECK();
   }
+  int64_t info[2];
+  XMGN_CUDA(cudaMemcpyAsync(info, w.info, sizeof(info), cudaMemcpyDeviceToHost, s));
+  XMGN_CUDA(cudaStreamSynchronize(s));
+  const int64_t E = info[0];
+  if (info[1] & DEV_ERR_RANGE) {
+    XMGN_CUDA(cudaMemsetAsync(err, 0, sizeof(uint32_t), s));
+    return fail(XMGN_ERR_RANGE, "coordinate outside the lattice range (|x*scale| >= 2^24 or not finite)");
+  }
+  *E_out = E;
+  if (E > E_cap) return fail(XMGN_ERR_WORKSPACE, "E=%lld exceeds E_cap=%lld", (long long)E, (long long)E_cap);
   return XMGN_OK;
 }
 
@@ -482,12 +672,11 @@ xmgn_status build_knn(const float* xyz, int64_t N, int32_t k, double scale, void
   if (!A.ok()) return fail(XMGN_ERR_WORKSPACE, "knn workspace too small: need %zu", A.used);
   uint32_t* err = device_error_word();
   if (nbr_out) w.nbr = nbr_out;
-  int32_t hb[6];
-  XMGN_TRY(quantize_all(xyz, N, scale, w, hb, err, s));
-  Grid G;
-  XMGN_TRY(grid_sort(N, hb, knn_max_cells(N), w, &G, s));
-  knn_search_kernel<<<grid_for(N, 128), 128, 0, s>>>(w.q, w.sorted, w.cstart, N, k, G, w.nbr, k, 0);
-  XMGN_LAUNCH_CHECK();
+  LevelSizes sizes{};
+  sizes.n[0] = N;
+  XMGN_TRY(quantize_all(xyz, N, scale, sizes, 1, w, err, s));
+  XMGN_TRY(grid_sort(N, w.grid, w, s));
+  XMGN_TRY(knn_launch<false>(w.q, w.pts, w.cstart, 0, N, k, w.grid, w.nbr, k, 0, w.rcnt, w.rank, s));
   return symmetrise_slots(N, k, w, row_ptr, col, recv, csc_perm, E_cap, E_out, err, s);
 }
 
@@ -533,22 +722,17 @@ xmgn_status build_multiscale(const float* xyz, int64_t N, const int64_t* sizes, 
   if (!A.ok()) return fail(XMGN_ERR_WORKSPACE, "multiscale workspace too small: need %zu", A.used);
   uint32_t* err = device_error_word();
   if (nbr_out) w.nbr = nbr_out;
-  int32_t hb[6];
-  XMGN_TRY(quantize_all(xyz, N, scale, w, hb, err, s));
+  LevelSizes ls{};
+  for (int l = 0; l < n_levels; ++l) ls.n[l] = sizes[l];
+  XMGN_TRY(quantize_all(xyz, N, scale, ls, n_levels, w, err, s));
   XMGN_CUDA(cudaMemsetAsync(w.nbr, 0xff, sizeof(int32_t) * size_t(N) * K, s));  // all slots empty (-1)
   for (int l = 0; l < n_levels; ++l) {
     // kNN within level l (the first sizes[l] points): slots [l*k, l*k + k)
-    Grid G;
-    XMGN_TRY(grid_sort(sizes[l], hb, knn_max_cells(N), w, &G, s));
-    knn_search_kernel<<<grid_for(sizes[l], 128), 128, 0, s>>>(w.q, w.sorted, w.cstart, sizes[l], k, G, w.nbr, K,
-                                                               l * k);
-    XMGN_LAUNCH_CHECK();
-    if (l > 0) {  // points new in level l -> k_cross nearest of level l-1: slots [L*k, L*k + k_cross)
-      XMGN_TRY(grid_sort(sizes[l - 1], hb, knn_max_cells(N), w, &G, s));
-      knn_query_kernel<<<grid_for(sizes[l] - sizes[l - 1], 128), 128, 0, s>>>(
-          w.q, w.sorted, w.cstart, sizes[l - 1], sizes[l], k_cross, G, w.nbr, K, n_levels * k);
-      XMGN_LAUNCH_CHECK();
-    }
+    XMGN_TRY(grid_sort(sizes[l], w.grid + l, w, s));
+    XMGN_TRY(knn_launch<false>(w.q, w.pts, w.cstart, 0, sizes[l], k, w.grid + l, w.nbr, K, l * k, w.rcnt, w.rank, s));
+    if (l + 1 < n_levels)  // points new in level l+1 -> k_cross nearest of level l: slots [L*k, L*k + k_cross)
+      XMGN_TRY(knn_launch<true>(w.q, w.pts, w.cstart, sizes[l], sizes[l + 1], k_cross, w.grid + l, w.nbr, K,
+                                n_levels * k, w.rcnt, w.rank, s));
   }
   return symmetrise_slots(N, K, w, row_ptr, col, recv, csc_perm, E_cap, E_out, err, s);
 }

@@ -32,7 +32,7 @@ namespace xmgn {
 
 __global__ void csc_perm_kernel(const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
                                 const int32_t* __restrict__ recv, const int32_t* __restrict__ key,
-                                int64_t n, int64_t e, int32_t* __restrict__ perm, uint32_t* err);
+                                int64_t n, int64_t e, int64_t cap, int32_t* __restrict__ perm, uint32_t* err);
 xmgn_status quantize_launch(const float* xyz, int64_t n, double scale, int32_t* q, int32_t* bbox,
                             uint32_t* err, cudaStream_t s);
 
@@ -793,7 +793,7 @@ xmgn_status partition_halo(const int64_t* row_ptr, const int32_t* col, int64_t N
       XMGN_LAUNCH_CHECK();
     }
     if (b_csc_perm && eb > 0) {
-      csc_perm_kernel<<<grid_for((eb + 3) / 4, 256), 256, 0, s>>>(b_row_ptr, b_col, b_recv, gid, nb, eb, b_csc_perm, err);
+      csc_perm_kernel<<<grid_for((eb + 3) / 4, 256), 256, 0, s>>>(b_row_ptr, b_col, b_recv, gid, nb, eb, eb, b_csc_perm, err);
       XMGN_LAUNCH_CHECK();
     }
     XMGN_CUDA(cudaMemsetAsync(w.stamp, 0, sizeof(int64_t) * 8, s));  // one emit per sizing pass
