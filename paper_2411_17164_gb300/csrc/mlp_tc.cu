@@ -453,17 +453,11 @@ __device__ __forceinline__ bool setup(uint64_t* wbar, uint64_t* mbar, uint32_t* 
 }
 
 // GEMM1 / GEMM2 of the forward direction: X W_hi [+ X W_lo].
-template <int MODE>
-__device__ __forceinline__ void fwd_gemm(uint32_t d, uint32_t xs, uint32_t R_b, uint32_t wh, uint32_t wl, int ksteps,
-                                         int N) {
-  using S = Shape<MODE>;
-  const uint32_t id = idesc_bf16(128, N, false, false);
-#pragma unroll 1
-  for (int k = 0; k < ksteps; ++k) mma_bf16(d, kmajor_desc(xs, 128, k), kmajor_desc(wh, R_b, k), id, k > 0);
-  if (S::SPLIT) {
-#pragma unroll 1
-    for (int k = 0; k < ksteps; ++k) mma_bf16(d, kmajor_desc(xs, 128, k), kmajor_desc(wl, R_b, k), id, 1u);
-  }
+template <int MODE, int STEPS, int N>
+__device__ __forceinline__ void fwd_gemm(uint32_t d, uint32_t xs, uint32_t wh, uint32_t wl) {
+  constexpr uint32_t id = idesc_bf16(128, N, false, false);
+  mma_chain<STEPS, 128, false, N, false>(d, xs, wh, id, false);
+  if (Shape<MODE>::SPLIT) mma_chain<STEPS, 128, false, N, false>(d, xs, wl, id, true);
 }
 
 // The four warps that hold the column slices of the same 32 rows (lane
@@ -560,7 +554,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_fwd_kernel(FwdArgs a) {
     __syncthreads();
     if (tid == 0) {
       tc_fence_after();
-      fwd_gemm<MODE>(tm, smem_u32(xa), kH, smem_u32(sm.w1h), S::SPLIT ? smem_u32(sm.w1l) : 0u, S::K1S, kH);
+      fwd_gemm<MODE, S::K1S, kH>(tm, smem_u32(xa), smem_u32(sm.w1h), S::SPLIT ? smem_u32(sm.w1l) : 0u);
       mma_commit(&mbar);
     }
     const int64_t row = r0 + r;
@@ -585,8 +579,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_fwd_kernel(FwdArgs a) {
     __syncthreads();
     if (tid == 0) {
       tc_fence_after();
-      fwd_gemm<MODE>(tm + kH, smem_u32(a1), S::N2, smem_u32(sm.w2h), S::SPLIT ? smem_u32(sm.w2l) : 0u, kH / 16,
-                     S::N2);
+      fwd_gemm<MODE, kH / 16, S::N2>(tm + kH, smem_u32(a1), smem_u32(sm.w2h), S::SPLIT ? smem_u32(sm.w2l) : 0u);
       mma_commit(&mbar);
     }
     ok = mbar_wait(&mbar, ph, a.err);
@@ -742,7 +735,7 @@ __global__ void __launch_bounds__(kThreads, 1) edge_fwd_kernel(FwdArgs a, const 
       }
       lok = mbar_wait(&eb[g], eph, a.err);
       tc_fence_after();
-      if (lok) fwd_gemm<M_EDGE>(T, smem_u32(X), kH, smem_u32(sm.w1h), smem_u32(sm.w1l), kH / 16, kH);
+      if (lok) fwd_gemm<M_EDGE, kH / 16, kH>(T, smem_u32(X), smem_u32(sm.w1h), smem_u32(sm.w1l));
       mma_commit(&mb[g]);
     }
     const int64_t row = r0 + r;
@@ -790,10 +783,8 @@ __global__ void __launch_bounds__(kThreads, 1) edge_fwd_kernel(FwdArgs a, const 
     if (gt == 0) {
       tc_fence_after();
       const uint32_t wh = smem_u32(sm.w2h), wl = smem_u32(sm.w2l);
-#pragma unroll 1
-      for (int kk = 0; kk < kH / 16; ++kk) mma_bf16_ts(T + kH, T + 8 * kk, kmajor_desc(wh, kH, kk), id_x, kk > 0);
-#pragma unroll 1
-      for (int kk = 0; kk < kH / 16; ++kk) mma_bf16_ts(T + kH, T + 8 * kk, kmajor_desc(wl, kH, kk), id_x, 1u);
+mma_chain_ts<kH / 16, kH>(T + kH, T, wh, id_x, false);
+mma_chain_ts<kH / 16, kH>(T + kH, T, wl, id_x, true);
       mma_commit(&mb[g]);
     }
     {  // the group's next tile's node projections, for its epi1, towards L2 (one line per block and row)
@@ -964,10 +955,8 @@ __global__ void __launch_bounds__(kThreads, 1) node_fwd_kernel(FwdArgs a) {
     if (tid == 0) {
       tc_fence_after();
       const uint32_t wh = smem_u32(sm.w1h), wl = smem_u32(sm.w1l);
-#pragma unroll 1
-      for (int kk = 0; kk < 2 * kH / 16; ++kk) mma_bf16_ts(tm + tZ1, tm + tX + 8 * kk, kmajor_desc(wh, kH, kk), id, kk > 0);
-#pragma unroll 1
-      for (int kk = 0; kk < 2 * kH / 16; ++kk) mma_bf16_ts(tm + tZ1, tm + tX + 8 * kk, kmajor_desc(wl, kH, kk), id, 1u);
+mma_chain_ts<2 * kH / 16, kH>(tm + tZ1, tm + tX, wh, id, false);
+mma_chain_ts<2 * kH / 16, kH>(tm + tZ1, tm + tX, wl, id, true);
       mma_commit(&mbar);
     }
     const int64_t row = r0 + r;
@@ -1000,10 +989,8 @@ __global__ void __launch_bounds__(kThreads, 1) node_fwd_kernel(FwdArgs a) {
     if (tid == 0) {
       tc_fence_after();
       const uint32_t wh = smem_u32(sm.w2h), wl = smem_u32(sm.w2l);
-#pragma unroll 1
-      for (int kk = 0; kk < kH / 16; ++kk) mma_bf16_ts(tm + tZ2, tm + tA + 8 * kk, kmajor_desc(wh, kH, kk), id, kk > 0);
-#pragma unroll 1
-      for (int kk = 0; kk < kH / 16; ++kk) mma_bf16_ts(tm + tZ2, tm + tA + 8 * kk, kmajor_desc(wl, kH, kk), id, 1u);
+mma_chain_ts<kH / 16, kH>(tm + tZ2, tm + tA, wh, id, false);
+mma_chain_ts<kH / 16, kH>(tm + tZ2, tm + tA, wl, id, true);
       mma_commit(&mbar);
     }
     float v[32], g0[32];
@@ -1096,7 +1083,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_bwd_kernel(BwdArgs a) {
     // ---- GEMM1
     if (tid == 0) {
       tc_fence_after();
-      fwd_gemm<MODE>(tm + tZ1, smem_u32(xa), kH, smem_u32(sm.w1h), S::SPLIT ? smem_u32(sm.w1l) : 0u, S::K1S, kH);
+      fwd_gemm<MODE, S::K1S, kH>(tm + tZ1, smem_u32(xa), smem_u32(sm.w1h), S::SPLIT ? smem_u32(sm.w1l) : 0u);
       mma_commit(&mbar);
     }
     const int64_t row = r0 + r;
@@ -1129,8 +1116,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_bwd_kernel(BwdArgs a) {
     if (LN) {
       if (tid == 0) {
         tc_fence_after();
-        fwd_gemm<MODE>(tm + tZ2, smem_u32(sm.a1), kH, smem_u32(sm.w2h), S::SPLIT ? smem_u32(sm.w2l) : 0u, kH / 16,
-                       kH);
+        fwd_gemm<MODE, kH / 16, kH>(tm + tZ2, smem_u32(sm.a1), smem_u32(sm.w2h), S::SPLIT ? smem_u32(sm.w2l) : 0u);
         mma_commit(&mbar);
       }
       // incoming gradient of this slice while the MMA runs
@@ -1203,14 +1189,10 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_bwd_kernel(BwdArgs a) {
       tc_fence_after();
       const uint32_t ds = smem_u32(sm.dz2), ws = smem_u32(sm.w2h), as = smem_u32(sm.a1);
       const uint32_t id = idesc_bf16(128, kH, false, true);
-#pragma unroll 1
-      for (int k = 0; k < S::N2 / 16; ++k)
-        mma_bf16(tm + tZ2, kmajor_desc(ds, 128, k), mnmajor_desc(ws, S::N2, k), id, k > 0);
+      mma_chain<S::N2 / 16, 128, false, S::N2, true>(tm + tZ2, ds, ws, id, false);
       if (TMW) {
         const uint32_t idw = idesc_bf16(128, kH, true, true);
-#pragma unroll 1
-        for (int k = 0; k < 8; ++k)
-          mma_bf16(tm + tW2, mnmajor_desc(as, 128, k), mnmajor_desc(ds, 128, k), idw, (first && k == 0) ? 0u : 1u);
+        mma_chain<8, 128, true, 128, true>(tm + tW2, as, ds, idw, !first);
       }
       mma_commit(&mbar);
     }
@@ -1247,14 +1229,11 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_bwd_kernel(BwdArgs a) {
       const uint32_t ds = smem_u32(sm.a1), ws = smem_u32(sm.w1h), xs = smem_u32(xa);
       if (HAS_DX) {
         const uint32_t id = idesc_bf16(128, NX, false, true);
-#pragma unroll 1
-        for (int k = 0; k < kH / 16; ++k) mma_bf16(tm + tDX, kmajor_desc(ds, 128, k), mnmajor_desc(ws, kH, k), id, k > 0);
+        mma_chain<kH / 16, 128, false, kH, true>(tm + tDX, ds, ws, id, false);
       }
       if (TMW) {
         const uint32_t idw = idesc_bf16(128, kH, true, true);
-#pragma unroll 1
-        for (int k = 0; k < 8; ++k)
-          mma_bf16(tm + tW1, mnmajor_desc(xs, 128, k), mnmajor_desc(ds, 128, k), idw, (first && k == 0) ? 0u : 1u);
+        mma_chain<8, 128, true, 128, true>(tm + tW1, xs, ds, idw, !first);
       }
       mma_commit(&mbar);
     }
@@ -1485,9 +1464,7 @@ __global__ void __launch_bounds__(kThreads, 1) edge_bwd_kernel(BwdArgs a, const 
       tc_fence_after();
       const uint32_t xs = smem_u32(sm.xe), ws = smem_u32(sm.w1);
       if (ok) {
-#pragma unroll 1
-        for (int kk = 0; kk < kH / 16; ++kk)
-          mma_bf16(tm + tZ1, kmajor_desc(xs, 128, kk), kmajor_desc(ws, kH, kk), id_f, kk > 0);
+mma_chain<kH / 16, 128, false, kH, false>(tm + tZ1, xs, ws, id_f, false);
       }
       mma_commit(&mbar);
     }
@@ -1523,8 +1500,7 @@ __global__ void __launch_bounds__(kThreads, 1) edge_bwd_kernel(BwdArgs a, const 
     if (tid == 0) {
       tc_fence_after();
       const uint32_t as = smem_u32(sm.a1), ws = smem_u32(sm.w2);
-#pragma unroll 1
-      for (int kk = 0; kk < kH / 16; ++kk) mma_bf16(tm + tZ2, kmajor_desc(as, 128, kk), kmajor_desc(ws, kH, kk), id_f, kk > 0);
+mma_chain<kH / 16, 128, false, kH, false>(tm + tZ2, as, ws, id_f, false);
       mma_commit(&mbar);
     }
     // incoming gradient dm = de + da[receiver] while the MMA runs
@@ -1584,12 +1560,8 @@ __global__ void __launch_bounds__(kThreads, 1) edge_bwd_kernel(BwdArgs a, const 
     if (tid == 0) {
       tc_fence_after();
       const uint32_t ds = smem_u32(sm.dz2), ws = smem_u32(sm.w2), as = smem_u32(sm.a1);
-#pragma unroll 1
-      for (int kk = 0; kk < kH / 16; ++kk)
-        mma_bf16(tm + tZ2, kmajor_desc(ds, 128, kk), mnmajor_desc(ws, kH, kk), id_t, kk > 0);
-#pragma unroll 1
-      for (int kk = 0; kk < 8; ++kk)
-        mma_bf16(tm + tW2, mnmajor_desc(as, 128, kk), mnmajor_desc(ds, 128, kk), id_w, (first && kk == 0) ? 0u : 1u);
+mma_chain<kH / 16, 128, false, kH, true>(tm + tZ2, ds, ws, id_t, false);
+mma_chain<8, 128, true, 128, true>(tm + tW2, as, ds, id_w, !first);
       mma_commit(&mbar);
     }
     ok = mbar_wait(&mbar, ph, a.err);
@@ -1618,12 +1590,8 @@ __global__ void __launch_bounds__(kThreads, 1) edge_bwd_kernel(BwdArgs a, const 
     if (tid == 0) {
       tc_fence_after();
       const uint32_t ds = smem_u32(sm.a1), ws = smem_u32(sm.w1), xs = smem_u32(sm.xe);
-#pragma unroll 1
-      for (int kk = 0; kk < kH / 16; ++kk)
-        mma_bf16(tm + tDX, kmajor_desc(ds, 128, kk), mnmajor_desc(ws, kH, kk), id_t, kk > 0);
-#pragma unroll 1
-      for (int kk = 0; kk < 8; ++kk)
-        mma_bf16(tm + tW1, mnmajor_desc(xs, 128, kk), mnmajor_desc(ds, 128, kk), id_w, (first && kk == 0) ? 0u : 1u);
+mma_chain<kH / 16, 128, false, kH, true>(tm + tDX, ds, ws, id_t, false);
+mma_chain<8, 128, true, 128, true>(tm + tW1, xs, ds, id_w, !first);
       mma_commit(&mbar);
     }
     if (tma_thread) {
@@ -1883,9 +1851,7 @@ __global__ void __launch_bounds__(kT32, 1) edge_bwd32_kernel(BwdArgs a, const __
       tc_fence_after();
       const uint32_t xs = smem_u32(sm.xe), ws = smem_u32(sm.w1);
       if (ok) {
-#pragma unroll 1
-        for (int kk = 0; kk < kH / 16; ++kk)
-          mma_bf16(tm + tZ1, kmajor_desc(xs, 128, kk), kmajor_desc(ws, kH, kk), id_f, kk > 0);
+mma_chain<kH / 16, 128, false, kH, false>(tm + tZ1, xs, ws, id_f, false);
       }
       mma_commit(&mbar);
     }
@@ -1920,8 +1886,7 @@ __global__ void __launch_bounds__(kT32, 1) edge_bwd32_kernel(BwdArgs a, const __
     if (tid == 0) {
       tc_fence_after();
       const uint32_t as = smem_u32(sm.a1), ws = smem_u32(sm.w2);
-#pragma unroll 1
-      for (int kk = 0; kk < kH / 16; ++kk) mma_bf16(tm + tZ2, kmajor_desc(as, 128, kk), kmajor_desc(ws, kH, kk), id_f, kk > 0);
+mma_chain<kH / 16, 128, false, kH, false>(tm + tZ2, as, ws, id_f, false);
       mma_commit(&mbar);
     }
 #pragma unroll
@@ -1980,12 +1945,8 @@ __global__ void __launch_bounds__(kT32, 1) edge_bwd32_kernel(BwdArgs a, const __
     if (tid == 0) {
       tc_fence_after();
       const uint32_t ds = smem_u32(sm.dz2), ws = smem_u32(sm.w2), as = smem_u32(sm.a1);
-#pragma unroll 1
-      for (int kk = 0; kk < kH / 16; ++kk)
-        mma_bf16(tm + tZ2, kmajor_desc(ds, 128, kk), mnmajor_desc(ws, kH, kk), id_t, kk > 0);
-#pragma unroll 1
-      for (int kk = 0; kk < 8; ++kk)
-        mma_bf16(tm + tW2, mnmajor_desc(as, 128, kk), mnmajor_desc(ds, 128, kk), id_w, (first && kk == 0) ? 0u : 1u);
+mma_chain<kH / 16, 128, false, kH, true>(tm + tZ2, ds, ws, id_t, false);
+mma_chain<8, 128, true, 128, true>(tm + tW2, as, ds, id_w, !first);
       mma_commit(&mbar);
     }
     ok = mbar_wait(&mbar, ph, a.err);
@@ -2013,12 +1974,8 @@ __global__ void __launch_bounds__(kT32, 1) edge_bwd32_kernel(BwdArgs a, const __
     if (tid == 0) {
       tc_fence_after();
       const uint32_t ds = smem_u32(sm.a1), ws = smem_u32(sm.w1), xs = smem_u32(sm.xe);
-#pragma unroll 1
-      for (int kk = 0; kk < kH / 16; ++kk)
-        mma_bf16(tm + tDX, kmajor_desc(ds, 128, kk), mnmajor_desc(ws, kH, kk), id_t, kk > 0);
-#pragma unroll 1
-      for (int kk = 0; kk < 8; ++kk)
-        mma_bf16(tm + tW1, mnmajor_desc(xs, 128, kk), mnmajor_desc(ds, 128, kk), id_w, (first && kk == 0) ? 0u : 1u);
+mma_chain<kH / 16, 128, false, kH, true>(tm + tDX, ds, ws, id_t, false);
+mma_chain<8, 128, true, 128, true>(tm + tW1, xs, ds, id_w, !first);
       mma_commit(&mbar);
     }
     if (tma_thread) {
@@ -2241,8 +2198,7 @@ __global__ void __launch_bounds__(kThreads, 1) edge_bwd2_kernel(BwdArgs a) {
     if (gt == 0) {
       tc_fence_after();
       const uint32_t xs = smem_u32(T1), ws = smem_u32(sm.w1);
-#pragma unroll 1
-      for (int kk = 0; kk < kH / 16; ++kk) mma_bf16(R, kmajor_desc(xs, 128, kk), kmajor_desc(ws, kH, kk), id_f, kk > 0);
+mma_chain<kH / 16, 128, false, kH, false>(R, xs, ws, id_f, false);
       mma_commit(&mb[g]);
     }
     uint32_t pr[16], ps[16];  // 32 bf16 node projections each, packed
@@ -2288,8 +2244,7 @@ __global__ void __launch_bounds__(kThreads, 1) edge_bwd2_kernel(BwdArgs a) {
     if (gt == 0) {
       tc_fence_after();
       const uint32_t as = smem_u32(T2), ws = smem_u32(sm.w2);
-#pragma unroll 1
-      for (int kk = 0; kk < kH / 16; ++kk) mma_bf16(R, kmajor_desc(as, 128, kk), kmajor_desc(ws, kH, kk), id_f, kk > 0);
+mma_chain<kH / 16, 128, false, kH, false>(R, as, ws, id_f, false);
       mma_commit(&mb[g]);
     }
     gok = group_all(g, mbar_wait(&mb[g], ph, a.err));
@@ -2379,14 +2334,11 @@ __global__ void __launch_bounds__(kThreads, 1) edge_bwd2_kernel(BwdArgs a) {
     if (gt == 0) {
       tc_fence_after();
       const uint32_t ds = smem_u32(T1), ws = smem_u32(sm.w2), as = smem_u32(T2);
-#pragma unroll 1
-      for (int kk = 0; kk < kH / 16; ++kk) mma_bf16(R, kmajor_desc(ds, 128, kk), mnmajor_desc(ws, kH, kk), id_t, kk > 0);
+mma_chain<kH / 16, 128, false, kH, true>(R, ds, ws, id_t, false);
       lok = token_wait(&tok[0], int32_t(j), a.err);
       if (lok) {
         tc_fence_after();
-#pragma unroll 1
-        for (int kk = 0; kk < 8; ++kk)
-          mma_bf16(tW2, mnmajor_desc(as, 128, kk), mnmajor_desc(ds, 128, kk), id_w, (j == 0 && kk == 0) ? 0u : 1u);
+mma_chain<8, 128, true, 128, true>(tW2, as, ds, id_w, !(j == 0));
       }
       mma_commit(&mb[g]);
       if (lok) {
@@ -2425,14 +2377,11 @@ __global__ void __launch_bounds__(kThreads, 1) edge_bwd2_kernel(BwdArgs a) {
     if (gt == 0) {
       tc_fence_after();
       const uint32_t ds = smem_u32(T2), ws = smem_u32(sm.w1), xs = smem_u32(T1);
-#pragma unroll 1
-      for (int kk = 0; kk < kH / 16; ++kk) mma_bf16(R, kmajor_desc(ds, 128, kk), mnmajor_desc(ws, kH, kk), id_t, kk > 0);
+mma_chain<kH / 16, 128, false, kH, true>(R, ds, ws, id_t, false);
       lok = token_wait(&tok[1], int32_t(j), a.err);
       if (lok) {
         tc_fence_after();
-#pragma unroll 1
-        for (int kk = 0; kk < 8; ++kk)
-          mma_bf16(tW1, mnmajor_desc(xs, 128, kk), mnmajor_desc(ds, 128, kk), id_w, (j == 0 && kk == 0) ? 0u : 1u);
+mma_chain<8, 128, true, 128, true>(tW1, xs, ds, id_w, !(j == 0));
       }
       mma_commit(&mb[g]);
       if (lok) {

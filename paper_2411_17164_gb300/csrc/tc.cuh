@@ -52,6 +52,18 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
       : "memory");
   return ok != 0;
 }
+// Whether the phase is complete now (no waiting).
+__device__ __forceinline__ bool mbar_test(uint64_t* bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok)
+      : "r"(smem_u32(bar)), "r"(parity)
+      : "memory");
+  return ok != 0;
+}
 // Bounded wait (about one second); on timeout flags DEV_ERR_TIMEOUT and
 // returns false so the caller can wind down without hanging the GPU.
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, uint32_t* err) {
@@ -283,6 +295,41 @@ __device__ __forceinline__ uint64_t kmajor_desc(uint32_t base, uint32_t R, uint3
 // Descriptor of the 16-row K step `k` of an MN-major tile with R rows at `base`.
 __device__ __forceinline__ uint64_t mnmajor_desc(uint32_t base, uint32_t R, uint32_t k) {
   return sdesc(base + k * 2048u, R * 128u, 1024u);
+}
+
+// STEPS 16-deep K steps of one product, D (+)= A B: A a K-major (or AMN:
+// MN-major) tile of RA rows, B one of RB rows.  Straight code: a step's
+// descriptors are the first ones plus a constant.  The issuing thread is on
+// the critical path of every tile; with the descriptors rebuilt in a loop a
+// step took it 105-130 cycles where the tensor core needs 64.
+template <uint32_t R, bool MN>
+__device__ __forceinline__ uint64_t desc_at(uint64_t first, int k) {
+  return first + (MN ? uint32_t(k) * 128u : (uint32_t(k) >> 2) * (R * 8u) + (uint32_t(k) & 3u) * 2u);
+}
+// The same value, opaque to the compiler: descriptors made from it are built
+// where they are used (hoisted out of a tile loop they would take the registers
+// of the epilogues).
+__device__ __forceinline__ uint32_t here(uint32_t x) {
+  asm volatile("" : "+r"(x));
+  return x;
+}
+template <int STEPS, uint32_t RA, bool AMN, uint32_t RB, bool BMN>
+__device__ __forceinline__ void mma_chain(uint32_t d, uint32_t a, uint32_t b, uint32_t idesc, bool accumulate) {
+  const uint32_t ah = here(a), bh = here(b);
+  const uint64_t da = AMN ? mnmajor_desc(ah, RA, 0) : kmajor_desc(ah, RA, 0);
+  const uint64_t db = BMN ? mnmajor_desc(bh, RB, 0) : kmajor_desc(bh, RB, 0);
+#pragma unroll
+  for (int k = 0; k < STEPS; ++k)
+    mma_bf16(d, desc_at<RA, AMN>(da, k), desc_at<RB, BMN>(db, k), idesc, (accumulate || k > 0) ? 1u : 0u);
+}
+// The same with A in TMEM (8 columns per step), B K-major.
+template <int STEPS, uint32_t RB>
+__device__ __forceinline__ void mma_chain_ts(uint32_t d, uint32_t a_tmem, uint32_t b, uint32_t idesc, bool accumulate) {
+  const uint64_t db = kmajor_desc(here(b), RB, 0);
+  const uint32_t ta = here(a_tmem);
+#pragma unroll
+  for (int k = 0; k < STEPS; ++k)
+    mma_bf16_ts(d, ta + 8 * k, desc_at<RB, false>(db, k), idesc, (accumulate || k > 0) ? 1u : 0u);
 }
 
 __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {

@@ -138,9 +138,11 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(GemmArgs a, const 
     if (tid == 0) {
       tc_fence_after();
       const uint32_t xs = smem_u32(xa), ws = smem_u32(wimg);
-      for (int k = 0; k < a.K / 16; ++k) {
-        uint64_t bd = a.b_mn ? mnmajor_desc(ws, a.R, k) : kmajor_desc(ws, a.R, k);
-        mma_bf16(tm, kmajor_desc(xs, 128, k), bd, idesc, k > 0);
+      uint64_t ad = kmajor_desc(xs, 128, 0), bd = a.b_mn ? mnmajor_desc(ws, a.R, 0) : kmajor_desc(ws, a.R, 0);
+      const uint32_t step = a.b_mn ? 128u : 2u, block = a.b_mn ? 512u : a.R * 8u;  // per 16 K and per 64 K, in 16 bytes
+      for (int kb = 0; kb < a.K / 64; ++kb, ad += 1024u, bd += block) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) mma_bf16(tm, ad + 2u * k, bd + step * k, idesc, (kb > 0 || k > 0) ? 1u : 0u);
       }
       mma_commit(&mbar);
     }
@@ -295,9 +297,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_tn_kernel(TnArgs a) {
       const uint32_t xs = smem_u32(smem + uint32_t(b) * stage);
       const uint32_t ys = xs + 128u * uint32_t(K1) * 2u;
       for (int mb = 0; mb < K1 / 128; ++mb)
-        for (int k = 0; k < 8; ++k)
-          mma_bf16(tm + uint32_t(mb * a.N), mnmajor_desc(xs + uint32_t(mb) * 32768u, 128, k),
-                   mnmajor_desc(ys, 128, k), idesc, (t > t0 || k > 0) ? 1u : 0u);
+        mma_chain<8, 128, true, 128, true>(tm + uint32_t(mb * a.N), xs + uint32_t(mb) * 32768u, ys, idesc, t > t0);
       mma_commit(&mbar);
     }
     ok = mbar_wait(&mbar, ph, a.err);
