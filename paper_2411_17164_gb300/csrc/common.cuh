@@ -107,6 +107,34 @@ size_t scan_tmp_elems(int64_t n);
 xmgn_status exclusive_scan_i32(const int32_t* in, int64_t* out, int64_t n, int64_t* tmp, cudaStream_t s);
 xmgn_status exclusive_scan_i32(const int32_t* in, int32_t* out, int64_t n, int64_t* tmp, cudaStream_t s);
 
+// ---------------------------------------------------------------- launches
+// Programmatic dependent launch.  A kernel started with launch_pdl may begin
+// while the kernel before it on the stream still runs: it sets itself up
+// (barriers, TMEM, weights that no kernel of the call writes), calls pdl_wait()
+// before it touches anything else in global memory, and then pdl_trigger() to
+// let the next one begin.  As the trigger comes after the wait, whatever ran
+// before the predecessor is complete when a kernel begins: only the
+// predecessor's own results must wait for pdl_wait().  Without it a launch costs
+// a drain, a start and the set-up in sequence: on a 2k-node graph, where a
+// kernel runs 4 to 20 us, a training step (274 launches) went from 2.57 to 1.92 ms.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+template <class... P, class... A>
+inline void launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A&&... args) {
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, kernel, P(args)...);  // errors: the XMGN_LAUNCH_CHECK that follows
+}
+
 // ---------------------------------------------------------------- device helpers
 __device__ __forceinline__ void dev_flag(uint32_t* err, uint32_t code) {
   if (err) atomicOr(err, code);

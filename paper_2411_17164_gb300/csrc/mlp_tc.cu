@@ -426,6 +426,7 @@ __device__ __forceinline__ bool setup(uint64_t* wbar, uint64_t* mbar, uint32_t* 
     tmem_alloc(tbase, ncols);
     tmem_relinquish();
   }
+  if (w.late) pdl_wait();  // the images come from the kernel before
   if (tid < kH) {
     sm.cst[tid] = p.b1[tid];
     sm.cst[kH + tid] = tid < n2 ? p.b2[tid] : 0.f;
@@ -449,6 +450,8 @@ __device__ __forceinline__ bool setup(uint64_t* wbar, uint64_t* mbar, uint32_t* 
       copy(sm.w2l, w.w2lo, w.w2_bytes);
     }
   }
+  if (!w.late) pdl_wait();
+  pdl_trigger();
   return mbar_wait(wbar, 0, err);
 }
 
@@ -2484,7 +2487,7 @@ xmgn_status launch_fwd(const FwdArgs& a, cudaStream_t s) {
     XMGN_TRY(rows_map(&me, a.a0, a.rows));
     probe_begin(probe, s);
     tune_begin(TUNE_EDGE_FWD_ORDER, s);
-    edge_fwd_kernel<<<mlp_grid(a.rows), kThreads, sm, s>>>(b, me);
+    launch_pdl(edge_fwd_kernel, mlp_grid(a.rows), kThreads, sm, s, b, me);
     tune_end(TUNE_EDGE_FWD_ORDER, s);
   } else if constexpr (MODE == M_NODE) {
     if (!attr) {
@@ -2494,7 +2497,7 @@ xmgn_status launch_fwd(const FwdArgs& a, cudaStream_t s) {
     const uint32_t sm = carve_node_fwd(a.w, nullptr, nullptr) + 1024u;
     XMGN_TRY(check_smem<MODE>(sm));
     probe_begin(probe, s);
-    node_fwd_kernel<<<mlp_grid(a.rows), kThreads, sm, s>>>(a);
+    launch_pdl(node_fwd_kernel, mlp_grid(a.rows), kThreads, sm, s, a);
   } else {
     if (!attr) {
       XMGN_TRY(allow_max_smem(mlp_fwd_kernel<MODE>));
@@ -2503,7 +2506,7 @@ xmgn_status launch_fwd(const FwdArgs& a, cudaStream_t s) {
     const uint32_t sm = smem_bytes<MODE>(a.w, false);
     XMGN_TRY(check_smem<MODE>(sm));
     probe_begin(probe, s);
-    mlp_fwd_kernel<MODE><<<mlp_grid(a.rows), kThreads, sm, s>>>(a);
+    launch_pdl(mlp_fwd_kernel<MODE>, mlp_grid(a.rows), kThreads, sm, s, a);
   }
   probe_end(probe, s);
   XMGN_LAUNCH_CHECK();
@@ -2542,7 +2545,7 @@ xmgn_status launch_bwd(const BwdArgs& a, cudaStream_t s) {
     tune_begin(TUNE_EDGE_BWD_ORDER, s);
     tune_begin(TUNE_EDGE_BWD_TILES, s);
     if (tiles2) {
-      edge_bwd2_kernel<<<mlp_grid(a.rows), kThreads, sm, s>>>(b);
+      launch_pdl(edge_bwd2_kernel, mlp_grid(a.rows), kThreads, sm, s, b);
     } else {
       EdgeBwdMaps mp;
       XMGN_TRY(rows_map(&mp.e, a.a0, a.rows));
@@ -2550,14 +2553,14 @@ xmgn_status launch_bwd(const BwdArgs& a, cudaStream_t s) {
       XMGN_TRY(rows_map(&mp.dz1, a.dZ1g, a.rows));
       XMGN_TRY(rows_map(&mp.deo, a.dX0h, a.rows));
       if (warps32)
-        edge_bwd32_kernel<<<mlp_grid(a.rows), kT32, sm, s>>>(b, mp);
+        launch_pdl(edge_bwd32_kernel, mlp_grid(a.rows), kT32, sm, s, b, mp);
       else
-        edge_bwd_kernel<<<mlp_grid(a.rows), kThreads, sm, s>>>(b, mp);
+        launch_pdl(edge_bwd_kernel, mlp_grid(a.rows), kThreads, sm, s, b, mp);
     }
     tune_end(TUNE_EDGE_BWD_TILES, s);
     tune_end(TUNE_EDGE_BWD_ORDER, s);
   } else {
-    mlp_bwd_kernel<MODE><<<mlp_grid(a.rows), kThreads, sm, s>>>(a);
+    launch_pdl(mlp_bwd_kernel<MODE>, mlp_grid(a.rows), kThreads, sm, s, a);
   }
   probe_end(probe, s);
   XMGN_LAUNCH_CHECK();
@@ -2574,6 +2577,8 @@ namespace {
 __global__ void edge_inputs_bf16_kernel(const float* __restrict__ xyz, const int32_t* __restrict__ gid,
                                         const int32_t* __restrict__ recv, const int32_t* __restrict__ col, int64_t E,
                                         bf16* __restrict__ out) {
+  pdl_wait();
+  pdl_trigger();
   for (int64_t e = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; e < E; e += int64_t(gridDim.x) * blockDim.x) {
     int64_t i = recv[e], j = col[e];
     if (gid) {
@@ -2595,7 +2600,7 @@ __global__ void edge_inputs_bf16_kernel(const float* __restrict__ xyz, const int
 xmgn_status edge_inputs_bf16(const float* xyz, const int32_t* gid, const int32_t* recv, const int32_t* col,
                              int64_t E, bf16* out, cudaStream_t s) {
   if (E <= 0) return XMGN_OK;
-  edge_inputs_bf16_kernel<<<grid_for(E, 256, int64_t(num_sms()) * 16), 256, 0, s>>>(xyz, gid, recv, col, E, out);
+  launch_pdl(edge_inputs_bf16_kernel, grid_for(E, 256, int64_t(num_sms()) * 16), 256, 0, s, xyz, gid, recv, col, E, out);
   XMGN_LAUNCH_CHECK();
   return XMGN_OK;
 }

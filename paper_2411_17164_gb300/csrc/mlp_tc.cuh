@@ -21,6 +21,7 @@ struct MlpImgs {
   const uint8_t* w1lo;  // bf16(W1 - bf16(W1)) (all modes but the node MLP)
   const uint8_t* w2lo;  // bf16(W2 - bf16(W2))
   uint32_t w1_bytes, w2_bytes;
+  int late;  // the images are written by the kernel launched just before
 };
 
 struct MlpParams {

@@ -157,6 +157,8 @@ __device__ __forceinline__ void acc_bf16x4(float4& s, uint2 u) {
 // one tile were written by the edge kernel and are skipped.
 __global__ void agg_fixup_kernel(const float* __restrict__ part, const int64_t* __restrict__ rp, int64_t n,
                                  bf16* __restrict__ a16) {
+  pdl_wait();
+  pdl_trigger();
   const int lane = threadIdx.x & 31;
   const int64_t warp = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
   const int64_t nw = (int64_t(gridDim.x) * blockDim.x) >> 5;
@@ -228,6 +230,8 @@ __global__ void __launch_bounds__(256) seg_sums_kernel(const bf16* __restrict__ 
                                                        const int32_t* __restrict__ perm, int64_t n,
                                                        const bf16* __restrict__ da, bf16* __restrict__ S,
                                                        float* __restrict__ colp) {
+  pdl_wait();
+  pdl_trigger();
   constexpr int C = 128 / LPN, NG = 8 * (32 / LPN);  // features per lane, node groups per block
   __shared__ float red[2][NG][128];
   const int lane = threadIdx.x & 31;
@@ -303,6 +307,8 @@ SegShape seg_shape(int64_t n, int choice) {
 __global__ void __launch_bounds__(256) edge_beta_mv_kernel(const float* __restrict__ P, int64_t w1e0, int64_t b10,
                                                            int64_t stride, const float* __restrict__ G,
                                                            float* __restrict__ v) {
+  pdl_wait();
+  pdl_trigger();
   __shared__ float db1[128];
   const int l = blockIdx.x, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int64_t o = int64_t(l) * stride;
@@ -320,6 +326,8 @@ __global__ void __launch_bounds__(256) edge_beta_mv_kernel(const float* __restri
 
 __global__ void edge_beta_kernel(int L, int64_t be0, int64_t stride, const float* __restrict__ tsum,
                                  const float* __restrict__ v, float* __restrict__ G) {
+  pdl_wait();
+  pdl_trigger();
   const int k = threadIdx.x;
   float D = 0.f;
   for (int l = L - 1; l >= 0; --l) {
@@ -346,6 +354,8 @@ struct RedBatch {
 };
 
 __global__ void __launch_bounds__(256) reduce_parts_kernel(RedBatch b) {
+  pdl_wait();
+  pdl_trigger();
   __shared__ float red[8][32];
   const RedJob& J = b.j[blockIdx.y];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -384,7 +394,7 @@ xmgn_status reduce_batch(const std::vector<RedJob>& jobs, cudaStream_t s) {
       if (b.j[i].count > most) most = b.j[i].count;
     }
     const int64_t gx = (most + 31) / 32 < 1024 ? (most + 31) / 32 : 1024;
-    reduce_parts_kernel<<<dim3(unsigned(gx), unsigned(b.n)), 256, 0, s>>>(b);
+    launch_pdl(reduce_parts_kernel, dim3(unsigned(gx), unsigned(b.n)), 256, 0, s, b);
     XMGN_LAUNCH_CHECK();
   }
   return XMGN_OK;
@@ -415,6 +425,7 @@ MlpImgs imgs_of(const uint8_t* base, const Img& a, const Img& b, const Img* al =
   m.w2lo = bl ? base + bl->off : nullptr;
   m.w1_bytes = a.bytes();
   m.w2_bytes = b.bytes();
+  m.late = 0;
   return m;
 }
 
@@ -549,6 +560,7 @@ xmgn_status bf16_forward(const ParamPlan& p, const float* P, const xmgn_graph& g
   f.xyz = xyz;
   f.fourier = p.fourier;
   f.w = imgs_of(c.img, ip.new1, ip.new2, &ip.new1l, &ip.new2l);
+  f.w.late = 1;
   f.p = params_of(P, p.ne);
   f.o32 = c.h32;
   f.o16 = c.h16;
@@ -591,7 +603,7 @@ xmgn_status bf16_forward(const ParamPlan& p, const float* P, const xmgn_graph& g
                                 layer_elems * sizeof(bf16), cudaMemcpyDeviceToHost, oc->copy));
       XMGN_CUDA(cudaEventRecord(oc->moved[l % kRing], oc->copy));
     }
-    agg_fixup_kernel<<<grid_for(n, 256, int64_t(num_sms()) * 16), 256, 0, s>>>(w.agg_part, g.row_ptr, n, a16);
+    launch_pdl(agg_fixup_kernel, grid_for(n, 256, int64_t(num_sms()) * 16), 256, 0, s, w.agg_part, g.row_ptr, n, a16);
     XMGN_LAUNCH_CHECK();
     FwdArgs fn = f;
     fn.rows = n;
@@ -738,9 +750,9 @@ xmgn_status bf16_backward(const ParamPlan& p, const float* P, const xmgn_graph& 
     const unsigned sg = ss.grid;
     tune_begin(TUNE_SEG_SUMS, s);
     if (ss.lpn == 32)
-      seg_sums_kernel<32><<<sg, 256, 0, s>>>(w.dZ1g, g.row_ptr, g.csc_perm, n, w.dagg, w.S16, w.colp);
+      launch_pdl(seg_sums_kernel<32>, sg, 256, 0, s, w.dZ1g, g.row_ptr, g.csc_perm, n, w.dagg, w.S16, w.colp);
     else
-      seg_sums_kernel<16><<<sg, 256, 0, s>>>(w.dZ1g, g.row_ptr, g.csc_perm, n, w.dagg, w.S16, w.colp);
+      launch_pdl(seg_sums_kernel<16>, sg, 256, 0, s, w.dZ1g, g.row_ptr, g.csc_perm, n, w.dagg, w.S16, w.colp);
     XMGN_LAUNCH_CHECK();
     tune_end(TUNE_SEG_SUMS, s);
     {  // dW1_e, dW2, db2, dgamma (per-CTA partials of the edge kernel), db1 and T_l (seg_sums partials)
@@ -764,10 +776,10 @@ xmgn_status bf16_backward(const ParamPlan& p, const float* P, const xmgn_graph& 
       if (p.edge[l].W1 != p.edge[0].W1 + l * stride || p.edge[l].b1 != p.edge[0].b1 + l * stride ||
           p.edge[l].be != p.edge[0].be + l * stride)
         return fail(XMGN_ERR_ARG, "edge MLP parameters are not laid out with a fixed stride per layer");
-    edge_beta_mv_kernel<<<p.L, 256, 0, s>>>(P, p.edge[0].W1 + 2 * int64_t(H) * H, p.edge[0].b1, stride, G,
+    launch_pdl(edge_beta_mv_kernel, p.L, 256, 0, s, P, p.edge[0].W1 + 2 * int64_t(H) * H, p.edge[0].b1, stride, G,
                                             w.vbeta);
     XMGN_LAUNCH_CHECK();
-    edge_beta_kernel<<<1, 128, 0, s>>>(p.L, p.edge[0].be, stride, w.tsum, w.vbeta, G);
+    launch_pdl(edge_beta_kernel, 1, 128, 0, s, p.L, p.edge[0].be, stride, w.tsum, w.vbeta, G);
     XMGN_LAUNCH_CHECK();
   }
   // edge encoder

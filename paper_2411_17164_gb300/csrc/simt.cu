@@ -522,6 +522,8 @@ __global__ void loss_kernel(const float* __restrict__ y, int64_t n, int out,
                             const float* __restrict__ t, const int32_t* __restrict__ gid,
                             const uint8_t* __restrict__ hop, float scale, float* __restrict__ dy,
                             float* __restrict__ yg, float* __restrict__ part) {
+  pdl_wait();
+  pdl_trigger();
   __shared__ float red[256];
   float s = 0.f;
   for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n;
@@ -549,6 +551,8 @@ __global__ void loss_kernel(const float* __restrict__ y, int64_t n, int out,
 }
 
 __global__ void loss_reduce_kernel(const float* __restrict__ part, int nb, float scale, float* loss) {
+  pdl_wait();
+  pdl_trigger();
   if (threadIdx.x == 0 && blockIdx.x == 0) {
     float s = 0.f;
     for (int b = 0; b < nb; ++b) s += part[b];
@@ -558,6 +562,8 @@ __global__ void loss_reduce_kernel(const float* __restrict__ part, int nb, float
 
 __global__ void accum_kernel(float* __restrict__ dst, float* __restrict__ comp,
                              const float* __restrict__ src, int64_t n) {
+  pdl_wait();
+  pdl_trigger();
   for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n;
        i += int64_t(gridDim.x) * blockDim.x) {
     float x = src[i];
@@ -743,17 +749,17 @@ xmgn_status mse_loss(const float* y, int64_t n, int out, const float* targets, c
                      const uint8_t* hop, int64_t n_norm, float* loss, float* dy, float* y_global,
                      float* part, cudaStream_t s) {
   const float scale = 1.f / (float(out) * float(n_norm));
-  loss_kernel<<<kLossBlocks, 256, 0, s>>>(y, n, out, targets, gid, hop, scale, dy, y_global, part);
+  launch_pdl(loss_kernel, kLossBlocks, 256, 0, s, y, n, out, targets, gid, hop, scale, dy, y_global, part);
   XMGN_LAUNCH_CHECK();
   if (loss) {
-    loss_reduce_kernel<<<1, 32, 0, s>>>(part, kLossBlocks, scale, loss);
+    launch_pdl(loss_reduce_kernel, 1, 32, 0, s, part, kLossBlocks, scale, loss);
     XMGN_LAUNCH_CHECK();
   }
   return XMGN_OK;
 }
 
 xmgn_status accumulate_grad(float* dst, float* comp, const float* src, int64_t n, cudaStream_t s) {
-  accum_kernel<<<grid_for(n, 256), 256, 0, s>>>(dst, comp, src, n);
+  launch_pdl(accum_kernel, grid_for(n, 256), 256, 0, s, dst, comp, src, n);
   XMGN_LAUNCH_CHECK();
   return XMGN_OK;
 }

@@ -21,6 +21,8 @@ struct PackBatch {
 
 // One image per blockIdx.y; element (r, c) of rows [r0, r0+nr) of the image.
 __global__ void pack_kernel(PackBatch b) {
+  pdl_wait();
+  pdl_trigger();
   const PackJob& J = b.j[blockIdx.y];
   const int64_t total = int64_t(J.nr) * J.C;
   for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < total;
@@ -113,6 +115,8 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(GemmArgs a, const 
       bulk_g2s(wimg + o, a.img + o, n, &wbar);
     }
   }
+  pdl_wait();  // the weight image is older than the kernel before; the rows are not
+  pdl_trigger();
   const int64_t tiles = (a.M + 127) / 128;
   if (blockIdx.x < tiles) issue_rows(xbuf[0], a.A, int64_t(blockIdx.x) * 128, a.M, tid);
   bool ok = mbar_wait(&wbar, 0, a.err);
@@ -264,6 +268,8 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_tn_kernel(TnArgs a) {
   __syncthreads();
   tc_fence_after();
   const uint32_t tm = tbase;
+  pdl_wait();
+  pdl_trigger();
   const int64_t tiles = (a.M + 127) / 128;
   const int64_t t0 = int64_t(blockIdx.x) * a.tiles_per_cta;
   const int64_t t1 = min(tiles, t0 + a.tiles_per_cta);
@@ -335,6 +341,8 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_tn_kernel(TnArgs a) {
 __global__ void __launch_bounds__(256) tn_reduce_kernel(const float* __restrict__ part, int nparts, int K1, int N,
                                                         int kvalid, int nvalid, int nsplit,
                                                         float* __restrict__ out) {
+  pdl_wait();
+  pdl_trigger();
   __shared__ float red[8][32];
   const int64_t len = int64_t(K1) * N;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -389,7 +397,7 @@ xmgn_status pack_images(const std::vector<PackJob>& jobs, cudaStream_t s) {
       if (e > most) most = e;
     }
     const int64_t gx = (most + 255) / 256 < 128 ? (most + 255) / 256 : 128;
-    pack_kernel<<<dim3(unsigned(gx), unsigned(b.n)), 256, 0, s>>>(b);
+    launch_pdl(pack_kernel, dim3(unsigned(gx), unsigned(b.n)), 256, 0, s, b);
     XMGN_LAUNCH_CHECK();
   }
   return XMGN_OK;
@@ -427,7 +435,7 @@ xmgn_status tc_gemm(const Bf16Rows& A, int64_t M, const uint8_t* img_base, const
     XMGN_TRY(allow_max_smem(tc_gemm_kernel));
     attr = true;
   }
-  tc_gemm_kernel<<<tc_grid((M + 127) / 128), kThreads, smem, s>>>(a, td);
+  launch_pdl(tc_gemm_kernel, tc_grid((M + 127) / 128), kThreads, smem, s, a, td);
   XMGN_LAUNCH_CHECK();
   return XMGN_OK;
 }
@@ -459,9 +467,9 @@ xmgn_status tc_gemm_tn(const Bf16Rows& X, const bf16* Y, int64_t ldy, int N, int
     attr = true;
   }
   tune_begin(TUNE_TN_GRID, s);
-  tc_gemm_tn_kernel<<<grid, kThreads, smem, s>>>(a);
+  launch_pdl(tc_gemm_tn_kernel, grid, kThreads, smem, s, a);
   XMGN_LAUNCH_CHECK();
-  tn_reduce_kernel<<<unsigned((int64_t(K1) * N + 31) / 32), 256, 0, s>>>(part, grid, K1, N, kvalid, nvalid, nsplit,
+  launch_pdl(tn_reduce_kernel, unsigned((int64_t(K1) * N + 31) / 32), 256, 0, s, part, grid, K1, N, kvalid, nvalid, nsplit,
                                                                          out);
   XMGN_LAUNCH_CHECK();
   tune_end(TUNE_TN_GRID, s);
