@@ -90,6 +90,8 @@ struct BWs {
   bf16 *dagg, *de;  // gradients of a (node level) and of the edge state, bf16
   float* agg_part;  // [edge tiles][2][H]: partial sums of receivers that cross a tile boundary
   bf16 *A1g, *dZ2g, *dZ1g, *S16, *X16;
+  bf16* dZ1n;    // dZ1 of the node-level MLPs (n x H), kept until the layer's weight-gradient products
+  float* cpartn; // column partials of the node-level MLPs
   float* colp;  // [seg_sums blocks][2][H]: column partials of the receiver sums and of indeg * da
   float* tsum;  // [L][H]: sum over nodes of indeg(i) * da_i, per layer
   float* vbeta; // [L][H]: db1_l W1_e,l^T, per layer
@@ -128,7 +130,10 @@ void ws_layout(Arena& A, const ParamPlan& p, int64_t n, int64_t E, BWs& w) {
   w.de = A.take<bf16>(size_t(E) * H);
   w.wpart = A.take<float>(size_t(g) * 2 * 128 * H);
   w.cpart = A.take<float>(size_t(g) * 4 * H);
-  w.tnpart = A.take<float>(tc_gemm_tn_part_elems(256, 256));
+  w.cpartn = A.take<float>(size_t(g) * 4 * H);
+  w.tnpart = A.take<float>(tc_gemm_tn_part_elems(256, 128) + tc_gemm_tn_part_elems(128, 128) +
+                           tc_gemm_tn_part_elems(128, 256));
+  w.dZ1n = A.take<bf16>(size_t(n) * H);
   w.A1g = A.take<bf16>(size_t(n) * H);
   w.dZ2g = A.take<bf16>(size_t(n) * H);
   w.dZ1g = A.take<bf16>(size_t(R) * H);
@@ -336,70 +341,6 @@ __global__ void edge_beta_kernel(int L, int64_t be0, int64_t stride, const float
   }
 }
 
-// Sums of per-CTA partials, out[i] = sum over parts p of part[p*stride + off
-// + i] for i < count, up to kRedJobs outputs per launch (blockIdx.y = job).
-// A block owns 32 consecutive outputs; warp w sums the parts p = w (mod 8) in
-// four interleaved running sums (p = w + 8m by m mod 4), and the sums are
-// combined in a fixed tree: deterministic.
-constexpr int kRedJobs = 8;
-struct RedJob {
-  const float* part;
-  int nparts;
-  int64_t stride, off, count;
-  float* out;
-};
-struct RedBatch {
-  int n;
-  RedJob j[kRedJobs];
-};
-
-__global__ void __launch_bounds__(256) reduce_parts_kernel(RedBatch b) {
-  pdl_wait();
-  pdl_trigger();
-  __shared__ float red[8][32];
-  const RedJob& J = b.j[blockIdx.y];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  for (int64_t i0 = int64_t(blockIdx.x) * 32; i0 < J.count; i0 += int64_t(gridDim.x) * 32) {
-    const int64_t i = i0 + lane;
-    float s = 0.f;
-    if (i < J.count) {  // parts w, w+8, ... in four interleaved running sums (independent loads in flight)
-      const float* q = J.part + J.off + i;
-      float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
-      int p = w;
-      for (; p + 24 < J.nparts; p += 32) {
-        s0 += q[int64_t(p) * J.stride];
-        s1 += q[int64_t(p + 8) * J.stride];
-        s2 += q[int64_t(p + 16) * J.stride];
-        s3 += q[int64_t(p + 24) * J.stride];
-      }
-      for (; p < J.nparts; p += 8) s0 += q[int64_t(p) * J.stride];
-      s = (s0 + s1) + (s2 + s3);
-    }
-    red[w][lane] = s;
-    __syncthreads();
-    if (w == 0 && i < J.count)
-      J.out[i] = ((red[0][lane] + red[1][lane]) + (red[2][lane] + red[3][lane])) +
-                 ((red[4][lane] + red[5][lane]) + (red[6][lane] + red[7][lane]));
-    __syncthreads();
-  }
-}
-
-xmgn_status reduce_batch(const std::vector<RedJob>& jobs, cudaStream_t s) {
-  for (size_t b0 = 0; b0 < jobs.size(); b0 += kRedJobs) {
-    RedBatch b;
-    b.n = int(jobs.size() - b0 < size_t(kRedJobs) ? jobs.size() - b0 : size_t(kRedJobs));
-    int64_t most = 1;
-    for (int i = 0; i < b.n; ++i) {
-      b.j[i] = jobs[b0 + i];
-      if (b.j[i].count > most) most = b.j[i].count;
-    }
-    const int64_t gx = (most + 31) / 32 < 1024 ? (most + 31) / 32 : 1024;
-    launch_pdl(reduce_parts_kernel, dim3(unsigned(gx), unsigned(b.n)), 256, 0, s, b);
-    XMGN_LAUNCH_CHECK();
-  }
-  return XMGN_OK;
-}
-
 // bias / gamma / beta gradients from the per-CTA column partials
 void col_jobs(std::vector<RedJob>& j, const float* cpart, int nparts, int H, const MlpOff& o, float* G) {
   j.push_back({cpart, nparts, 4 * int64_t(H), 0, o.hid, G + o.b1});
@@ -408,12 +349,6 @@ void col_jobs(std::vector<RedJob>& j, const float* cpart, int nparts, int H, con
     j.push_back({cpart, nparts, 4 * int64_t(H), 2 * int64_t(H), o.out, G + o.g});
     j.push_back({cpart, nparts, 4 * int64_t(H), 3 * int64_t(H), o.out, G + o.be});
   }
-}
-
-xmgn_status reduce_cols(const float* cpart, int nparts, int H, const MlpOff& o, float* G, cudaStream_t s) {
-  std::vector<RedJob> j;
-  col_jobs(j, cpart, nparts, H, o, G);
-  return reduce_batch(j, s);
 }
 
 MlpImgs imgs_of(const uint8_t* base, const Img& a, const Img& b, const Img* al = nullptr,
@@ -697,11 +632,23 @@ xmgn_status bf16_backward(const ParamPlan& p, const float* P, const xmgn_graph& 
   bd.dY1 = w.dy32;
   bd.dX0 = w.dh;
   bd.out_w = p.out;
+  bd.dZ1g = w.dZ1n;
+  bd.cpart = w.cpartn;
   XMGN_TRY(mlp_bwd_tc(M_DEC, bd, s));
-  XMGN_TRY(reduce_cols(w.cpart, gn, H, p.dec, G, s));
-  XMGN_TRY(tc_gemm_tn(rows_of(hL, H), w.dZ1g, H, H, n, G + p.dec.W1, H, H, H, w.tnpart, s));
-  XMGN_TRY(tc_gemm_tn(rows_of(w.A1g, H), w.dZ2g, 64, 64, n, G + p.dec.W2, H, p.out, p.out, w.tnpart, s));
+  {
+    std::vector<RedJob> red;
+    XMGN_TRY(tc_gemm_tn({{rows_of(hL, H), w.dZ1n, H, H, G + p.dec.W1, H, H, H},
+                         {rows_of(w.A1g, H), w.dZ2g, 64, 64, G + p.dec.W2, H, p.out, p.out}}, n, w.tnpart, red, s));
+    col_jobs(red, w.cpartn, gn, H, p.dec, G);
+    XMGN_TRY(reduce_batch(red, s));
+  }
 
+  // Weight-gradient products of the node MLP: with the layer's other one in a
+  // single launch after the edge kernel, or, where their five operands (10 H
+  // bytes a node) and partials take longer to read again after the edge kernel
+  // has streamed through L2 than two launches cost, right behind the node kernel
+  // (2k nodes: 1.93 -> 1.63 ms a step in one; 200k nodes: 31.12 ms, 32.0 in one).
+  const bool node_products_now = size_t(n) * H * 10 > (size_t(32) << 20);
   for (int l = p.L - 1; l >= 0; --l) {
     const LayerImgs& li = ip.layer[l];
     const bf16* h16 = c.h16 + size_t(l) * n * H;
@@ -720,10 +667,20 @@ xmgn_status bf16_backward(const ParamPlan& p, const float* P, const xmgn_graph& 
     bn.dY1 = w.dh;
     bn.dX0 = w.dh;
     bn.dX1h = w.dagg;
+    bn.dZ1g = w.dZ1n;
+    bn.cpart = w.cpartn;
     XMGN_TRY(mlp_bwd_tc(M_NODE, bn, s));
-    XMGN_TRY(reduce_cols(w.cpart, gn, H, on, G, s));
-    XMGN_TRY(tc_gemm_tn(rows_of(h16, H, a16, H), w.dZ1g, H, H, n, G + on.W1, 2 * H, H, H, w.tnpart, s));
-    XMGN_TRY(tc_gemm_tn(rows_of(w.A1g, H), w.dZ2g, H, H, n, G + on.W2, H, H, H, w.tnpart, s));
+    // the layer's node-level weight gradients: products, then every sum of partials in one launch
+    std::vector<TnJob> tn = {{rows_of(h16, H, a16, H), w.dZ1n, H, H, G + on.W1, 2 * H, H, H},
+                             {rows_of(w.A1g, H), w.dZ2g, H, H, G + on.W2, H, H, H}};
+    std::vector<RedJob> red;
+    col_jobs(red, w.cpartn, gn, H, on, G);
+    if (node_products_now) {
+      XMGN_TRY(tc_gemm_tn(tn, n, w.tnpart, red, s));
+      XMGN_TRY(reduce_batch(red, s));
+      tn.clear();
+      red.clear();
+    }
     // edge update e' = e + m, a_i = sum_j m_ij (node projections checkpointed, or recomputed with offload)
     const bf16* Pl = w.P;
     if (c.P16)
@@ -755,20 +712,22 @@ xmgn_status bf16_backward(const ParamPlan& p, const float* P, const xmgn_graph& 
       launch_pdl(seg_sums_kernel<16>, sg, 256, 0, s, w.dZ1g, g.row_ptr, g.csc_perm, n, w.dagg, w.S16, w.colp);
     XMGN_LAUNCH_CHECK();
     tune_end(TUNE_SEG_SUMS, s);
-    {  // dW1_e, dW2, db2, dgamma (per-CTA partials of the edge kernel), db1 and T_l (seg_sums partials)
-      const int64_t cs = 4 * int64_t(H), ps = 2 * int64_t(H);
-      std::vector<RedJob> j = {{w.colp, int(sg), ps, 0, H, G + oe.b1},
-                               {w.colp, int(sg), ps, H, H, w.tsum + int64_t(l) * H}};
-      if (E > 0) {  // without edges the edge kernel left no partials (those gradients stay zero)
-        j.push_back({w.wpart, ge, 2 * 128 * int64_t(H), 0, int64_t(H) * H, G + oe.W1 + 2 * int64_t(H) * H});
-        j.push_back({w.wpart, ge, 2 * 128 * int64_t(H), 128 * int64_t(H), int64_t(H) * H, G + oe.W2});
-        j.push_back({w.cpart, ge, cs, H, H, G + oe.b2});
-        j.push_back({w.cpart, ge, cs, 2 * int64_t(H), H, G + oe.g});
-      }
-      XMGN_TRY(reduce_batch(j, s));
-    }
     XMGN_TRY(tc_gemm(rows_of(w.S16, 2 * H), n, c.img, li.ewrs, true, H, w.dh, H, true, s));
-    XMGN_TRY(tc_gemm_tn(rows_of(h16, H), w.S16, 2 * H, 2 * H, n, G + oe.W1, H, 2 * H, H, w.tnpart, s));
+    {
+      tn.push_back({rows_of(h16, H), w.S16, 2 * H, 2 * H, G + oe.W1, H, 2 * H, H});
+      XMGN_TRY(tc_gemm_tn(tn, n, w.tnpart, red, s));
+      // db1 and T_l (seg_sums partials); dW1_e, dW2, db2, dgamma (per-CTA partials of the edge kernel)
+      const int64_t cs = 4 * int64_t(H), ps = 2 * int64_t(H);
+      red.push_back({w.colp, int(sg), ps, 0, H, G + oe.b1});
+      red.push_back({w.colp, int(sg), ps, H, H, w.tsum + int64_t(l) * H});
+      if (E > 0) {  // without edges the edge kernel left no partials (those gradients stay zero)
+        red.push_back({w.wpart, ge, 2 * 128 * int64_t(H), 0, int64_t(H) * H, G + oe.W1 + 2 * int64_t(H) * H});
+        red.push_back({w.wpart, ge, 2 * 128 * int64_t(H), 128 * int64_t(H), int64_t(H) * H, G + oe.W2});
+        red.push_back({w.cpart, ge, cs, H, H, G + oe.b2});
+        red.push_back({w.cpart, ge, cs, 2 * int64_t(H), H, G + oe.g});
+      }
+      XMGN_TRY(reduce_batch(red, s));
+    }
   }
   {  // dbeta of the edge MLPs from db1 and T_l (the edge kernel does not sum it)
     const int64_t stride = p.L > 1 ? p.edge[1].W1 - p.edge[0].W1 : 0;
@@ -808,10 +767,16 @@ xmgn_status bf16_backward(const ParamPlan& p, const float* P, const xmgn_graph& 
   bne.w = imgs_of(c.img, ip.new1, ip.new2, &ip.new1l, &ip.new2l);
   bne.p = params_of(P, p.ne);
   bne.dY1 = w.dh;
+  bne.dZ1g = w.dZ1n;
+  bne.cpart = w.cpartn;
   XMGN_TRY(mlp_bwd_tc(M_NENC, bne, s));
-  XMGN_TRY(reduce_cols(w.cpart, gn, H, p.ne, G, s));
-  XMGN_TRY(tc_gemm_tn(rows_of(w.X16, 128), w.dZ1g, H, H, n, G + p.ne.W1, p.in_enc, H, H, w.tnpart, s));
-  XMGN_TRY(tc_gemm_tn(rows_of(w.A1g, H), w.dZ2g, H, H, n, G + p.ne.W2, H, H, H, w.tnpart, s));
+  {
+    std::vector<RedJob> red;
+    XMGN_TRY(tc_gemm_tn({{rows_of(w.X16, 128), w.dZ1n, H, H, G + p.ne.W1, p.in_enc, H, H},
+                         {rows_of(w.A1g, H), w.dZ2g, H, H, G + p.ne.W2, H, H, H}}, n, w.tnpart, red, s));
+    col_jobs(red, w.cpartn, gn, H, p.ne, G);
+    XMGN_TRY(reduce_batch(red, s));
+  }
   if (off) {  // join the copy stream
     XMGN_CUDA(cudaEventRecord(oc->sync[1], oc->copy));
     XMGN_CUDA(cudaStreamWaitEvent(s, oc->sync[1], 0));

@@ -246,8 +246,12 @@ struct TnArgs {
   float* part;  // [cta][K1][N]
   uint32_t* err;
 };
+struct TnLaunch {
+  TnArgs j[kTnBatch];  // blockIdx.y
+};
 
-__global__ void __launch_bounds__(kThreads, 1) tc_gemm_tn_kernel(TnArgs a) {
+__global__ void __launch_bounds__(kThreads, 1) tc_gemm_tn_kernel(const __grid_constant__ TnLaunch L) {
+  const TnArgs& a = L.j[blockIdx.y];
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   __shared__ uint64_t mbar;
@@ -335,29 +339,66 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_tn_kernel(TnArgs a) {
   if (warp == 0) tmem_dealloc(tm, 512);
 }
 
-// Sums the per-CTA partials: a block owns 32 consecutive outputs, warp w sums
-// the parts p = w (mod 8) in increasing order, the eight warp sums combine in
-// a fixed tree (deterministic).
-__global__ void __launch_bounds__(256) tn_reduce_kernel(const float* __restrict__ part, int nparts, int K1, int N,
-                                                        int kvalid, int nvalid, int nsplit,
-                                                        float* __restrict__ out) {
+// Sums of per-CTA partials, up to kRedJobs outputs per launch: a block owns 32
+// consecutive outputs of one job, warp w sums the parts p = w (mod 8) (plain
+// jobs in four interleaved running sums, p = w + 8m by m mod 4), and the warps'
+// sums are combined in a fixed tree: deterministic.  Jobs are batched because
+// each is a few microseconds of latency: a layer's nine sums took four launches.
+constexpr int kRedJobs = 16;
+struct RedBatch {
+  int n;
+  int block0[kRedJobs + 1];  // first block of each job
+  RedJob j[kRedJobs];
+};
+
+__global__ void __launch_bounds__(256) reduce_parts_kernel(const __grid_constant__ RedBatch b) {
   pdl_wait();
   pdl_trigger();
   __shared__ float red[8][32];
-  const int64_t len = int64_t(K1) * N;
+  int at = 0;
+  while (at + 1 < b.n && int(blockIdx.x) >= b.block0[at + 1]) ++at;
+  const RedJob& J = b.j[at];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int64_t i = int64_t(blockIdx.x) * 32 + lane;
+  const int64_t i = int64_t(int(blockIdx.x) - b.block0[at]) * 32 + lane;
   float s = 0.f;
-  if (i < len)
-    for (int p = w; p < nparts; p += 8) s += part[int64_t(p) * len + i];
+  if (i < J.count) {
+    const int np = J.nparts;
+    const int64_t step = 8 * J.stride;
+    const float* __restrict__ q = J.part + J.off + i + w * J.stride;
+    int p = w;
+    if (J.K1) {
+      for (; p + 56 < np; p += 64, q += 8 * step) {  // eight loads in flight, added in part order
+        float v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) v[u] = q[u * step];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) s += v[u];
+      }
+      for (; p < np; p += 8, q += step) s += *q;
+    } else {
+      float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
+#pragma unroll 2
+      for (; p + 24 < np; p += 32, q += 4 * step) {
+        s0 += q[0];
+        s1 += q[step];
+        s2 += q[2 * step];
+        s3 += q[3 * step];
+      }
+      for (; p < np; p += 8, q += step) s0 += *q;
+      s = (s0 + s1) + (s2 + s3);
+    }
+  }
   red[w][lane] = s;
   __syncthreads();
-  if (w != 0 || i >= len) return;
-  const int k = int(i / N), n = int(i % N);
-  if (k >= kvalid || n >= nvalid) return;
-  out[(int64_t(n / nsplit) * K1 + k) * nsplit + n % nsplit] =
-      ((red[0][lane] + red[1][lane]) + (red[2][lane] + red[3][lane])) +
-      ((red[4][lane] + red[5][lane]) + (red[6][lane] + red[7][lane]));
+  if (w != 0 || i >= J.count) return;
+  int64_t o = i;
+  if (J.K1) {
+    const int k = int(i / J.N), n = int(i % J.N);
+    if (k >= J.kvalid || n >= J.nvalid) return;
+    o = (int64_t(n / J.nsplit) * J.K1 + k) * J.nsplit + n % J.nsplit;
+  }
+  J.out[o] = ((red[0][lane] + red[1][lane]) + (red[2][lane] + red[3][lane])) +
+             ((red[4][lane] + red[5][lane]) + (red[6][lane] + red[7][lane]));
 }
 
 }  // namespace
@@ -442,37 +483,62 @@ xmgn_status tc_gemm(const Bf16Rows& A, int64_t M, const uint8_t* img_base, const
 
 size_t tc_gemm_tn_part_elems(int K1, int N) { return size_t(num_sms()) * size_t(K1) * size_t(N); }
 
-xmgn_status tc_gemm_tn(const Bf16Rows& X, const bf16* Y, int64_t ldy, int N, int64_t M, float* out,
-                       int kvalid, int nvalid, int nsplit, float* part, cudaStream_t s) {
-  const int K1 = X.K();
-  if ((K1 != 128 && K1 != 256) || N % 64 || N > 256 || (K1 / 128) * N > 512)
-    return fail(XMGN_ERR_UNSUPPORTED, "tc_gemm_tn shape K1=%d N=%d", K1, N);
+xmgn_status tc_gemm_tn(const std::vector<TnJob>& jobs, int64_t M, float* part, std::vector<RedJob>& red,
+                       cudaStream_t s) {
   const int64_t tiles = (M + 127) / 128;
   // one CTA per SM, or (tuned) one per two SMs: half the partials to reduce
   const int full = tc_grid(tiles);
   const int grid = tune_choice(TUNE_TN_GRID, M) == 1 && full > 1 ? (full + 1) / 2 : full;
-  TnArgs a;
-  a.X = X;
-  a.Y = Y;
-  a.ldy = ldy;
-  a.N = N;
-  a.M = M;
-  a.tiles_per_cta = (tiles + grid - 1) / grid;
-  a.part = part;
-  a.err = device_error_word();
-  const size_t smem = 1024 + 2 * size_t(128) * (K1 + N) * 2;
+  if (jobs.empty() || jobs.size() > size_t(kTnBatch)) return fail(XMGN_ERR_ARG, "tc_gemm_tn: %zu jobs", jobs.size());
+  TnLaunch L{};
+  size_t smem = 0;
+  for (size_t i = 0; i < jobs.size(); ++i) {
+    const TnJob& j = jobs[i];
+    const int K1 = j.X.K(), N = j.N;
+    if ((K1 != 128 && K1 != 256) || N % 64 || N > 256 || (K1 / 128) * N > 512)
+      return fail(XMGN_ERR_UNSUPPORTED, "tc_gemm_tn shape K1=%d N=%d", K1, N);
+    TnArgs& a = L.j[i];
+    a.X = j.X;
+    a.Y = j.Y;
+    a.ldy = j.ldy;
+    a.N = N;
+    a.M = M;
+    a.tiles_per_cta = (tiles + grid - 1) / grid;
+    a.part = part;
+    a.err = device_error_word();
+    const size_t need = 1024 + 2 * size_t(128) * (K1 + N) * 2;
+    if (need > smem) smem = need;
+    const int64_t len = int64_t(K1) * N;
+    red.push_back({part, grid, len, 0, len, j.out, K1, N, j.kvalid, j.nvalid, j.nsplit});
+    part += tc_gemm_tn_part_elems(K1, N);
+  }
   static bool attr = false;
   if (!attr) {
     XMGN_TRY(allow_max_smem(tc_gemm_tn_kernel));
     attr = true;
   }
   tune_begin(TUNE_TN_GRID, s);
-  launch_pdl(tc_gemm_tn_kernel, grid, kThreads, smem, s, a);
-  XMGN_LAUNCH_CHECK();
-  launch_pdl(tn_reduce_kernel, unsigned((int64_t(K1) * N + 31) / 32), 256, 0, s, part, grid, K1, N, kvalid, nvalid, nsplit,
-                                                                         out);
+  launch_pdl(tc_gemm_tn_kernel, dim3(unsigned(grid), unsigned(jobs.size())), kThreads, smem, s, L);
   XMGN_LAUNCH_CHECK();
   tune_end(TUNE_TN_GRID, s);
+  return XMGN_OK;
+}
+
+xmgn_status reduce_batch(const std::vector<RedJob>& jobs, cudaStream_t s) {
+  for (size_t b0 = 0; b0 < jobs.size(); b0 += kRedJobs) {
+    RedBatch b{};
+    b.n = int(jobs.size() - b0 < size_t(kRedJobs) ? jobs.size() - b0 : size_t(kRedJobs));
+    int64_t blocks = 0;
+    for (int i = 0; i < b.n; ++i) {
+      b.j[i] = jobs[b0 + i];
+      b.block0[i] = int(blocks);
+      blocks += (b.j[i].count + 31) / 32;
+    }
+    b.block0[b.n] = int(blocks);
+    if (blocks == 0) continue;
+    launch_pdl(reduce_parts_kernel, unsigned(blocks), 256, 0, s, b);
+    XMGN_LAUNCH_CHECK();
+  }
   return XMGN_OK;
 }
 

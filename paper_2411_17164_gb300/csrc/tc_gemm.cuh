@@ -58,13 +58,37 @@ struct Bf16Rows {
 xmgn_status tc_gemm(const Bf16Rows& A, int64_t M, const uint8_t* img_base, const Img& img, bool b_mn,
                     int N, float* D, int64_t ldd, bool accumulate, cudaStream_t s, bf16* D16 = nullptr);
 
-// G = X^T Y summed over M rows; X has K1 columns (128 or 256), Y has N
-// columns (64..256).  Result element (k, n), for k < kvalid and n < nvalid,
-// lands in out[((n / nsplit) * K1 + k) * nsplit + n % nsplit] (written, not
-// added).  `part` needs tc_gemm_tn_part_elems floats.
+// Sums of per-CTA partials in a fixed order.  Plain (K1 = 0): out[i] = sum over
+// parts p of part[p*stride + off + i], i < count.  Of an X^T Y product (K1 > 0,
+// part [p][K1][N], count = K1 N): element (k, n), for k < kvalid and n <
+// nvalid, lands in out[((n / nsplit) * K1 + k) * nsplit + n % nsplit].
+struct RedJob {
+  const float* part;
+  int nparts;
+  int64_t stride, off, count;
+  float* out;
+  int K1 = 0, N = 0, kvalid = 0, nvalid = 0, nsplit = 0;
+};
+xmgn_status reduce_batch(const std::vector<RedJob>& jobs, cudaStream_t s);
+
+// One product G = X^T Y summed over rows; X has K1 columns (128 or 256), Y has
+// N columns (64..256); the result goes where the RedJob form above says
+// (written, not added).
+struct TnJob {
+  Bf16Rows X;
+  const bf16* Y;
+  int64_t ldy;
+  int N;
+  float* out;
+  int kvalid, nvalid, nsplit;
+};
+constexpr int kTnBatch = 3;  // products per launch
+// The products of up to kTnBatch jobs over the same M rows in one launch: per-CTA
+// partials in `part` (tc_gemm_tn_part_elems of every job, added up), and the
+// jobs that sum them appended to `red`.
 size_t tc_gemm_tn_part_elems(int K1, int N);
-xmgn_status tc_gemm_tn(const Bf16Rows& X, const bf16* Y, int64_t ldy, int N, int64_t M, float* out,
-                       int kvalid, int nvalid, int nsplit, float* part, cudaStream_t s);
+xmgn_status tc_gemm_tn(const std::vector<TnJob>& jobs, int64_t M, float* part, std::vector<RedJob>& red,
+                       cudaStream_t s);
 
 int tc_grid(int64_t tiles);
 
