@@ -11,20 +11,24 @@
 // no padding in memory beyond that: TMA reads zeros past the last row and
 // column, so K, N and M are arbitrary.
 //
-// One persistent CTA per SM of 192 threads: warp 0 moves 64-deep slices of A
+// One persistent CTA per SM of 320 threads: warp 0 moves 64-deep slices of A
 // and B into a ring of four shared-memory stages with TMA (128-byte swizzle,
 // the layout tcgen05.mma reads), warp 1 issues the MMAs (one thread) into one
-// of two TMEM accumulators of 128 x BN fp32, warps 2-5 read the finished
-// accumulator (lane quadrant w % 4) and store it, so that one output tile's
-// stores overlap the next tile's products.  The epilogue writes each 128 x 32
-// fp32 chunk of the accumulator into one of two 16 KB shared-memory staging
-// buffers (128-byte swizzle, conflict-free) and one thread sends it out with a
-// TMA tensor store (a TMA reduce-add for the accumulating form), so global
-// memory sees whole 128-byte row segments.  The first-layer form
-// (wg_gemm_silu) applies bias and SiLU in the epilogue and stores bf16 blocks
-// of 64 columns (optionally also the fp32 pre-activation), so the fp32
-// product never goes to memory.  Every wait is bounded: a wait that gives up
-// flags the device error word and the roles wind down.
+// of two TMEM accumulators of 128 x BN fp32, warps 2-9 read the finished
+// accumulator (lane quadrant w % 4; warps 2-5 its first half of columns, 6-9
+// the second) and store it, so that one output tile's stores overlap the next
+// tile's products.  Each set of four writes a 128 x 32 fp32 chunk of the
+// accumulator into its 16 KB shared-memory staging buffer (128-byte swizzle,
+// conflict-free) and one thread sends it out with a TMA tensor store (a TMA
+// reduce-add for the accumulating form), so global memory sees whole 128-byte
+// row segments.  The first-layer form (wg_gemm_silu) applies bias and SiLU in
+// the epilogue and stores bf16 blocks of 64 columns (optionally also the fp32
+// pre-activation), so the fp32 product never goes to memory.  Two sets because
+// with four warps the epilogue of a K = 512 product is as long as the product
+// it hides behind (H = 512, 50k nodes: 16.56 -> 16.44 ms a
+// step).
+// Every wait is bounded: a wait that gives up flags the device error word and
+// the roles wind down.
 #include <cuda.h>
 
 #include "model.cuh"
@@ -37,7 +41,7 @@ using namespace tc;
 
 namespace {
 
-constexpr int kBM = 128, kBK = 64, kStages = 4, kWgThreads = 192;
+constexpr int kBM = 128, kBK = 64, kStages = 4, kWgThreads = 320;
 constexpr uint32_t kAStage = kBM * kBK * 2;  // 16 KB
 constexpr uint32_t kStage = kBM * 32 * 4;    // an output staging buffer: 128 rows x 32 fp32, 16 KB
 
@@ -98,15 +102,16 @@ __device__ __forceinline__ int64_t kblocks(const WgArgs& a, int sp, int64_t& kb0
   return e > kb0 ? e - kb0 : 0;
 }
 
-__device__ __forceinline__ void epi_sync() { asm volatile("bar.sync 1, 128;" ::: "memory"); }
-// AND of p over the 128 epilogue threads (also a barrier among them), so that
-// they leave the tile loop together.
-__device__ __forceinline__ bool epi_all(bool p) {
+// Barrier of one epilogue set's 128 threads.
+__device__ __forceinline__ void epi_sync(int set) { asm volatile("bar.sync %0, 128;" ::"r"(1 + set) : "memory"); }
+// AND of p over the 128 threads of an epilogue set (also a barrier among them),
+// so that they leave the tile loop together.
+__device__ __forceinline__ bool epi_all(int set, bool p) {
   uint32_t r;
   asm volatile(
-      "{\n\t.reg .pred q, o;\n\tsetp.ne.u32 q, %1, 0;\n\tbar.red.and.pred o, 1, 128, q;\n\tselp.u32 %0, 1, 0, o;\n\t}"
+      "{\n\t.reg .pred q, o;\n\tsetp.ne.u32 q, %1, 0;\n\tbar.red.and.pred o, %2, 128, q;\n\tselp.u32 %0, 1, 0, o;\n\t}"
       : "=r"(r)
-      : "r"(p ? 1u : 0u)
+      : "r"(p ? 1u : 0u), "r"(1 + set)
       : "memory");
   return r != 0;
 }
@@ -132,7 +137,7 @@ __global__ void __launch_bounds__(kWgThreads, 1) wg_kernel(WgArgs a, const __gri
     }
     for (int i = 0; i < 2; ++i) {
       mbar_init(&accf[i], 1);
-      mbar_init(&acce[i], 128);
+      mbar_init(&acce[i], 256);
     }
     quit = 0;
     fence_barrier_init();
@@ -190,7 +195,7 @@ __global__ void __launch_bounds__(kWgThreads, 1) wg_kernel(WgArgs a, const __gri
         int64_t kb0;
         const int64_t nk = kblocks(a, sp, kb0);
         const uint32_t acc = i & 1u;
-        // the epilogue has emptied this accumulator (its 128 arrivals complete one phase per use;
+        // the epilogue has emptied this accumulator (its 256 arrivals complete one phase per use;
         // the first use of each accumulator finds it free)
         if (i >= 2 && !wg_wait(&acce[acc], ((i >> 1) - 1) & 1u, a.err, &quit)) break;
         tc_fence_after();
@@ -214,102 +219,101 @@ __global__ void __launch_bounds__(kWgThreads, 1) wg_kernel(WgArgs a, const __gri
       }
     }
   } else {
-    // ------------------------------------------------------------ epilogue (warps 2..5)
+    // ------------------------------------------------------------ epilogue (warps 2..9)
     const int q = warp & 3;  // TMEM lane quadrant of this warp
     const int r = 32 * q + lane;
+    const int set = (warp - 2) >> 2;
     const uint32_t lane_base = uint32_t(32 * q) << 16;
-    const bool leader = tid == 64;
-    uint8_t* const stg = base + kStages * stage;  // two staging buffers
-    uint32_t i = 0, nchunk = 0;
+    const bool leader = tid == 64 || tid == 192;
+    uint8_t* const buf = base + kStages * stage + set * kStage;  // this set's staging buffer
+    // this set's columns of a tile: a half, or (64-wide tiles) all for the first set
+    const int c_begin = BN >= 128 ? set * (BN / 2) : (set ? BN : 0), c_end = BN >= 128 ? c_begin + BN / 2 : BN;
+    // the buffer is free once the store that last used it has read it; then written, then sent
+    auto send = [&](const CUtensorMap* map, int x, int y, auto&& fill, bool add) {
+      if (leader) bulk_wait_read0();
+      epi_sync(set);
+      fill();
+      fence_proxy_async();
+      epi_sync(set);
+      if (leader) {
+        if (add)
+          tma_reduce_add_2d(map, x, y, buf);
+        else
+          tma_store_2d(map, x, y, buf);
+        bulk_commit();
+      }
+    };
+    auto put32 = [&](const float (&v)[32]) {
+#pragma unroll
+      for (int j = 0; j < 8; ++j)
+        *reinterpret_cast<float4*>(buf + r * 128 + ((j ^ (r & 7)) << 4)) =
+            make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+    };
+    const bool bias4 = (reinterpret_cast<uintptr_t>(a.bias) & 15) == 0;  // parameter vectors may lie at any address
+    uint32_t i = 0;
     for (int64_t t = blockIdx.x; t < tiles; t += gridDim.x, ++i) {
       int tm, tn, sp;
       tile_of(a, t, tm, tn, sp);
       int64_t kb0;
       const int64_t nk = kblocks(a, sp, kb0);
       const uint32_t acc = i & 1u;
-      if (!epi_all(wg_wait(&accf[acc], (i >> 1) & 1u, a.err, &quit))) break;
-      tc_fence_after();
-      const uint32_t d = tacc + acc * uint32_t(BN) + lane_base;
       // output coordinates of the tile: NN/NT the rows and columns of D, TN the
       // tile's rows in the partial array (one 128 x BN block per split and tile)
       const int y0 = a.mode == WG_TN ? int(((int64_t(sp) * a.tiles_m + tm) * a.tiles_n + tn) * kBM) : tm * kBM;
       const int x0 = a.mode == WG_TN ? 0 : tn * BN;
+      const uint32_t d = tacc + acc * uint32_t(BN) + lane_base;
       if (a.silu) {  // 64-column blocks: A1 = bf16(SiLU(product + b1)), one TMA store each
-        for (int c = 0; c < BN; c += 64, ++nchunk) {
+        if (!epi_all(set, wg_wait(&accf[acc], (i >> 1) & 1u, a.err, &quit))) break;
+        tc_fence_after();
+        for (int c = c_begin; c < c_end; c += 64) {
           uint32_t h[32];
-#pragma unroll 1
+#pragma unroll
           for (int half = 0; half < 2; ++half) {
             float v[32];
-            tmem_ld32(d + c + 32 * half, v);
-            const int col = x0 + c + 32 * half;
+            const int cc = c + 32 * half, col = x0 + cc;
+            tmem_ld32(d + cc, v);
 #pragma unroll
-            for (int j = 0; j < 32; ++j) v[j] += col + j < a.N ? a.bias[col + j] : 0.f;
-            if (a.pre) {  // the pre-activation, 32 fp32 columns, through a staging buffer
-              uint8_t* const pb = stg + (nchunk & 1u) * kStage;
-              ++nchunk;
-              if (leader) bulk_wait_read1();
-              epi_sync();
+            for (int j = 0; j < 32; j += 4) {
+              if (bias4 && col + j + 4 <= a.N) {
+                const float4 b = *reinterpret_cast<const float4*>(a.bias + col + j);
+                v[j] += b.x, v[j + 1] += b.y, v[j + 2] += b.z, v[j + 3] += b.w;
+              } else {
 #pragma unroll
-              for (int j = 0; j < 8; ++j)
-                *reinterpret_cast<float4*>(pb + r * 128 + ((j ^ (r & 7)) << 4)) =
-                    make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
-              fence_proxy_async();
-              epi_sync();
-              if (leader) {
-                tma_store_2d(&tp, col, y0, pb);
-                bulk_commit();
+                for (int u = 0; u < 4; ++u) v[j + u] += col + j + u < a.N ? a.bias[col + j + u] : 0.f;
               }
             }
+            if (a.pre)  // the pre-activation, 32 fp32 columns
+              send(&tp, col, y0, [&] { put32(v); }, false);
 #pragma unroll
             for (int j = 0; j < 32; j += 2) h[16 * half + j / 2] = pack_bf16(silu_fast(v[j]), silu_fast(v[j + 1]));
           }
-          uint8_t* const buf = stg + (nchunk & 1u) * kStage;
-          if (leader) bulk_wait_read1();  // the store that last used this buffer has read it
-          epi_sync();
+          send(&td, x0 + c, y0, [&] {
 #pragma unroll
-          for (int j = 0; j < 8; ++j)
-            *reinterpret_cast<uint4*>(buf + r * 128 + ((j ^ (r & 7)) << 4)) =
-                make_uint4(h[4 * j], h[4 * j + 1], h[4 * j + 2], h[4 * j + 3]);
-          fence_proxy_async();
-          epi_sync();
-          if (leader) {
-            tma_store_2d(&td, x0 + c, y0, buf);
-            bulk_commit();
-          }
+            for (int j = 0; j < 8; ++j)
+              *reinterpret_cast<uint4*>(buf + r * 128 + ((j ^ (r & 7)) << 4)) =
+                  make_uint4(h[4 * j], h[4 * j + 1], h[4 * j + 2], h[4 * j + 3]);
+          }, false);
         }
         tc_fence_before();
         mbar_arrive(&acce[acc]);
         continue;
       }
-      for (int c = 0; c < BN; c += 32, ++nchunk) {
+      if (!epi_all(set, wg_wait(&accf[acc], (i >> 1) & 1u, a.err, &quit))) break;
+      tc_fence_after();
+      for (int c = c_begin; c < c_end; c += 32) {
         float v[32];
         tmem_ld32(d + c, v);
         if (nk == 0) {
 #pragma unroll
           for (int j = 0; j < 32; ++j) v[j] = 0.f;
         }
-        uint8_t* const buf = stg + (nchunk & 1u) * kStage;
-        if (leader) bulk_wait_read1();  // the store that last used this buffer has read it
-        epi_sync();
-#pragma unroll
-        for (int j = 0; j < 8; ++j)
-          *reinterpret_cast<float4*>(buf + r * 128 + ((j ^ (r & 7)) << 4)) =
-              make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
-        fence_proxy_async();
-        epi_sync();
-        if (leader) {
-          if (a.accum)
-            tma_reduce_add_2d(&td, x0 + c, y0, buf);
-          else
-            tma_store_2d(&td, x0 + c, y0, buf);
-          bulk_commit();
-        }
+        send(&td, x0 + c, y0, [&] { put32(v); }, a.accum != 0);
       }
       tc_fence_before();
       mbar_arrive(&acce[acc]);
     }
   }
-  if (tid == 64) bulk_wait0();  // every output store is complete
+  if (tid == 64 || tid == 192) bulk_wait0();  // every output store is complete
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -390,7 +394,7 @@ namespace {
 
 int tile_width(int N) { return N > 128 ? 256 : (N > 64 ? 128 : 64); }
 
-uint32_t smem_of(int BN) { return kStages * (kAStage + uint32_t(BN) * kBK * 2u) + 2u * kStage + 1024u; }
+uint32_t smem_of(int BN) { return kStages * (kAStage + uint32_t(BN) * kBK * 2u) + 2u * kStage + 1024u; }  // a staging buffer per epilogue set
 
 xmgn_status launch(WgArgs& a, const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap& td, cudaStream_t s,
                    const CUtensorMap* tp = nullptr) {
