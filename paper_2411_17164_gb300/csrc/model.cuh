@@ -144,13 +144,14 @@ xmgn_status layernorm_fwd_agg_f32(const float* Z, const float* bias, const int64
                                   const float* gamma, const float* beta, const float* resid_in, float* resid_out,
                                   float* agg, cudaStream_t s);
 // LayerNorm backward at the input Z + bias (bias optional).
-// dY(r) = dY1[r] + (dY2 ? dY2[idx2[r]] : 0); dZ = LN'(Z + bias)^T dY; dgamma,
-// dbeta written (deterministic for a given device).
+// dY(r) = dY1[r] + (dY2 ? dY2[idx2[r]] : 0); dZ = LN'(Z + bias)^T dY, in fp32
+// (dZ) and / or rounded to bf16 (dZ16); dgamma, dbeta and db = the column sums
+// of dZ written (deterministic for a given device).
 size_t ln_bwd_part_elems(int N);
 xmgn_status layernorm_bwd_f32(const float* Z, int64_t M, int N, const float* gamma,
                               const float* dY1, const float* dY2, const int32_t* idx2, float* dZ,
-                              float* dgamma, float* dbeta, float* part, cudaStream_t s,
-                              const float* bias = nullptr);
+                              __nv_bfloat16* dZ16, float* dgamma, float* dbeta, float* db, float* part,
+                              cudaStream_t s, const float* bias = nullptr);
 
 // out[i] (+)= sum_{e in row i} v[e]            (receiver segments, CSR order)
 xmgn_status seg_sum_rows_f32(const float* v, int64_t ldv, const int64_t* row_ptr, int64_t n, int H,

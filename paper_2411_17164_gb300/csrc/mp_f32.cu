@@ -147,16 +147,15 @@ xmgn_status mlp_bwd_wide(const WideScratch& x, const MlpOff& o, const float* P, 
   XMGN_TRY(wide_round(P + o.W2, H, o.out, o.out, x.w2, s));
   XMGN_TRY(wide_gather(X, M, x.x, s));
   XMGN_TRY(wide_nn_silu(x.x, M, K, x.w1, H, P + o.b1, x.a1, s, w.Z1));  // A1 and the pre-activation Z1
-  const float* dZ2 = dY1;
-  if (o.ln) {
+  if (o.ln) {  // dZ2 leaves in bf16, its column sums with it
     XMGN_TRY(wide_nn(x.a1, M, H, x.w2, o.out, x.acc, s));
-    XMGN_TRY(layernorm_bwd_f32(x.acc, M, o.out, P + o.g, dY1, dY2, idx2, w.dZ2, g + o.g, g + o.be, w.lnpart, s,
-                               P + o.b2));
-    dZ2 = w.dZ2;
+    XMGN_TRY(layernorm_bwd_f32(x.acc, M, o.out, P + o.g, dY1, dY2, idx2, nullptr, x.dz2, g + o.g, g + o.be, g + o.b2,
+                               w.lnpart, s, P + o.b2));
+  } else {
+    XMGN_TRY(wide_round(dY1, M, o.out, o.out, x.dz2, s));
+    XMGN_TRY(colsum_f32(dY1, M, o.out, o.out, g + o.b2, w.cspart, s));
   }
-  XMGN_TRY(wide_round(dZ2, M, o.out, o.out, x.dz2, s));
   XMGN_TRY(wide_tn(x.a1, M, H, x.dz2, o.out, g + o.W2, x.part, s));
-  XMGN_TRY(colsum_f32(dZ2, M, o.out, o.out, g + o.b2, w.cspart, s));
   XMGN_TRY(wide_nt(x.dz2, M, o.out, x.w2, H, x.acc, s));
   XMGN_TRY(wide_silu_grad_colsum(x.acc, M, H, w.Z1, x.dz1, g + o.b1, w.cspart, s));
   return wide_tn(x.x, M, K, x.dz1, H, g + o.W1, x.part, s);
@@ -178,12 +177,13 @@ xmgn_status mlp_bwd(const Gemm& gm, const MlpOff& o, const float* P, const RowSr
   if (o.ln) {
     XMGN_TRY(gemm_nn_f32(rows1(w.A1, H, H), M, P + o.W2, o.out, P + o.b2, w.Z2, o.out, EPI_STORE, nullptr, nullptr,
                          s));
-    XMGN_TRY(layernorm_bwd_f32(w.Z2, M, o.out, P + o.g, dY1, dY2, idx2, w.dZ2, g + o.g, g + o.be,
+    XMGN_TRY(layernorm_bwd_f32(w.Z2, M, o.out, P + o.g, dY1, dY2, idx2, w.dZ2, nullptr, g + o.g, g + o.be, g + o.b2,
                                w.lnpart, s));
     dZ2 = w.dZ2;
+  } else {
+    XMGN_TRY(colsum_f32(dY1, M, o.out, o.out, g + o.b2, w.cspart, s));
   }
   XMGN_TRY(gemm_tn_f32(rows1(w.A1, H, H), M, dZ2, o.out, o.out, g + o.W2, w.tnpart, s));
-  XMGN_TRY(colsum_f32(dZ2, M, o.out, o.out, g + o.b2, w.cspart, s));
   XMGN_TRY(gemm_nt_f32(rows1(dZ2, o.out, o.out), M, P + o.W2, H, w.dZ1, H, EPI_SILU_GRAD, w.Z1, s));
   XMGN_TRY(gemm_tn_f32(X, M, w.dZ1, H, H, g + w1, w.tnpart, s));
   if (!add.p) XMGN_TRY(colsum_f32(w.dZ1, M, H, H, g + o.b1, w.cspart, s));
