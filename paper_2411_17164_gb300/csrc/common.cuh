@@ -2,6 +2,8 @@
 // helpers).  Everything here is internal; the public surface is include/xmgn.h.
 #pragma once
 
+#include <utility>
+
 #include <cuda_runtime.h>
 #include <stdint.h>
 #include <stdio.h>
@@ -121,7 +123,8 @@ __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;"
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 template <class... P, class... A>
-inline void launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A&&... args) {
+inline void launch_pdl_if(bool early, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                          A&&... args) {
   cudaLaunchAttribute at{};
   at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at.val.programmaticStreamSerializationAllowed = 1;
@@ -131,9 +134,19 @@ inline void launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem,
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
   cfg.attrs = &at;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = early ? 1 : 0;
   cudaLaunchKernelEx(&cfg, kernel, P(args)...);  // errors: the XMGN_LAUNCH_CHECK that follows
 }
+template <class... P, class... A>
+inline void launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A&&... args) {
+  launch_pdl_if(true, kernel, grid, block, smem, s, std::forward<A>(args)...);
+}
+// Row kernels (LayerNorm, operand rounding, SiLU', segment sums) begin early only
+// while their rows are this few bytes: over more, each takes 100 us and up and an
+// early start costs more than the 2 us it saves (H = 512, 50k nodes, 725 MB a
+// pass: 14.95 ms a step without, 15.55 with; H = 256, 30k nodes, 217 MB: 1.71
+// without, 1.68 with).
+inline bool rows_early(int64_t rows, int cols) { return rows * cols * 4 <= (int64_t(256) << 20); }
 
 // ---------------------------------------------------------------- device helpers
 __device__ __forceinline__ void dev_flag(uint32_t* err, uint32_t code) {

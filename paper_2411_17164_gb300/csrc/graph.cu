@@ -30,6 +30,8 @@ constexpr int kMaxK = 32;
 __global__ void quantize_kernel(const float* __restrict__ xyz, int64_t n, float scale,
                                 int32_t* __restrict__ q, int32_t* __restrict__ bbox,
                                 uint32_t* err) {
+  pdl_wait();
+  pdl_trigger();
   int lo[3] = {INT32_MAX, INT32_MAX, INT32_MAX}, hi[3] = {INT32_MIN, INT32_MIN, INT32_MIN};
   for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n;
        i += int64_t(gridDim.x) * blockDim.x) {
@@ -66,6 +68,8 @@ __global__ void quantize_kernel(const float* __restrict__ xyz, int64_t n, float 
 }
 
 __global__ void bbox_init_kernel(int32_t* bbox) {
+  pdl_wait();
+  pdl_trigger();
   if (threadIdx.x < 3) {
     bbox[threadIdx.x] = INT32_MAX;
     bbox[3 + threadIdx.x] = INT32_MIN;
@@ -100,6 +104,8 @@ __host__ __device__ inline int64_t cell_budget(int64_t n) {
 // The grid of every level (thread l: the first sizes.n[l] points) over the box
 // of all points: at most cell_budget cells.
 __global__ void grid_layout_kernel(const int32_t* __restrict__ bbox, LevelSizes sizes, int levels, Grid* __restrict__ out) {
+  pdl_wait();
+  pdl_trigger();
   const int l = threadIdx.x;
   if (l >= levels) return;
   const int64_t budget = cell_budget(sizes.n[l]);
@@ -131,6 +137,8 @@ __device__ __forceinline__ int cell_coord(int32_t q, int32_t lo, int32_t c) { re
 // Cell of every reference point, and its place among the cell's points.
 __global__ void cell_count_kernel(const int32_t* __restrict__ q, int64_t n, const Grid* __restrict__ grid,
                                   int32_t* __restrict__ cell_of, int32_t* __restrict__ at, int32_t* __restrict__ cnt) {
+  pdl_wait();
+  pdl_trigger();
   const Grid G = *grid;
   for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n;
        i += int64_t(gridDim.x) * blockDim.x) {
@@ -146,6 +154,8 @@ __global__ void cell_count_kernel(const int32_t* __restrict__ q, int64_t n, cons
 __global__ void cell_scatter_kernel(const int32_t* __restrict__ q, const int32_t* __restrict__ cell_of,
                                     const int32_t* __restrict__ at, int64_t n, const int32_t* __restrict__ start,
                                     int4* __restrict__ pts) {
+  pdl_wait();
+  pdl_trigger();
   for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n;
        i += int64_t(gridDim.x) * blockDim.x)
     pts[start[cell_of[i]] + at[i]] = make_int4(q[3 * i], q[3 * i + 1], q[3 * i + 2], int32_t(i));
@@ -211,6 +221,8 @@ __global__ void __launch_bounds__(128) knn_kernel(const int32_t* __restrict__ q,
                                                   const Grid* __restrict__ grid, int32_t* __restrict__ nbr,
                                                   int64_t stride, int off, int32_t* __restrict__ rcnt,
                                                   int32_t* __restrict__ rank) {
+  pdl_wait();
+  pdl_trigger();
   const Grid gr = *grid;
   const int lane = threadIdx.x & 31, gl = lane % G;
   const uint32_t mask = G == 1 ? 0u : ((G == 32 ? 0xffffffffu : ((1u << G) - 1u)) << (lane - gl));
@@ -313,15 +325,15 @@ void knn_launch_g(unsigned grid, cudaStream_t s, const int32_t* q, const int4* p
                   int64_t q1, int k, const Grid* gr, int32_t* nbr, int64_t stride, int off, int32_t* rcnt,
                   int32_t* rank) {
   if (k <= 3)
-    knn_kernel<3, G, QUERY><<<grid, 128, 0, s>>>(q, pts, start, q0, q1, k, gr, nbr, stride, off, rcnt, rank);
+    launch_pdl(knn_kernel<3, G, QUERY>, grid, 128, 0, s, q, pts, start, q0, q1, k, gr, nbr, stride, off, rcnt, rank);
   else if (k <= 6)
-    knn_kernel<6, G, QUERY><<<grid, 128, 0, s>>>(q, pts, start, q0, q1, k, gr, nbr, stride, off, rcnt, rank);
+    launch_pdl(knn_kernel<6, G, QUERY>, grid, 128, 0, s, q, pts, start, q0, q1, k, gr, nbr, stride, off, rcnt, rank);
   else if (k <= 8)
-    knn_kernel<8, G, QUERY><<<grid, 128, 0, s>>>(q, pts, start, q0, q1, k, gr, nbr, stride, off, rcnt, rank);
+    launch_pdl(knn_kernel<8, G, QUERY>, grid, 128, 0, s, q, pts, start, q0, q1, k, gr, nbr, stride, off, rcnt, rank);
   else if (k <= 16)
-    knn_kernel<16, G, QUERY><<<grid, 128, 0, s>>>(q, pts, start, q0, q1, k, gr, nbr, stride, off, rcnt, rank);
+    launch_pdl(knn_kernel<16, G, QUERY>, grid, 128, 0, s, q, pts, start, q0, q1, k, gr, nbr, stride, off, rcnt, rank);
   else
-    knn_kernel<kMaxK, G, QUERY><<<grid, 128, 0, s>>>(q, pts, start, q0, q1, k, gr, nbr, stride, off, rcnt, rank);
+    launch_pdl(knn_kernel<kMaxK, G, QUERY>, grid, 128, 0, s, q, pts, start, q0, q1, k, gr, nbr, stride, off, rcnt, rank);
 }
 
 // Lanes per point: eight while that still leaves at most one wave of resident
@@ -347,6 +359,8 @@ xmgn_status knn_launch(const int32_t* q, const int4* pts, const int32_t* start, 
 // of j's list.
 __global__ void sym_rev_kernel(const int32_t* __restrict__ nbr, int64_t n, int k, const int64_t* __restrict__ rstart,
                                const int32_t* __restrict__ rank, int32_t* __restrict__ rev) {
+  pdl_wait();
+  pdl_trigger();
   for (int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; t < n * k;
        t += int64_t(gridDim.x) * blockDim.x) {
     const int32_t j = nbr[t];
@@ -368,6 +382,8 @@ __global__ void __launch_bounds__(256) sym_sort_kernel(const int32_t* __restrict
                                                        const int64_t* __restrict__ rstart,
                                                        const int32_t* __restrict__ rev, int32_t* __restrict__ out,
                                                        int32_t* __restrict__ deg) {
+  pdl_wait();
+  pdl_trigger();
   __shared__ __align__(16) int32_t raw[16][kRow], srt[16][kRow];
   const int lane = threadIdx.x & 31, l = lane & 15, gi = threadIdx.x >> 4, hs = lane & 16;
   constexpr uint32_t kAll = 0xffffffffu;
@@ -458,6 +474,8 @@ __global__ void sym_emit_kernel(const int32_t* __restrict__ rows, const int64_t*
                                 const int64_t* __restrict__ row_ptr, int64_t n, int64_t cap,
                                 int32_t* __restrict__ col, int32_t* __restrict__ recv,
                                 const uint32_t* __restrict__ err, int64_t* __restrict__ info) {
+  pdl_wait();
+  pdl_trigger();
   if (blockIdx.x == 0 && threadIdx.x == 0) {  // what the host reads at the end, in one copy
     info[0] = row_ptr[n];
     info[1] = int64_t(*err);
@@ -479,9 +497,9 @@ __global__ void sym_emit_kernel(const int32_t* __restrict__ rows, const int64_t*
 
 xmgn_status quantize_launch(const float* xyz, int64_t n, double scale, int32_t* q, int32_t* bbox,
                             uint32_t* err, cudaStream_t s) {
-  bbox_init_kernel<<<1, 32, 0, s>>>(bbox);
+  launch_pdl(bbox_init_kernel, 1, 32, 0, s, bbox);
   XMGN_LAUNCH_CHECK();
-  quantize_kernel<<<grid_for(n, 256, int64_t(num_sms()) * 8), 256, 0, s>>>(xyz, n, float(scale), q, bbox, err);
+  launch_pdl(quantize_kernel, grid_for(n, 256, int64_t(num_sms()) * 8), 256, 0, s, xyz, n, float(scale), q, bbox, err);
   XMGN_LAUNCH_CHECK();
   return XMGN_OK;
 }
@@ -499,6 +517,8 @@ __global__ void __launch_bounds__(256) csc_perm_kernel(const int64_t* __restrict
                                                        const int32_t* __restrict__ recv,
                                                        const int32_t* __restrict__ key, int64_t n, int64_t e,
                                                        int64_t cap, int32_t* __restrict__ perm, uint32_t* err) {
+  pdl_wait();
+  pdl_trigger();
   if (e < 0) {
     e = row_ptr[n];
     if (e > cap) return;
@@ -586,7 +606,7 @@ static void knn_layout(int64_t N, int32_t K, Arena& A, KnnWs& w) {
 static xmgn_status quantize_all(const float* xyz, int64_t N, double scale, const LevelSizes& sizes, int levels,
                                 KnnWs& w, uint32_t* err, cudaStream_t s) {
   XMGN_TRY(quantize_launch(xyz, N, scale, w.q, w.bbox, err, s));
-  grid_layout_kernel<<<1, 32, 0, s>>>(w.bbox, sizes, levels, w.grid);
+  launch_pdl(grid_layout_kernel, 1, 32, 0, s, w.bbox, sizes, levels, w.grid);
   XMGN_LAUNCH_CHECK();
   XMGN_CUDA(cudaMemsetAsync(w.rcnt, 0, sizeof(int32_t) * size_t(N), s));
   return XMGN_OK;
@@ -596,10 +616,10 @@ static xmgn_status quantize_all(const float* xyz, int64_t N, double scale, const
 static xmgn_status grid_sort(int64_t n_ref, const Grid* grid, KnnWs& w, cudaStream_t s) {
   const int64_t cells = cell_budget(n_ref);
   XMGN_CUDA(cudaMemsetAsync(w.cnt, 0, sizeof(int32_t) * size_t(cells), s));
-  cell_count_kernel<<<grid_for(n_ref, 256), 256, 0, s>>>(w.q, n_ref, grid, w.cell_of, w.at, w.cnt);
+  launch_pdl(cell_count_kernel, grid_for(n_ref, 256), 256, 0, s, w.q, n_ref, grid, w.cell_of, w.at, w.cnt);
   XMGN_LAUNCH_CHECK();
   XMGN_TRY(exclusive_scan_i32(w.cnt, w.cstart, cells, w.scan_tmp, s));
-  cell_scatter_kernel<<<grid_for(n_ref, 256), 256, 0, s>>>(w.q, w.cell_of, w.at, n_ref, w.cstart, w.pts);
+  launch_pdl(cell_scatter_kernel, grid_for(n_ref, 256), 256, 0, s, w.q, w.cell_of, w.at, n_ref, w.cstart, w.pts);
   XMGN_LAUNCH_CHECK();
   return XMGN_OK;
 }
@@ -611,16 +631,16 @@ static xmgn_status symmetrise_slots(int64_t N, int32_t K, KnnWs& w, int64_t* row
                                     int32_t* recv, int32_t* csc_perm, int64_t E_cap, int64_t* E_out,
                                     uint32_t* err, cudaStream_t s) {
   XMGN_TRY(exclusive_scan_i32(w.rcnt, w.rstart, N, w.scan_tmp, s));
-  sym_rev_kernel<<<grid_for(N * K, 256), 256, 0, s>>>(w.nbr, N, K, w.rstart, w.rank, w.rev);
+  launch_pdl(sym_rev_kernel, grid_for(N * K, 256), 256, 0, s, w.nbr, N, K, w.rstart, w.rank, w.rev);
   XMGN_LAUNCH_CHECK();
-  sym_sort_kernel<<<grid_for(N * 16, 256), 256, 0, s>>>(w.nbr, N, K, w.rstart, w.rev, w.rows, w.deg);
+  launch_pdl(sym_sort_kernel, grid_for(N * 16, 256), 256, 0, s, w.nbr, N, K, w.rstart, w.rev, w.rows, w.deg);
   XMGN_LAUNCH_CHECK();
   XMGN_TRY(exclusive_scan_i32(w.deg, row_ptr, N, w.scan_tmp, s));
-  sym_emit_kernel<<<grid_for(N * 8, 256), 256, 0, s>>>(w.rows, w.rstart, K, row_ptr, N, E_cap, col, recv, err, w.info);
+  launch_pdl(sym_emit_kernel, grid_for(N * 8, 256), 256, 0, s, w.rows, w.rstart, K, row_ptr, N, E_cap, col, recv, err, w.info);
   XMGN_LAUNCH_CHECK();
   if (csc_perm) {
     const int64_t most = 2 * N * K < E_cap ? 2 * N * K : E_cap;
-    csc_perm_kernel<<<grid_for((most + kPermEdges - 1) / kPermEdges, 256), 256, 0, s>>>(row_ptr, col, recv, nullptr, N,
+    launch_pdl(csc_perm_kernel, grid_for((most + kPermEdges - 1) / kPermEdges, 256), 256, 0, s, row_ptr, col, recv, nullptr, N,
                                                                                         -1, E_cap, csc_perm, err);
     XMGN_LAUNCH_CHECK();
   }

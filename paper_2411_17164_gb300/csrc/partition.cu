@@ -61,6 +61,8 @@ struct RcbState {
 
 __global__ void rcb_begin_kernel(const int32_t* __restrict__ ext, const RcbSeg* __restrict__ plan, int nseg,
                                  RcbState* __restrict__ st, int32_t* __restrict__ next_ext, int nnext) {
+  pdl_wait();
+  pdl_trigger();
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nnext; i += gridDim.x * blockDim.x)
     for (int a = 0; a < 3; ++a) {
       next_ext[6 * i + a] = INT32_MAX;
@@ -89,6 +91,8 @@ __global__ void __launch_bounds__(1024) rcb_hist_kernel(const int32_t* __restric
                                                         const int32_t* __restrict__ q,
                                                         const RcbState* __restrict__ st, int nseg, int on_id,
                                                         int shift, int bits, uint32_t* __restrict__ hist) {
+  pdl_wait();
+  pdl_trigger();
   extern __shared__ uint32_t sh[];
   const int nb = 1 << bits;
   if (SMEM) {
@@ -127,6 +131,8 @@ __global__ void __launch_bounds__(1024) rcb_hist_kernel(const int32_t* __restric
 // digit.  Leaves the histogram zeroed for the next pass.
 __global__ void __launch_bounds__(256) rcb_find_kernel(RcbState* __restrict__ st, int on_id, int shift, int bits,
                                                        uint32_t* __restrict__ hist) {
+  pdl_wait();
+  pdl_trigger();
   __shared__ uint32_t wsum[8];
   const int s = blockIdx.x, tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   const RcbState t = st[s];
@@ -172,6 +178,8 @@ __global__ void __launch_bounds__(512) rcb_split_kernel(int32_t* __restrict__ se
                                                         const RcbSeg* __restrict__ plan, int nnext,
                                                         int32_t* __restrict__ ext, const int32_t* __restrict__ base,
                                                         int32_t* __restrict__ part) {
+  pdl_wait();
+  pdl_trigger();
   __shared__ int32_t sx[256 * 6];
   const bool sm = !part && nnext <= 256;
   if (sm) {
@@ -236,6 +244,8 @@ __device__ __forceinline__ uint64_t mkey(uint32_t p, uint32_t hop, uint32_t v) {
 // this warp alone writes (no atomics).
 __global__ void bfs_seed_kernel(const int32_t* __restrict__ part, int64_t n, int P, uint32_t* __restrict__ bits,
                                 int64_t words, int32_t* __restrict__ map, uint32_t* err) {
+  pdl_wait();
+  pdl_trigger();
   const int64_t n32 = (n + 31) & ~int64_t(31);
   for (int64_t v = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; v < n32; v += int64_t(gridDim.x) * blockDim.x) {
     int p = v < n ? part[v] : -1;
@@ -307,6 +317,8 @@ __global__ void __launch_bounds__(256) bfs_first_kernel(const int64_t* __restric
                                                         int32_t* __restrict__ map, uint64_t* __restrict__ list,
                                                         unsigned long long* __restrict__ cnt, int64_t cap,
                                                         uint32_t* err) {
+  pdl_wait();
+  pdl_trigger();
   __shared__ uint64_t found[kFound];
   __shared__ int nfound;
   __shared__ unsigned long long pos0;
@@ -343,6 +355,8 @@ __global__ void __launch_bounds__(256) bfs_round_kernel(const int64_t* __restric
                                                         int32_t* __restrict__ map, uint64_t* __restrict__ list,
                                                         unsigned long long* __restrict__ cnt, int h, int64_t cap,
                                                         uint32_t* err) {
+  pdl_wait();
+  pdl_trigger();
   __shared__ uint64_t found[kFound];
   __shared__ int nfound;
   __shared__ unsigned long long pos0;
@@ -407,6 +421,8 @@ __device__ __forceinline__ void count_hops(const uint32_t* __restrict__ bits, co
 __global__ void __launch_bounds__(256) hop_count_kernel(const uint32_t* __restrict__ bits,
                                                         const int32_t* __restrict__ map, int64_t words, int64_t n,
                                                         int L, int32_t* __restrict__ cnt) {
+  pdl_wait();
+  pdl_trigger();
   __shared__ uint32_t hist[8][256];
   uint32_t word;
   count_hops(bits, map, words, n, L, hist, word);
@@ -426,6 +442,8 @@ __global__ void __launch_bounds__(256) hop_place_kernel(const uint32_t* __restri
                                                         const int64_t* __restrict__ base,
                                                         uint64_t* __restrict__ members, int32_t* __restrict__ gid,
                                                         uint8_t* __restrict__ hops) {
+  pdl_wait();
+  pdl_trigger();
   __shared__ uint32_t hist[8][256];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int64_t p = blockIdx.y, w0 = int64_t(blockIdx.x) * 256 + 32 * w;
@@ -468,6 +486,8 @@ __global__ void __launch_bounds__(256) hop_place_kernel(const uint32_t* __restri
 // info = [members, error word, node_ptr of every part, inner nodes of every part]
 __global__ void part_sizes_kernel(const int64_t* __restrict__ base, int64_t nblk, int P, int L,
                                   const uint32_t* __restrict__ err, int64_t* __restrict__ info) {
+  pdl_wait();
+  pdl_trigger();
   const int64_t row = int64_t(L + 1) * nblk;
   for (int p = blockIdx.x * blockDim.x + threadIdx.x; p <= P; p += gridDim.x * blockDim.x) {
     info[2 + p] = base[p * row];
@@ -481,12 +501,16 @@ __global__ void part_sizes_kernel(const int64_t* __restrict__ base, int64_t nblk
 
 __global__ void part_edges_kernel(const int64_t* __restrict__ brp, const int64_t* __restrict__ node_ptr, int P,
                                   int64_t* __restrict__ edge_ptr) {
+  pdl_wait();
+  pdl_trigger();
   for (int p = blockIdx.x * blockDim.x + threadIdx.x; p <= P; p += gridDim.x * blockDim.x)
     edge_ptr[p] = brp[node_ptr[p]];
 }
 
 __global__ void batch_ids_kernel(const uint64_t* __restrict__ members, int64_t nb, int32_t* __restrict__ gid,
                                  uint8_t* __restrict__ hop) {
+  pdl_wait();
+  pdl_trigger();
   for (int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; t < nb; t += int64_t(gridDim.x) * blockDim.x) {
     const uint64_t key = members[t];
     gid[t] = int32_t(uint32_t(key));
@@ -510,6 +534,8 @@ __global__ void batch_deg_kernel(const uint64_t* __restrict__ members, int64_t n
                                  const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
                                  const uint32_t* __restrict__ bits, int64_t words, int32_t* __restrict__ deg,
                                  uint32_t* err) {
+  pdl_wait();
+  pdl_trigger();
   for (int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; t < nb; t += int64_t(gridDim.x) * blockDim.x) {
     const uint64_t key = members[t];
     const uint32_t v = uint32_t(key);
@@ -534,6 +560,8 @@ __global__ void __launch_bounds__(256) batch_edges_kernel(const uint64_t* __rest
                                                           const uint32_t* __restrict__ bits, int64_t words, int L,
                                                           const int64_t* __restrict__ brp, int32_t* __restrict__ bcol,
                                                           int32_t* __restrict__ brecv, uint32_t* err) {
+  pdl_wait();
+  pdl_trigger();
   constexpr int U = 2;
   const int lane = threadIdx.x & 31, sub = lane >> 3, l = lane & 7;
   const int64_t warp = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
@@ -723,7 +751,7 @@ xmgn_status bisect(const float* xyz, int64_t N, double scale, int32_t P, PartLay
     const RcbSeg* pl = w.plan + level[l];
     const int32_t* ext = l ? w.ext[l & 1] : w.bbox;
     const bool last = l + 1 == nl;
-    rcb_begin_kernel<<<grid_for(nnext, 256), 256, 0, s>>>(ext, pl, nseg, w.state, w.ext[(l + 1) & 1], nnext);
+    launch_pdl(rcb_begin_kernel, grid_for(nnext, 256), 256, 0, s, ext, pl, nseg, w.state, w.ext[(l + 1) & 1], nnext);
     XMGN_LAUNCH_CHECK();
     for (const Digit& d : digits) {
       const int words = nseg << d.bits;
@@ -731,16 +759,16 @@ xmgn_status bisect(const float* xyz, int64_t N, double scale, int32_t P, PartLay
       // one histogram per block in shared memory while all segments' fit; with more segments the
       // atomics spread over that many more addresses and go to memory
       if (words <= kHistSmem)
-        rcb_hist_kernel<true><<<grid_for(N, 1024, int64_t(num_sms()) * 2), 1024, size_t(words) * 4, s>>>(
+        launch_pdl(rcb_hist_kernel<true>, grid_for(N, 1024, int64_t(num_sms()) * 2), 1024, size_t(words) * 4, s, 
             seg, N, w.q, w.state, nseg, d.on_id, d.shift, d.bits, w.hist);
       else
-        rcb_hist_kernel<false><<<grid_for(N, 1024, int64_t(num_sms()) * 2), 1024, 0, s>>>(
+        launch_pdl(rcb_hist_kernel<false>, grid_for(N, 1024, int64_t(num_sms()) * 2), 1024, 0, s, 
             seg, N, w.q, w.state, nseg, d.on_id, d.shift, d.bits, w.hist);
       XMGN_LAUNCH_CHECK();
-      rcb_find_kernel<<<unsigned(nseg), 256, 0, s>>>(w.state, d.on_id, d.shift, d.bits, w.hist);
+      launch_pdl(rcb_find_kernel, unsigned(nseg), 256, 0, s, w.state, d.on_id, d.shift, d.bits, w.hist);
       XMGN_LAUNCH_CHECK();
     }
-    rcb_split_kernel<<<grid_for(N, 512, int64_t(num_sms()) * 4), 512, 0, s>>>(
+    launch_pdl(rcb_split_kernel, grid_for(N, 512, int64_t(num_sms()) * 4), 512, 0, s, 
         w.seg, l == 0 ? 1 : 0, N, w.q, w.state, pl, nnext, w.ext[(l + 1) & 1], w.base, last ? part : nullptr);
     XMGN_LAUNCH_CHECK();
   }
@@ -788,12 +816,12 @@ xmgn_status partition_halo(const int64_t* row_ptr, const int32_t* col, int64_t N
   // edges and the CSC permutation, once ids and row offsets are in place
   auto emit_edges = [&](int64_t nb, int64_t eb) -> xmgn_status {
     if (nb > 0) {
-      batch_edges_kernel<<<grid_for(nb * 4, 256), 256, 0, s>>>(w.members, nb, N, row_ptr, col, w.map, w.bits, words, L,
+      launch_pdl(batch_edges_kernel, grid_for(nb * 4, 256), 256, 0, s, w.members, nb, N, row_ptr, col, w.map, w.bits, words, L,
                                                                b_row_ptr, b_col, b_recv, err);
       XMGN_LAUNCH_CHECK();
     }
     if (b_csc_perm && eb > 0) {
-      csc_perm_kernel<<<grid_for((eb + 3) / 4, 256), 256, 0, s>>>(b_row_ptr, b_col, b_recv, gid, nb, eb, eb, b_csc_perm, err);
+      launch_pdl(csc_perm_kernel, grid_for((eb + 3) / 4, 256), 256, 0, s, b_row_ptr, b_col, b_recv, gid, nb, eb, eb, b_csc_perm, err);
       XMGN_LAUNCH_CHECK();
     }
     XMGN_CUDA(cudaMemsetAsync(w.stamp, 0, sizeof(int64_t) * 8, s));  // one emit per sizing pass
@@ -812,7 +840,7 @@ xmgn_status partition_halo(const int64_t* row_ptr, const int32_t* col, int64_t N
     if (cap_nodes < nb) return fail(XMGN_ERR_WORKSPACE, "cap_nodes %lld < %lld", (long long)cap_nodes, (long long)nb);
     if (cap_edges < eb) return fail(XMGN_ERR_WORKSPACE, "cap_edges %lld < %lld", (long long)cap_edges, (long long)eb);
     if (nb > 0) {  // the sizing pass left members, map, mask and row offsets
-      batch_ids_kernel<<<grid_for(nb, 256), 256, 0, s>>>(w.members, nb, gid, hop);
+      launch_pdl(batch_ids_kernel, grid_for(nb, 256), 256, 0, s, w.members, nb, gid, hop);
       XMGN_LAUNCH_CHECK();
     }
     XMGN_CUDA(cudaMemcpyAsync(b_row_ptr, w.brp, sizeof(int64_t) * size_t(nb + 1), cudaMemcpyDeviceToDevice, s));
@@ -831,15 +859,15 @@ xmgn_status partition_halo(const int64_t* row_ptr, const int32_t* col, int64_t N
   // ---------------- halo BFS
   XMGN_CUDA(cudaMemsetAsync(w.bits, 0, sizeof(uint32_t) * size_t(int64_t(P) * words), s));
   XMGN_CUDA(cudaMemsetAsync(w.counters, 0, sizeof(unsigned long long) * 260, s));
-  bfs_seed_kernel<<<grid_for(N, 256), 256, 0, s>>>(part, N, P, w.bits, words, w.map, err);
+  launch_pdl(bfs_seed_kernel, grid_for(N, 256), 256, 0, s, part, N, P, w.bits, words, w.map, err);
   XMGN_LAUNCH_CHECK();
   if (L > 0) {
-    bfs_first_kernel<<<grid_for(N, 256, int64_t(num_sms()) * 8), 256, 0, s>>>(row_ptr, col, N, part, P, w.bits, words,
+    launch_pdl(bfs_first_kernel, grid_for(N, 256, int64_t(num_sms()) * 8), 256, 0, s, row_ptr, col, N, part, P, w.bits, words,
                                                                               w.map, w.members, w.counters, w.cap, err);
     XMGN_LAUNCH_CHECK();
   }
   for (int h = 2; h <= L; ++h) {
-    bfs_round_kernel<<<grid_for(N * 8, 256, int64_t(num_sms()) * 8), 256, 0, s>>>(
+    launch_pdl(bfs_round_kernel, grid_for(N * 8, 256, int64_t(num_sms()) * 8), 256, 0, s, 
         row_ptr, col, N, w.bits, words, w.map, w.members, w.counters, h, w.cap, err);
     XMGN_LAUNCH_CHECK();
   }
@@ -847,10 +875,10 @@ xmgn_status partition_halo(const int64_t* row_ptr, const int32_t* col, int64_t N
   // ---------------- batch order and sizes
   const int64_t nblk = hop_blocks(N), hc = int64_t(P) * (L + 1) * nblk;
   const dim3 hgrid(static_cast<unsigned>(nblk), static_cast<unsigned>(P));
-  hop_count_kernel<<<hgrid, 256, 0, s>>>(w.bits, w.map, words, N, L, w.hcnt);
+  launch_pdl(hop_count_kernel, hgrid, 256, 0, s, w.bits, w.map, words, N, L, w.hcnt);
   XMGN_LAUNCH_CHECK();
   XMGN_TRY(exclusive_scan_i32(w.hcnt, w.hbase, hc, w.scan_tmp, s));
-  part_sizes_kernel<<<grid_for(P + 1, 256), 256, 0, s>>>(w.hbase, nblk, P, L, err, w.info);
+  launch_pdl(part_sizes_kernel, grid_for(P + 1, 256), 256, 0, s, w.hbase, nblk, P, L, err, w.info);
   XMGN_LAUNCH_CHECK();
   std::vector<int64_t> info(size_t(2) * P + 3);
   XMGN_CUDA(cudaMemcpyAsync(info.data(), w.info, sizeof(int64_t) * info.size(), cudaMemcpyDeviceToHost, s));
@@ -868,17 +896,17 @@ xmgn_status partition_halo(const int64_t* row_ptr, const int32_t* col, int64_t N
   for (int p = 0; p < P; ++p) inner_cnt[p] = info[3 + P + p];
 
   // ---------------- batch nodes and degrees
-  hop_place_kernel<<<hgrid, 256, 0, s>>>(w.bits, w.map, words, N, L, w.hbase, w.members, emit ? gid : nullptr,
+  launch_pdl(hop_place_kernel, hgrid, 256, 0, s, w.bits, w.map, words, N, L, w.hbase, w.members, emit ? gid : nullptr,
                                          emit ? hop : nullptr);
   XMGN_LAUNCH_CHECK();
   if (nb > 0) {
-    batch_deg_kernel<<<grid_for(nb, 256), 256, 0, s>>>(w.members, nb, N, L, row_ptr, col, w.bits, words, w.deg, err);
+    launch_pdl(batch_deg_kernel, grid_for(nb, 256), 256, 0, s, w.members, nb, N, L, row_ptr, col, w.bits, words, w.deg, err);
     XMGN_LAUNCH_CHECK();
   }
   int64_t* brp = emit ? b_row_ptr : w.brp;
   XMGN_TRY(exclusive_scan_i32(w.deg, brp, nb, w.scan_tmp, s));
   int64_t* d_edge_ptr = w.info + 2 * int64_t(P) + 3;
-  part_edges_kernel<<<grid_for(P + 1, 256), 256, 0, s>>>(brp, w.info + 2, P, d_edge_ptr);
+  launch_pdl(part_edges_kernel, grid_for(P + 1, 256), 256, 0, s, brp, w.info + 2, P, d_edge_ptr);
   XMGN_LAUNCH_CHECK();
   XMGN_CUDA(cudaMemcpyAsync(edge_ptr, d_edge_ptr, sizeof(int64_t) * size_t(P + 1), cudaMemcpyDeviceToHost, s));
   XMGN_CUDA(cudaStreamSynchronize(s));

@@ -41,6 +41,8 @@ __device__ __forceinline__ int64_t block_sum64(int64_t x, int64_t* red) {
 template <class T>
 __global__ void __launch_bounds__(kScanThreads) tile_sum_kernel(const T* __restrict__ in, int64_t n,
                                                                 int64_t* __restrict__ sums) {
+  pdl_wait();
+  pdl_trigger();
   __shared__ int64_t red[kScanThreads / 32];
   const int64_t base = int64_t(blockIdx.x) * kScanTile;
   int64_t s = 0;
@@ -59,6 +61,8 @@ template <class T, class O>
 __global__ void __launch_bounds__(kScanThreads) tile_scan_kernel(const T* __restrict__ in, O* __restrict__ out,
                                                                  int64_t n, const int64_t* __restrict__ sums,
                                                                  int scanned) {
+  pdl_wait();
+  pdl_trigger();
   __shared__ int64_t red[kScanThreads / 32];
   __shared__ int64_t tile[kScanTile + kScanTile / kScanItems];
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
@@ -114,7 +118,7 @@ xmgn_status scan_impl(const T* in, O* out, int64_t n, int64_t* tmp, cudaStream_t
   const int64_t nt = (n + kScanTile - 1) / kScanTile;
   const int64_t* sums = nullptr;
   if (nt > 1) {
-    tile_sum_kernel<T><<<unsigned(nt), kScanThreads, 0, s>>>(in, n, tmp);
+    launch_pdl(tile_sum_kernel<T>, unsigned(nt), kScanThreads, 0, s, in, n, tmp);
     XMGN_LAUNCH_CHECK();
     sums = tmp;
     if (nt > kDirectTiles) {
@@ -122,7 +126,7 @@ xmgn_status scan_impl(const T* in, O* out, int64_t n, int64_t* tmp, cudaStream_t
       sums = tmp + nt;
     }
   }
-  tile_scan_kernel<T, O><<<unsigned(nt), kScanThreads, 0, s>>>(in, out, n, sums, nt > kDirectTiles ? 1 : 0);
+  launch_pdl(tile_scan_kernel<T, O>, unsigned(nt), kScanThreads, 0, s, in, out, n, sums, nt > kDirectTiles ? 1 : 0);
   XMGN_LAUNCH_CHECK();
   return XMGN_OK;
 }

@@ -70,6 +70,8 @@ __global__ void __launch_bounds__(256) general_nnt_kernel(RowSrc A, int64_t M, c
                                                           const float* __restrict__ bias, float* __restrict__ C,
                                                           int64_t ldc, int epi, float* __restrict__ pre,
                                                           const float* __restrict__ aux, RowAdd add) {
+  pdl_wait();
+  pdl_trigger();
   __shared__ float As[BK][GT + 4];
   __shared__ float Bs[BK][GT + 4];
   const int K = A.K;
@@ -125,6 +127,8 @@ __global__ void __launch_bounds__(256) general_nnt_kernel(RowSrc A, int64_t M, c
 __global__ void __launch_bounds__(256) general_tn_kernel(RowSrc A, int64_t M, const float* __restrict__ B,
                                                          int64_t ldb, int N, int64_t rows_per_chunk,
                                                          float* __restrict__ part) {
+  pdl_wait();
+  pdl_trigger();
   __shared__ float As[BK][GT + 4];
   __shared__ float Bs[BK][GT + 4];
   const int K1 = A.K;
@@ -244,6 +248,8 @@ struct SgemmArgs {
 // every base 16-byte aligned.
 template <int FORM, int BN>
 __global__ void __launch_bounds__(256, 2) sgemm_kernel(const __grid_constant__ SgemmArgs a) {
+  pdl_wait();
+  pdl_trigger();
   constexpr int TN = BN / 16;  // output columns per thread
   __shared__ __align__(16) float As[2][BK][BM + 4];
   __shared__ __align__(16) float Bs[2][BK][BN + 4];
@@ -454,9 +460,9 @@ xmgn_status run_fast(const SgemmArgs& a, int64_t rows, int64_t chunks, cudaStrea
   const int64_t tn = wide ? (a.N + 127) / 128 : (a.N + 63) / 64;
   const dim3 grid = FORM == G_TN ? dim3(unsigned(tm * tn), unsigned(chunks)) : dim3(unsigned(tm), unsigned(tn));
   if (wide)
-    sgemm_kernel<FORM, 128><<<grid, 256, 0, s>>>(a);
+    launch_pdl(sgemm_kernel<FORM, 128>, grid, 256, 0, s, a);
   else
-    sgemm_kernel<FORM, 64><<<grid, 256, 0, s>>>(a);
+    launch_pdl(sgemm_kernel<FORM, 64>, grid, 256, 0, s, a);
   XMGN_LAUNCH_CHECK();
   return XMGN_OK;
 }
@@ -479,7 +485,7 @@ xmgn_status gemm_nn_f32(const RowSrc& A, int64_t M, const float* B, int N, const
   const SgemmArgs a{A, M, B, N, N, bias, C, ldc, epi, pre, aux, add, 0};
   if (fast(a)) return run_fast<G_NN>(a, M, 1, s);
   dim3 grid(unsigned((M + GT - 1) / GT), unsigned((N + GT - 1) / GT));
-  general_nnt_kernel<false><<<grid, 256, 0, s>>>(A, M, B, N, bias, C, ldc, epi, pre, aux, add);
+  launch_pdl(general_nnt_kernel<false>, grid, 256, 0, s, A, M, B, N, bias, C, ldc, epi, pre, aux, add);
   XMGN_LAUNCH_CHECK();
   return XMGN_OK;
 }
@@ -490,7 +496,7 @@ xmgn_status gemm_nt_f32(const RowSrc& A, int64_t M, const float* B, int N, float
   const SgemmArgs a{A, M, B, A.K, N, nullptr, C, ldc, epi, nullptr, aux, RowAdd{}, 0};
   if (fast(a)) return run_fast<G_NT>(a, M, 1, s);
   dim3 grid(unsigned((M + GT - 1) / GT), unsigned((N + GT - 1) / GT));
-  general_nnt_kernel<true><<<grid, 256, 0, s>>>(A, M, B, N, nullptr, C, ldc, epi, nullptr, aux, RowAdd{});
+  launch_pdl(general_nnt_kernel<true>, grid, 256, 0, s, A, M, B, N, nullptr, C, ldc, epi, nullptr, aux, RowAdd{});
   XMGN_LAUNCH_CHECK();
   return XMGN_OK;
 }
@@ -515,7 +521,7 @@ xmgn_status gemm_tn_f32(const RowSrc& A, int64_t M, const float* B, int64_t ldb,
     XMGN_TRY(run_fast<G_TN>(a, K1, nc, s));
   } else {
     const int tiles = ((K1 + GT - 1) / GT) * ((N + GT - 1) / GT);
-    general_tn_kernel<<<dim3(tiles, nc), 256, 0, s>>>(A, M, B, ldb, N, rpc, part);
+    launch_pdl(general_tn_kernel, dim3(tiles, nc), 256, 0, s, A, M, B, ldb, N, rpc, part);
     XMGN_LAUNCH_CHECK();
   }
   return sum_parts_f32(part, nc, K1 * N, G, s);

@@ -28,6 +28,8 @@ __device__ __forceinline__ float sum_strided(const float* __restrict__ x, int n,
 // Column sums of one chunk of rows (eight loads in flight per thread).
 __global__ void colsum_kernel(const float* __restrict__ X, int64_t M, int N, int64_t ld,
                               int64_t rows_per_chunk, float* __restrict__ part) {
+  pdl_wait();
+  pdl_trigger();
   const int64_t r0 = int64_t(blockIdx.x) * rows_per_chunk;
   const int64_t r1 = min(M, r0 + rows_per_chunk);
   for (int n = threadIdx.x; n < N; n += blockDim.x)
@@ -48,6 +50,8 @@ constexpr int kMaxVpl = 16;  // features per lane (N <= 512)
 __global__ void ln_fwd_kernel(const float* __restrict__ Z, const float* __restrict__ bias, int64_t M, int N,
                               const float* __restrict__ gamma, const float* __restrict__ beta,
                               float* __restrict__ Y, const float* resid_in, float* resid_out) {
+  pdl_wait();
+  pdl_trigger();
   const int lane = threadIdx.x & 31;
   const int64_t warp = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
   const int64_t nw = (int64_t(gridDim.x) * blockDim.x) >> 5;
@@ -96,6 +100,8 @@ __global__ void __launch_bounds__(256, 3)
                   const float* __restrict__ gamma, const float* __restrict__ dY1, const float* __restrict__ dY2,
                   const int32_t* __restrict__ idx2, float* __restrict__ dZ, bf16* __restrict__ dZ16,
                   float* __restrict__ part) {
+  pdl_wait();
+  pdl_trigger();
   extern __shared__ float ln_acc[];  // [8 warps][dgamma N | dbeta N | column sums of dZ N]
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   float* acc = ln_acc + wib * 3 * N;
@@ -174,6 +180,8 @@ __global__ void __launch_bounds__(256, 3)
 __global__ void __launch_bounds__(256) sum_parts_kernel(const float* __restrict__ part, int nb, int len,
                                                         float* __restrict__ out, int split, float* __restrict__ out2,
                                                         float* __restrict__ out3) {
+  pdl_wait();
+  pdl_trigger();
   __shared__ float red[8][32];
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   const int c = blockIdx.x * 32 + lane;
@@ -196,6 +204,8 @@ __global__ void ln_fwd_agg_kernel(const float* __restrict__ Z, const float* __re
                                   const int64_t* __restrict__ rp, int64_t n, int N, const float* __restrict__ gamma,
                                   const float* __restrict__ beta, const float* resid_in, float* resid_out,
                                   float* __restrict__ agg) {
+  pdl_wait();
+  pdl_trigger();
   const int lane = threadIdx.x & 31;
   const int64_t warp = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
   const int64_t nw = (int64_t(gridDim.x) * blockDim.x) >> 5;
@@ -289,6 +299,8 @@ __global__ void __launch_bounds__(256) ln_fwd_v4_kernel(const float* __restrict_
                                                         int64_t M, const float* __restrict__ gamma,
                                                         const float* __restrict__ beta, float* __restrict__ Y,
                                                         const float* resid_in, float* resid_out) {
+  pdl_wait();
+  pdl_trigger();
   constexpr int N = 128 * V4;
   const int lane = threadIdx.x & 31;
   const int64_t warp = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
@@ -326,6 +338,8 @@ __global__ void __launch_bounds__(256) ln_fwd_agg_v4_kernel(const float* __restr
                                                             const float* __restrict__ gamma,
                                                             const float* __restrict__ beta, const float* resid_in,
                                                             float* resid_out, float* __restrict__ agg) {
+  pdl_wait();
+  pdl_trigger();
   constexpr int N = 128 * V4;
   const int lane = threadIdx.x & 31;
   const int64_t warp = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
@@ -371,6 +385,8 @@ __global__ void __launch_bounds__(256, 3)
                      const float* __restrict__ gamma, const float* __restrict__ dY1, const float* __restrict__ dY2,
                      const int32_t* __restrict__ idx2, float* __restrict__ dZ, bf16* __restrict__ dZ16,
                      float* __restrict__ part) {
+  pdl_wait();
+  pdl_trigger();
   constexpr int N = 128 * V4;
   extern __shared__ float ln_acc[];  // [8 warps][dgamma N | dbeta N | column sums of dZ N]
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
@@ -456,6 +472,8 @@ template <bool PERM>
 __global__ void seg_sum_v4_kernel(const float* __restrict__ v, int64_t ldv, const int64_t* __restrict__ rp,
                                   const int32_t* __restrict__ perm, int64_t n, int H, float* __restrict__ out,
                                   int64_t ldo, int acc) {
+  pdl_wait();
+  pdl_trigger();
   const int lane = threadIdx.x & 31;
   const int64_t warp = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
   const int64_t nw = (int64_t(gridDim.x) * blockDim.x) >> 5;
@@ -485,6 +503,8 @@ __global__ void seg_sum_v4_kernel(const float* __restrict__ v, int64_t ldv, cons
 
 __global__ void seg_rows_kernel(const float* __restrict__ v, int64_t ldv, const int64_t* __restrict__ rp,
                                 int64_t n, int H, float* __restrict__ out, int64_t ldo, int acc) {
+  pdl_wait();
+  pdl_trigger();
   const int lane = threadIdx.x & 31;
   const int64_t warp = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
   const int64_t nw = (int64_t(gridDim.x) * blockDim.x) >> 5;
@@ -501,6 +521,8 @@ __global__ void seg_rows_kernel(const float* __restrict__ v, int64_t ldv, const 
 __global__ void seg_cols_kernel(const float* __restrict__ v, int64_t ldv, const int64_t* __restrict__ rp,
                                 const int32_t* __restrict__ perm, int64_t n, int H,
                                 float* __restrict__ out, int64_t ldo, int acc) {
+  pdl_wait();
+  pdl_trigger();
   const int lane = threadIdx.x & 31;
   const int64_t warp = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
   const int64_t nw = (int64_t(gridDim.x) * blockDim.x) >> 5;
@@ -517,6 +539,8 @@ __global__ void seg_cols_kernel(const float* __restrict__ v, int64_t ldv, const 
 __global__ void edge_feat_kernel(const float* __restrict__ xyz, const int32_t* __restrict__ gid,
                                  const int32_t* __restrict__ recv, const int32_t* __restrict__ col,
                                  int64_t E, float* __restrict__ f) {
+  pdl_wait();
+  pdl_trigger();
   for (int64_t e = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; e < E;
        e += int64_t(gridDim.x) * blockDim.x) {
     int64_t r = recv[e], s = col[e];
@@ -606,9 +630,9 @@ xmgn_status colsum_f32(const float* X, int64_t M, int N, int64_t ld, float* g, f
   const int nc = colsum_chunks(M);
   int64_t rpc = (M + nc - 1) / nc;
   if (rpc < 1) rpc = 1;
-  colsum_kernel<<<nc, 256, 0, s>>>(X, M, N, ld, rpc, part);
+  launch_pdl_if(rows_early(M, N), colsum_kernel, nc, 256, 0, s, X, M, N, ld, rpc, part);
   XMGN_LAUNCH_CHECK();
-  sum_parts_kernel<<<(N + 31) / 32, 256, 0, s>>>(part, nc, N, g, N, nullptr, nullptr);
+  launch_pdl(sum_parts_kernel, (N + 31) / 32, 256, 0, s, part, nc, N, g, N, nullptr, nullptr);
   XMGN_LAUNCH_CHECK();
   return XMGN_OK;
 }
@@ -629,13 +653,13 @@ xmgn_status layernorm_fwd_f32(const float* Z, int64_t M, int N, const float* gam
   if (M <= 0) return XMGN_OK;
   const unsigned grid = grid_for(M * 32, 256, int64_t(num_sms()) * 16);
   if (rows_vec4(N, {Z, Y, resid_in, resid_out})) {
-    if (N == 128) ln_fwd_v4_kernel<1><<<grid, 256, 0, s>>>(Z, bias, M, gamma, beta, Y, resid_in, resid_out);
-    if (N == 256) ln_fwd_v4_kernel<2><<<grid, 256, 0, s>>>(Z, bias, M, gamma, beta, Y, resid_in, resid_out);
-    if (N == 512) ln_fwd_v4_kernel<4><<<grid, 256, 0, s>>>(Z, bias, M, gamma, beta, Y, resid_in, resid_out);
+    if (N == 128) launch_pdl_if(rows_early(M, N), ln_fwd_v4_kernel<1>, grid, 256, 0, s, Z, bias, M, gamma, beta, Y, resid_in, resid_out);
+    if (N == 256) launch_pdl_if(rows_early(M, N), ln_fwd_v4_kernel<2>, grid, 256, 0, s, Z, bias, M, gamma, beta, Y, resid_in, resid_out);
+    if (N == 512) launch_pdl_if(rows_early(M, N), ln_fwd_v4_kernel<4>, grid, 256, 0, s, Z, bias, M, gamma, beta, Y, resid_in, resid_out);
     XMGN_LAUNCH_CHECK();
     return XMGN_OK;
   }
-  ln_fwd_kernel<<<grid, 256, 0, s>>>(Z, bias, M, N, gamma, beta, Y, resid_in, resid_out);
+  launch_pdl_if(rows_early(M, N), ln_fwd_kernel, grid, 256, 0, s, Z, bias, M, N, gamma, beta, Y, resid_in, resid_out);
   XMGN_LAUNCH_CHECK();
   return XMGN_OK;
 }
@@ -647,13 +671,13 @@ xmgn_status layernorm_fwd_agg_f32(const float* Z, const float* bias, const int64
   if (n <= 0) return XMGN_OK;
   const unsigned grid = grid_for(n * 32, 256, int64_t(num_sms()) * 16);
   if (rows_vec4(N, {Z, resid_in, resid_out, agg})) {
-    if (N == 128) ln_fwd_agg_v4_kernel<1><<<grid, 256, 0, s>>>(Z, bias, row_ptr, n, gamma, beta, resid_in, resid_out, agg);
-    if (N == 256) ln_fwd_agg_v4_kernel<2><<<grid, 256, 0, s>>>(Z, bias, row_ptr, n, gamma, beta, resid_in, resid_out, agg);
-    if (N == 512) ln_fwd_agg_v4_kernel<4><<<grid, 256, 0, s>>>(Z, bias, row_ptr, n, gamma, beta, resid_in, resid_out, agg);
+    if (N == 128) launch_pdl_if(rows_early(8 * n, N), ln_fwd_agg_v4_kernel<1>, grid, 256, 0, s, Z, bias, row_ptr, n, gamma, beta, resid_in, resid_out, agg);
+    if (N == 256) launch_pdl_if(rows_early(8 * n, N), ln_fwd_agg_v4_kernel<2>, grid, 256, 0, s, Z, bias, row_ptr, n, gamma, beta, resid_in, resid_out, agg);
+    if (N == 512) launch_pdl_if(rows_early(8 * n, N), ln_fwd_agg_v4_kernel<4>, grid, 256, 0, s, Z, bias, row_ptr, n, gamma, beta, resid_in, resid_out, agg);
     XMGN_LAUNCH_CHECK();
     return XMGN_OK;
   }
-  ln_fwd_agg_kernel<<<grid, 256, 0, s>>>(Z, bias, row_ptr, n, N, gamma, beta, resid_in, resid_out, agg);
+  launch_pdl_if(rows_early(8 * n, N), ln_fwd_agg_kernel, grid, 256, 0, s, Z, bias, row_ptr, n, N, gamma, beta, resid_in, resid_out, agg);
   XMGN_LAUNCH_CHECK();
   return XMGN_OK;
 }
@@ -662,7 +686,7 @@ int colsum_chunk_count(int64_t M) { return colsum_chunks(M); }
 
 xmgn_status sum_parts_f32(const float* part, int nb, int len, float* out, cudaStream_t s) {
   if (len <= 0) return XMGN_OK;
-  sum_parts_kernel<<<(len + 31) / 32, 256, 0, s>>>(part, nb, len, out, len, nullptr, nullptr);
+  launch_pdl(sum_parts_kernel, (len + 31) / 32, 256, 0, s, part, nb, len, out, len, nullptr, nullptr);
   XMGN_LAUNCH_CHECK();
   return XMGN_OK;
 }
@@ -681,14 +705,14 @@ xmgn_status layernorm_bwd_f32(const float* Z, int64_t M, int N, const float* gam
   if (nb < 1) nb = 1;
   const size_t sh = size_t(8) * 3 * N * sizeof(float);
   if (rows_vec4(N, {Z, dY1, dY2, dZ, reinterpret_cast<const float*>(dZ16)})) {
-    if (N == 128) ln_bwd_v4_kernel<1><<<unsigned(nb), 256, sh, s>>>(Z, bias, M, gamma, dY1, dY2, idx2, dZ, dZ16, part);
-    if (N == 256) ln_bwd_v4_kernel<2><<<unsigned(nb), 256, sh, s>>>(Z, bias, M, gamma, dY1, dY2, idx2, dZ, dZ16, part);
-    if (N == 512) ln_bwd_v4_kernel<4><<<unsigned(nb), 256, sh, s>>>(Z, bias, M, gamma, dY1, dY2, idx2, dZ, dZ16, part);
+    if (N == 128) launch_pdl_if(rows_early(M, N), ln_bwd_v4_kernel<1>, unsigned(nb), 256, sh, s, Z, bias, M, gamma, dY1, dY2, idx2, dZ, dZ16, part);
+    if (N == 256) launch_pdl_if(rows_early(M, N), ln_bwd_v4_kernel<2>, unsigned(nb), 256, sh, s, Z, bias, M, gamma, dY1, dY2, idx2, dZ, dZ16, part);
+    if (N == 512) launch_pdl_if(rows_early(M, N), ln_bwd_v4_kernel<4>, unsigned(nb), 256, sh, s, Z, bias, M, gamma, dY1, dY2, idx2, dZ, dZ16, part);
   } else {
-    ln_bwd_kernel<<<unsigned(nb), 256, sh, s>>>(Z, bias, M, N, gamma, dY1, dY2, idx2, dZ, dZ16, part);
+    launch_pdl_if(rows_early(M, N), ln_bwd_kernel, unsigned(nb), 256, sh, s, Z, bias, M, N, gamma, dY1, dY2, idx2, dZ, dZ16, part);
   }
   XMGN_LAUNCH_CHECK();
-  sum_parts_kernel<<<(3 * N + 31) / 32, 256, 0, s>>>(part, int(nb), 3 * N, dgamma, N, dbeta, db);
+  launch_pdl(sum_parts_kernel, (3 * N + 31) / 32, 256, 0, s, part, int(nb), 3 * N, dgamma, N, dbeta, db);
   XMGN_LAUNCH_CHECK();
   return XMGN_OK;
 }
@@ -704,9 +728,9 @@ xmgn_status seg_sum_rows_f32(const float* v, int64_t ldv, const int64_t* row_ptr
   if (n <= 0) return XMGN_OK;
   const unsigned grid = grid_for(n * 32, 256, int64_t(num_sms()) * 16);
   if (seg_vec4(v, ldv, H, out, ldo))
-    seg_sum_v4_kernel<false><<<grid, 256, 0, s>>>(v, ldv, row_ptr, nullptr, n, H, out, ldo, accumulate ? 1 : 0);
+    launch_pdl_if(rows_early(8 * n, H), seg_sum_v4_kernel<false>, grid, 256, 0, s, v, ldv, row_ptr, nullptr, n, H, out, ldo, accumulate ? 1 : 0);
   else
-    seg_rows_kernel<<<grid, 256, 0, s>>>(v, ldv, row_ptr, n, H, out, ldo, accumulate ? 1 : 0);
+    launch_pdl_if(rows_early(8 * n, H), seg_rows_kernel, grid, 256, 0, s, v, ldv, row_ptr, n, H, out, ldo, accumulate ? 1 : 0);
   XMGN_LAUNCH_CHECK();
   return XMGN_OK;
 }
@@ -717,9 +741,9 @@ xmgn_status seg_sum_cols_f32(const float* v, int64_t ldv, const int64_t* row_ptr
   if (n <= 0) return XMGN_OK;
   const unsigned grid = grid_for(n * 32, 256, int64_t(num_sms()) * 16);
   if (seg_vec4(v, ldv, H, out, ldo))
-    seg_sum_v4_kernel<true><<<grid, 256, 0, s>>>(v, ldv, row_ptr, perm, n, H, out, ldo, accumulate ? 1 : 0);
+    launch_pdl_if(rows_early(8 * n, H), seg_sum_v4_kernel<true>, grid, 256, 0, s, v, ldv, row_ptr, perm, n, H, out, ldo, accumulate ? 1 : 0);
   else
-    seg_cols_kernel<<<grid, 256, 0, s>>>(v, ldv, row_ptr, perm, n, H, out, ldo, accumulate ? 1 : 0);
+    launch_pdl_if(rows_early(8 * n, H), seg_cols_kernel, grid, 256, 0, s, v, ldv, row_ptr, perm, n, H, out, ldo, accumulate ? 1 : 0);
   XMGN_LAUNCH_CHECK();
   return XMGN_OK;
 }
@@ -729,6 +753,8 @@ namespace {
 // 2^(q+1) pi x_c for the three coordinates (sines first).
 __global__ void node_feat_kernel(const float* __restrict__ node_in, int in_node, const float* __restrict__ xyz,
                                  const int32_t* __restrict__ gid, int64_t n, int F, float* __restrict__ out) {
+  pdl_wait();
+  pdl_trigger();
   const int w = in_node + 6 * F;
   for (int64_t r = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; r < n;
        r += int64_t(gridDim.x) * blockDim.x) {
@@ -749,7 +775,7 @@ __global__ void node_feat_kernel(const float* __restrict__ node_in, int in_node,
 
 xmgn_status node_features(const float* node_in, int in_node, const float* xyz, const int32_t* gid, int64_t n,
                           int fourier, float* out, cudaStream_t s) {
-  node_feat_kernel<<<grid_for(n, 256), 256, 0, s>>>(node_in, in_node, xyz, gid, n, fourier, out);
+  launch_pdl(node_feat_kernel, grid_for(n, 256), 256, 0, s, node_in, in_node, xyz, gid, n, fourier, out);
   XMGN_LAUNCH_CHECK();
   return XMGN_OK;
 }
@@ -757,7 +783,7 @@ xmgn_status node_features(const float* node_in, int in_node, const float* xyz, c
 xmgn_status edge_features(const float* xyz, const int32_t* gid, const int32_t* recv,
                           const int32_t* col, int64_t E, float* f, cudaStream_t s) {
   if (E <= 0) return XMGN_OK;
-  edge_feat_kernel<<<grid_for(E, 256), 256, 0, s>>>(xyz, gid, recv, col, E, f);
+  launch_pdl(edge_feat_kernel, grid_for(E, 256), 256, 0, s, xyz, gid, recv, col, E, f);
   XMGN_LAUNCH_CHECK();
   return XMGN_OK;
 }

@@ -150,6 +150,7 @@ __global__ void __launch_bounds__(kWgThreads, 1) wg_kernel(WgArgs a, const __gri
   __syncthreads();
   tc_fence_after();
   const uint32_t tacc = tbase;
+  pdl_wait();
   if (warp == 0) {
     // ------------------------------------------------------------ TMA producer
     if (lane == 0) {
@@ -314,6 +315,9 @@ __global__ void __launch_bounds__(kWgThreads, 1) wg_kernel(WgArgs a, const __gri
     }
   }
   if (tid == 64 || tid == 192) bulk_wait0();  // every output store is complete
+  // Only now: a row kernel started beside this one would run with the little L1
+  // that this one's shared memory leaves.
+  pdl_trigger();
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -323,6 +327,8 @@ __global__ void __launch_bounds__(kWgThreads, 1) wg_kernel(WgArgs a, const __gri
 // G[K1, N] = sum over splits of the partial tiles, in split order.
 __global__ void __launch_bounds__(256) wg_reduce_kernel(const float* __restrict__ part, int splits, int tiles_m,
                                                         int tiles_n, int BN, int K1, int N, float* __restrict__ G) {
+  pdl_wait();
+  pdl_trigger();
   const int64_t total = int64_t(K1) * N;
   for (int64_t e = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; e < total; e += int64_t(gridDim.x) * blockDim.x) {
     const int k = int(e / N), n = int(e % N);
@@ -410,7 +416,7 @@ xmgn_status launch(WgArgs& a, const CUtensorMap& ta, const CUtensorMap& tb, cons
   probe_begin(PROBE_WIDE_GEMM, s);
   CUtensorMap none;
   memset(&none, 0, sizeof(none));
-  wg_kernel<<<grid, kWgThreads, smem, s>>>(a, ta, tb, td, tp ? *tp : none);
+  launch_pdl(wg_kernel, grid, kWgThreads, smem, s, a, ta, tb, td, tp ? *tp : none);
   probe_end(PROBE_WIDE_GEMM, s);
   XMGN_LAUNCH_CHECK();
   return XMGN_OK;
@@ -506,7 +512,7 @@ xmgn_status wg_gemm_tn(const bf16* A, int64_t lda, const bf16* B, int64_t ldb, i
   XMGN_TRY(f32_map(&td, part, int64_t(a.splits) * tiles * kBM, a.BN, a.BN));  // [split][tile] blocks of 128 x BN
   XMGN_TRY(launch(a, ta, tb, td, s));
   const int64_t total = int64_t(K1) * N;
-  wg_reduce_kernel<<<grid_for(total, 256, int64_t(num_sms()) * 8), 256, 0, s>>>(part, a.splits, a.tiles_m, a.tiles_n,
+  launch_pdl(wg_reduce_kernel, grid_for(total, 256, int64_t(num_sms()) * 8), 256, 0, s, part, a.splits, a.tiles_m, a.tiles_n,
                                                                                a.BN, K1, N, G);
   XMGN_LAUNCH_CHECK();
   return XMGN_OK;

@@ -36,6 +36,8 @@ __device__ __forceinline__ uint2 bf16x4(float4 v) {
 // segments whose width, leading dimension and offsets are multiples of 4 move
 // four values per lane (16-byte loads, 8-byte stores).
 __global__ void gather_bf16_kernel(RowSrc A, int64_t M, bf16* __restrict__ out, int64_t ldo) {
+  pdl_wait();
+  pdl_trigger();
   const int lane = threadIdx.x & 31;
   for (int64_t r = warp_id(); r < M; r += warp_count()) {
     int k0 = 0;
@@ -84,6 +86,8 @@ __device__ __forceinline__ float epi_one(float z, int epi, float* pre_el, float 
 __global__ void epilogue_kernel(const float* __restrict__ acc, int64_t M, int N, const float* __restrict__ bias,
                                 float* __restrict__ C, int64_t ldc, int epi, float* __restrict__ pre,
                                 const float* __restrict__ aux, bf16* __restrict__ C16) {
+  pdl_wait();
+  pdl_trigger();
   const int lane = threadIdx.x & 31;
   const bool vec = ((N | ldc) & 3) == 0;
   for (int64_t r = warp_id(); r < M; r += warp_count()) {
@@ -127,6 +131,8 @@ __global__ void epilogue_kernel(const float* __restrict__ acc, int64_t M, int N,
 __global__ void __launch_bounds__(256) silu_grad_colsum_kernel(const float* __restrict__ acc, int64_t M, int N,
                                                                const float* __restrict__ Z1, bf16* __restrict__ C16,
                                                                int64_t rpc, float* __restrict__ part) {
+  pdl_wait();
+  pdl_trigger();
   __shared__ float red[8][512];
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   float cs[16];
@@ -209,7 +215,7 @@ WideScratch wide_scratch(void* p, int64_t R, int H, int Kmax, int out) {
 
 xmgn_status wide_gather(const RowSrc& A, int64_t M, bf16* out, cudaStream_t s) {
   if (M <= 0) return XMGN_OK;
-  gather_bf16_kernel<<<blocks(M), 256, 0, s>>>(A, M, out, pad8(A.K));
+  launch_pdl_if(rows_early(M, A.K), gather_bf16_kernel, blocks(M), 256, 0, s, A, M, out, pad8(A.K));
   XMGN_LAUNCH_CHECK();
   return XMGN_OK;
 }
@@ -238,7 +244,7 @@ xmgn_status wide_tn(const bf16* A, int64_t M, int K1, const bf16* B, int N, floa
 xmgn_status wide_epilogue(const float* acc, int64_t M, int N, const float* bias, float* C, int64_t ldc, int epi,
                           float* pre, const float* aux, bf16* C16, cudaStream_t s) {
   if (M <= 0) return XMGN_OK;
-  epilogue_kernel<<<blocks(M), 256, 0, s>>>(acc, M, N, bias, C, ldc, epi, pre, aux, C16);
+  launch_pdl_if(rows_early(M, N), epilogue_kernel, blocks(M), 256, 0, s, acc, M, N, bias, C, ldc, epi, pre, aux, C16);
   XMGN_LAUNCH_CHECK();
   return XMGN_OK;
 }
@@ -249,7 +255,7 @@ xmgn_status wide_silu_grad_colsum(const float* acc, int64_t M, int N, const floa
   const int nb = colsum_chunk_count(M);
   int64_t rpc = (M + nb - 1) / nb;
   if (rpc < 1) rpc = 1;
-  silu_grad_colsum_kernel<<<nb, 256, 0, s>>>(acc, M, N, Z1, C16, rpc, part);
+  launch_pdl_if(rows_early(M, N), silu_grad_colsum_kernel, nb, 256, 0, s, acc, M, N, Z1, C16, rpc, part);
   XMGN_LAUNCH_CHECK();
   return sum_parts_f32(part, nb, N, db, s);
 }
