@@ -42,11 +42,12 @@ def _check(xyz, k):
 
 
 @pytest.mark.parametrize("k", [1, 3, 4, 7, 16, 17, 32])
-@pytest.mark.parametrize("kind,n", [("sphere", 33), ("line", 257), ("dup", 600), ("volume", 900), ("flat", 640)])
+@pytest.mark.parametrize("kind,n", [("sphere", 33), ("line", 257), ("dup", 600), ("dup", 9000), ("volume", 900),
+                                    ("flat", 640)])
 def test_candidate_lists_rings_and_rows(kind, n, k):
     deg = _check(_cloud(kind, n, k), k)
     if kind == "dup":
-        assert deg.max() > 64  # the global sort has run
+        assert deg.max() > (1040 if n > 8500 else 64)  # rows past the shared-memory sort
 
 
 def test_one_lane_per_point():
