@@ -137,13 +137,6 @@ __device__ __forceinline__ void ld_g32(float (&v)[32], const float* src) {
   for (int q = 0; q < 4; ++q) ld8(src + 8 * q, v + 8 * q);
 }
 
-__device__ __forceinline__ void add_g32(float (&v)[32], const float* src) {
-  float t[32];
-  ld_g32(t, src);
-#pragma unroll
-  for (int j = 0; j < 32; ++j) v[j] += t[j];
-}
-
 // v += 32 bf16 values at src (64 bytes, two 256-bit loads)
 __device__ __forceinline__ void add_g16(float (&v)[32], const bf16* src) {
 #pragma unroll
@@ -177,9 +170,10 @@ __device__ __forceinline__ float bf16_at(const uint32_t (&u)[16], int j) {
 
 // v = 32 bf16 values at src
 __device__ __forceinline__ void ld_g16(float (&v)[32], const bf16* src) {
+  uint32_t u[16];
+  ld_raw16(u, src);
 #pragma unroll
-  for (int j = 0; j < 32; ++j) v[j] = 0.f;
-  add_g16(v, src);
+  for (int j = 0; j < 32; ++j) v[j] = bf16_at(u, j);
 }
 
 // Copies rows [r0, min(r0+128, rows)) of a swizzled 128 x 128 bf16 tile to
@@ -786,8 +780,8 @@ __global__ void __launch_bounds__(kThreads, 1) edge_fwd_kernel(FwdArgs a, const 
     if (gt == 0) {
       tc_fence_after();
       const uint32_t wh = smem_u32(sm.w2h), wl = smem_u32(sm.w2l);
-mma_chain_ts<kH / 16, kH>(T + kH, T, wh, id_x, false);
-mma_chain_ts<kH / 16, kH>(T + kH, T, wl, id_x, true);
+      mma_chain_ts<kH / 16, kH>(T + kH, T, wh, id_x, false);
+      mma_chain_ts<kH / 16, kH>(T + kH, T, wl, id_x, true);
       mma_commit(&mb[g]);
     }
     {  // the group's next tile's node projections, for its epi1, towards L2 (one line per block and row)
@@ -819,15 +813,18 @@ mma_chain_ts<kH / 16, kH>(T + kH, T, wl, id_x, true);
       for (int w = 0; w < sp; ++w) idx += __popc(sstart[w]);
       sfirst[idx] = uint8_t(r);
     }
-    // ---- epi2: LayerNorm statistics over the two column halves of each row
+    // ---- epi2: LayerNorm statistics over the two column halves of each row; Z2 + b2 stays in registers
+    float v[2][32];
     float sum = 0.f;
 #pragma unroll
     for (int c = 0; c < 2; ++c) {
       const int cc = cA + 32 * c;
-      float v[32];
-      tmem_ld32(T + lane_base + kH + cc, v);
+      tmem_ld32(T + lane_base + kH + cc, v[c]);
 #pragma unroll
-      for (int j = 0; j < 32; ++j) sum += v[j] + cst(b2 + cc, j);
+      for (int j = 0; j < 32; ++j) {
+        v[c][j] += cst(b2 + cc, j);
+        sum += v[c][j];
+      }
     }
     red[(0 * 2 + ch) * 128 + r] = sum;
     group_sync(g);
@@ -835,13 +832,10 @@ mma_chain_ts<kH / 16, kH>(T + kH, T, wl, id_x, true);
     float qs = 0.f;
 #pragma unroll
     for (int c = 0; c < 2; ++c) {
-      const int cc = cA + 32 * c;
-      float v[32];
-      tmem_ld32(T + lane_base + kH + cc, v);
 #pragma unroll
       for (int j = 0; j < 32; ++j) {
-        const float d = v[j] + cst(b2 + cc, j) - mu;
-        qs += d * d;
+        v[c][j] -= mu;
+        qs += v[c][j] * v[c][j];
       }
     }
     red[(1 * 2 + ch) * 128 + r] = qs;
@@ -853,18 +847,16 @@ mma_chain_ts<kH / 16, kH>(T + kH, T, wl, id_x, true);
 #pragma unroll
     for (int c = 0; c < 2; ++c) {
       const int cc = cA + 32 * c;
-      float v[32];
-      tmem_ld32(T + lane_base + kH + cc, v);
 #pragma unroll
-      for (int j = 0; j < 32; ++j) v[j] = (v[j] + cst(b2 + cc, j) - mu) * rstd * cst(gam + cc, j) + cst(bet + cc, j);
+      for (int j = 0; j < 32; ++j) v[c][j] = v[c][j] * rstd * cst(gam + cc, j) + cst(bet + cc, j);
       if (a.o16) {
         float e[32];
         ld_tile32(X, 128, r, cc, e);
 #pragma unroll
-        for (int j = 0; j < 32; ++j) e[j] += v[j];
+        for (int j = 0; j < 32; ++j) e[j] += v[c][j];
         if (valid) st_g16(a.o16 + row * kH + cc, e);
       }
-      st_tile32(X, 128, r, cc, v);
+      st_tile32(X, 128, r, cc, v[c]);
     }
     tc_fence_before();
     group_sync(g);
@@ -958,8 +950,8 @@ __global__ void __launch_bounds__(kThreads, 1) node_fwd_kernel(FwdArgs a) {
     if (tid == 0) {
       tc_fence_after();
       const uint32_t wh = smem_u32(sm.w1h), wl = smem_u32(sm.w1l);
-mma_chain_ts<2 * kH / 16, kH>(tm + tZ1, tm + tX, wh, id, false);
-mma_chain_ts<2 * kH / 16, kH>(tm + tZ1, tm + tX, wl, id, true);
+      mma_chain_ts<2 * kH / 16, kH>(tm + tZ1, tm + tX, wh, id, false);
+      mma_chain_ts<2 * kH / 16, kH>(tm + tZ1, tm + tX, wl, id, true);
       mma_commit(&mbar);
     }
     const int64_t row = r0 + r;
@@ -992,8 +984,8 @@ mma_chain_ts<2 * kH / 16, kH>(tm + tZ1, tm + tX, wl, id, true);
     if (tid == 0) {
       tc_fence_after();
       const uint32_t wh = smem_u32(sm.w2h), wl = smem_u32(sm.w2l);
-mma_chain_ts<kH / 16, kH>(tm + tZ2, tm + tA, wh, id, false);
-mma_chain_ts<kH / 16, kH>(tm + tZ2, tm + tA, wl, id, true);
+      mma_chain_ts<kH / 16, kH>(tm + tZ2, tm + tA, wh, id, false);
+      mma_chain_ts<kH / 16, kH>(tm + tZ2, tm + tA, wl, id, true);
       mma_commit(&mbar);
     }
     float v[32], g0[32];
@@ -1123,14 +1115,13 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_bwd_kernel(BwdArgs a) {
         mma_commit(&mbar);
       }
       // incoming gradient of this slice while the MMA runs
+      if (valid && MODE == M_EENC) {
+        ld_g16(g0, a.dY1h + row * kH + c0);
+      } else if (valid) {
+        ld_g32(g0, a.dY1 + row * kH + c0);
+      } else {
 #pragma unroll
-      for (int j = 0; j < 32; ++j) g0[j] = 0.f;
-      if (valid) {
-        const int64_t r2 = a.idx2 ? int64_t(a.idx2[row]) : row;
-        if (a.dY1) add_g32(g0, a.dY1 + row * kH + c0);
-        if (a.dY1h) add_g16(g0, a.dY1h + row * kH + c0);
-        if (a.dY2) add_g32(g0, a.dY2 + r2 * kH + c0);
-        if (a.dY2h) add_g16(g0, a.dY2h + r2 * kH + c0);
+        for (int j = 0; j < 32; ++j) g0[j] = 0.f;
       }
       // the node update's residual passes the same gradient on: it waits in
       // TMEM columns the node MLP leaves free (no weight gradients there)
@@ -1218,7 +1209,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_bwd_kernel(BwdArgs a) {
       tmem_ld32(tm + lane_base + tZ2 + c0, v);
       tmem_ld32(tm + lane_base + tZ1 + c0, z);
 #pragma unroll
-      for (int j = 0; j < 32; ++j) v[j] = valid ? v[j] * z[j] : 0.f;  // z holds SiLU'(Z1)
+      for (int j = 0; j < 32; ++j) v[j] *= z[j];  // z holds SiLU'(Z1); rows past the end: dY and so dA1 are 0
       st_tile32(sm.a1, 128, r, c0, v);
       cacc[0] += col_reduce32(v);
     }
@@ -1341,20 +1332,6 @@ __host__ __device__ __forceinline__ uint32_t carve_edge_bwd(const MlpImgs& w, Ed
   return o;
 }
 
-// cp.async of rows r0..r0+127 of a row-major [rows, 128] bf16 array into a
-// swizzled tile (rows past the end, or a null source, read as zeros).
-__device__ __forceinline__ void issue_rows16(uint8_t* tile, const bf16* src, int64_t rows, int64_t r0, int tid) {
-  for (int q = tid; q < 128 * 16; q += kThreads) {
-    const int r = q >> 4, j = q & 15;
-    if (!src) {  // no source: plain zero stores, no copy is issued
-      *reinterpret_cast<uint4*>(tile + sw_chunk(128, r, j)) = make_uint4(0u, 0u, 0u, 0u);
-      continue;
-    }
-    const bool ok = r0 + r < rows;
-    cp_async16(tile + sw_chunk(128, r, j), ok ? src + (r0 + r) * kH + 8 * j : src, ok ? 16u : 0u);
-  }
-}
-
 // cp.async of the node-projection rows P[idx[k]] (the 128 columns from `off`
 // on) of one 128-edge tile into a swizzled tile; idx[k] < 0 reads zeros.
 __device__ __forceinline__ void issue_gather16(uint8_t* tile, const bf16* P, const int32_t* idx, int off, int tid) {
@@ -1467,7 +1444,7 @@ __global__ void __launch_bounds__(kThreads, 1) edge_bwd_kernel(BwdArgs a, const 
       tc_fence_after();
       const uint32_t xs = smem_u32(sm.xe), ws = smem_u32(sm.w1);
       if (ok) {
-mma_chain<kH / 16, 128, false, kH, false>(tm + tZ1, xs, ws, id_f, false);
+        mma_chain<kH / 16, 128, false, kH, false>(tm + tZ1, xs, ws, id_f, false);
       }
       mma_commit(&mbar);
     }
@@ -1503,13 +1480,16 @@ mma_chain<kH / 16, 128, false, kH, false>(tm + tZ1, xs, ws, id_f, false);
     if (tid == 0) {
       tc_fence_after();
       const uint32_t as = smem_u32(sm.a1), ws = smem_u32(sm.w2);
-mma_chain<kH / 16, 128, false, kH, false>(tm + tZ2, as, ws, id_f, false);
+      mma_chain<kH / 16, 128, false, kH, false>(tm + tZ2, as, ws, id_f, false);
       mma_commit(&mbar);
     }
     // incoming gradient dm = de + da[receiver] while the MMA runs
+    if (valid && a.dY2h) {
+      ld_g16(g0, a.dY2h + rcv * kH + c0);
+    } else {
 #pragma unroll
-    for (int j = 0; j < 32; ++j) g0[j] = 0.f;
-    if (valid && a.dY2h) add_g16(g0, a.dY2h + rcv * kH + c0);
+      for (int j = 0; j < 32; ++j) g0[j] = 0.f;
+    }
     bool dok = true;
     if (has_de) {
       dok = mbar_wait(&dbar, dph, a.err);  // the gradient tile
@@ -1563,8 +1543,8 @@ mma_chain<kH / 16, 128, false, kH, false>(tm + tZ2, as, ws, id_f, false);
     if (tid == 0) {
       tc_fence_after();
       const uint32_t ds = smem_u32(sm.dz2), ws = smem_u32(sm.w2), as = smem_u32(sm.a1);
-mma_chain<kH / 16, 128, false, kH, true>(tm + tZ2, ds, ws, id_t, false);
-mma_chain<8, 128, true, 128, true>(tm + tW2, as, ds, id_w, !first);
+      mma_chain<kH / 16, 128, false, kH, true>(tm + tZ2, ds, ws, id_t, false);
+      mma_chain<8, 128, true, 128, true>(tm + tW2, as, ds, id_w, !first);
       mma_commit(&mbar);
     }
     ok = mbar_wait(&mbar, ph, a.err);
@@ -1583,7 +1563,7 @@ mma_chain<8, 128, true, 128, true>(tm + tW2, as, ds, id_w, !first);
       tmem_ld32(tm + lane_base + tZ2 + c0, v);
       tmem_ld32(tm + lane_base + tZ1 + c0, z);
 #pragma unroll
-      for (int j = 0; j < 32; ++j) v[j] = valid ? v[j] * z[j] : 0.f;  // z holds SiLU'(Z1)
+      for (int j = 0; j < 32; ++j) v[j] *= z[j];  // z holds SiLU'(Z1); rows past the end: dA1 = 0, as da, de and so dZ2 are
       st_tile32(sm.a1, 128, r, c0, v);
     }
     fence_proxy_async();
@@ -1593,8 +1573,8 @@ mma_chain<8, 128, true, 128, true>(tm + tW2, as, ds, id_w, !first);
     if (tid == 0) {
       tc_fence_after();
       const uint32_t ds = smem_u32(sm.a1), ws = smem_u32(sm.w1), xs = smem_u32(sm.xe);
-mma_chain<kH / 16, 128, false, kH, true>(tm + tDX, ds, ws, id_t, false);
-mma_chain<8, 128, true, 128, true>(tm + tW1, xs, ds, id_w, !first);
+      mma_chain<kH / 16, 128, false, kH, true>(tm + tDX, ds, ws, id_t, false);
+      mma_chain<8, 128, true, 128, true>(tm + tW1, xs, ds, id_w, !first);
       mma_commit(&mbar);
     }
     if (tma_thread) {
@@ -1854,7 +1834,7 @@ __global__ void __launch_bounds__(kT32, 1) edge_bwd32_kernel(BwdArgs a, const __
       tc_fence_after();
       const uint32_t xs = smem_u32(sm.xe), ws = smem_u32(sm.w1);
       if (ok) {
-mma_chain<kH / 16, 128, false, kH, false>(tm + tZ1, xs, ws, id_f, false);
+        mma_chain<kH / 16, 128, false, kH, false>(tm + tZ1, xs, ws, id_f, false);
       }
       mma_commit(&mbar);
     }
@@ -1889,7 +1869,7 @@ mma_chain<kH / 16, 128, false, kH, false>(tm + tZ1, xs, ws, id_f, false);
     if (tid == 0) {
       tc_fence_after();
       const uint32_t as = smem_u32(sm.a1), ws = smem_u32(sm.w2);
-mma_chain<kH / 16, 128, false, kH, false>(tm + tZ2, as, ws, id_f, false);
+      mma_chain<kH / 16, 128, false, kH, false>(tm + tZ2, as, ws, id_f, false);
       mma_commit(&mbar);
     }
 #pragma unroll
@@ -1948,8 +1928,8 @@ mma_chain<kH / 16, 128, false, kH, false>(tm + tZ2, as, ws, id_f, false);
     if (tid == 0) {
       tc_fence_after();
       const uint32_t ds = smem_u32(sm.dz2), ws = smem_u32(sm.w2), as = smem_u32(sm.a1);
-mma_chain<kH / 16, 128, false, kH, true>(tm + tZ2, ds, ws, id_t, false);
-mma_chain<8, 128, true, 128, true>(tm + tW2, as, ds, id_w, !first);
+      mma_chain<kH / 16, 128, false, kH, true>(tm + tZ2, ds, ws, id_t, false);
+      mma_chain<8, 128, true, 128, true>(tm + tW2, as, ds, id_w, !first);
       mma_commit(&mbar);
     }
     ok = mbar_wait(&mbar, ph, a.err);
@@ -1977,8 +1957,8 @@ mma_chain<8, 128, true, 128, true>(tm + tW2, as, ds, id_w, !first);
     if (tid == 0) {
       tc_fence_after();
       const uint32_t ds = smem_u32(sm.a1), ws = smem_u32(sm.w1), xs = smem_u32(sm.xe);
-mma_chain<kH / 16, 128, false, kH, true>(tm + tDX, ds, ws, id_t, false);
-mma_chain<8, 128, true, 128, true>(tm + tW1, xs, ds, id_w, !first);
+      mma_chain<kH / 16, 128, false, kH, true>(tm + tDX, ds, ws, id_t, false);
+      mma_chain<8, 128, true, 128, true>(tm + tW1, xs, ds, id_w, !first);
       mma_commit(&mbar);
     }
     if (tma_thread) {
@@ -2201,7 +2181,7 @@ __global__ void __launch_bounds__(kThreads, 1) edge_bwd2_kernel(BwdArgs a) {
     if (gt == 0) {
       tc_fence_after();
       const uint32_t xs = smem_u32(T1), ws = smem_u32(sm.w1);
-mma_chain<kH / 16, 128, false, kH, false>(R, xs, ws, id_f, false);
+      mma_chain<kH / 16, 128, false, kH, false>(R, xs, ws, id_f, false);
       mma_commit(&mb[g]);
     }
     uint32_t pr[16], ps[16];  // 32 bf16 node projections each, packed
@@ -2247,7 +2227,7 @@ mma_chain<kH / 16, 128, false, kH, false>(R, xs, ws, id_f, false);
     if (gt == 0) {
       tc_fence_after();
       const uint32_t as = smem_u32(T2), ws = smem_u32(sm.w2);
-mma_chain<kH / 16, 128, false, kH, false>(R, as, ws, id_f, false);
+      mma_chain<kH / 16, 128, false, kH, false>(R, as, ws, id_f, false);
       mma_commit(&mb[g]);
     }
     gok = group_all(g, mbar_wait(&mb[g], ph, a.err));
@@ -2337,11 +2317,11 @@ mma_chain<kH / 16, 128, false, kH, false>(R, as, ws, id_f, false);
     if (gt == 0) {
       tc_fence_after();
       const uint32_t ds = smem_u32(T1), ws = smem_u32(sm.w2), as = smem_u32(T2);
-mma_chain<kH / 16, 128, false, kH, true>(R, ds, ws, id_t, false);
+      mma_chain<kH / 16, 128, false, kH, true>(R, ds, ws, id_t, false);
       lok = token_wait(&tok[0], int32_t(j), a.err);
       if (lok) {
         tc_fence_after();
-mma_chain<8, 128, true, 128, true>(tW2, as, ds, id_w, !(j == 0));
+        mma_chain<8, 128, true, 128, true>(tW2, as, ds, id_w, !(j == 0));
       }
       mma_commit(&mb[g]);
       if (lok) {
@@ -2380,11 +2360,11 @@ mma_chain<8, 128, true, 128, true>(tW2, as, ds, id_w, !(j == 0));
     if (gt == 0) {
       tc_fence_after();
       const uint32_t ds = smem_u32(T2), ws = smem_u32(sm.w1), xs = smem_u32(T1);
-mma_chain<kH / 16, 128, false, kH, true>(R, ds, ws, id_t, false);
+      mma_chain<kH / 16, 128, false, kH, true>(R, ds, ws, id_t, false);
       lok = token_wait(&tok[1], int32_t(j), a.err);
       if (lok) {
         tc_fence_after();
-mma_chain<8, 128, true, 128, true>(tW1, xs, ds, id_w, !(j == 0));
+        mma_chain<8, 128, true, 128, true>(tW1, xs, ds, id_w, !(j == 0));
       }
       mma_commit(&mb[g]);
       if (lok) {

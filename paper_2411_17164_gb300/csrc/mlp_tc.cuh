@@ -72,13 +72,11 @@ struct BwdArgs {
   const bf16* P;  // EDGE: as in FwdArgs
   MlpImgs w;
   MlpParams p;
-  // incoming gradient dY = dY1[row] + dY2[idx2[row]]; each given either as
-  // fp32 (dY*) or bf16 (dY*h), the other pointer null
+  // incoming gradient of row r: dY1[r] in fp32 or dY1h[r] in bf16, and for the
+  // edge update the receiver's dY2h[recv[r]] with it
   const float* dY1;  // NODE: dh; DEC: dy [rows, out]; NENC: dh
-  const bf16* dY1h;  // EDGE, EENC: de (edge-state gradient, bf16; null = 0)
-  const float* dY2;
+  const bf16* dY1h;  // EDGE, EENC: de (edge-state gradient, bf16; EDGE: null = 0)
   const bf16* dY2h;  // EDGE: d a (aggregated-message gradient, bf16)
-  const int32_t* idx2;
   // outputs
   float* dX0;   // NODE: dh_out (= dY1 + dX_h); DEC: dh
   bf16* dX0h;   // EDGE: de_out (= dY1 + dX_e, may alias dY1h)

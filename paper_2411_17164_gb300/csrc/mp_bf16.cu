@@ -695,7 +695,6 @@ xmgn_status bf16_backward(const ParamPlan& p, const float* P, const xmgn_graph& 
     be.p = params_of(P, oe);
     be.dY1h = l + 1 < p.L ? w.de : nullptr;  // nothing reads the top layer's edge output
     be.dY2h = w.dagg;
-    be.idx2 = g.recv;
     be.dX0h = w.de;
     if (off) XMGN_CUDA(cudaStreamWaitEvent(s, oc->moved[l % kRing], 0));
     XMGN_TRY(mlp_bwd_tc(M_EDGE, be, s));
