@@ -387,9 +387,10 @@ __global__ void sym_rev_kernel(const int32_t* __restrict__ nbr, int64_t n, int k
 // end: apart, the halves would take turns); longer ones, points that many
 // others list, are sorted on the global arrays.  out row i starts at rstart[i]
 // + K i.  Bound by the latency of the row's reads; 1.25M rows of 21 slots: 1216
-// us (a thread per row, insertion sort in global memory) -> 415 us.
+// us (a thread per row, insertion sort in global memory) -> 415 us, and 12 us
+// less with six blocks per SM (40 registers, nothing spilled) instead of five.
 constexpr int kRow = 64;
-__global__ void __launch_bounds__(256) sym_sort_kernel(const int32_t* __restrict__ nbr, int64_t n, int k,
+__global__ void __launch_bounds__(256, 6) sym_sort_kernel(const int32_t* __restrict__ nbr, int64_t n, int k,
                                                        const int64_t* __restrict__ rstart,
                                                        const int32_t* __restrict__ rev, int32_t* __restrict__ out,
                                                        int32_t* __restrict__ deg) {
