@@ -283,16 +283,21 @@ struct Claims {
     if (k < kFound) found[k] = key;
     else store(out + atomicAdd(cnt, 1ull), key);  // a step of many long rows: straight to the list
   }
-  // By all threads of the block, after every add.
+  // By all threads of the block, after every add.  No thread passes the second
+  // barrier, and so claims for the next step, before every thread has read the
+  // count: with the barriers only where there is something to store, a thread
+  // held back would read a claim of the next step and wait in them alone.
   __device__ __forceinline__ void flush() const {
     __syncthreads();
     const int k = *nfound < kFound ? *nfound : kFound;
-    if (k > 0) {  // uniform
-      if (threadIdx.x == 0) *pos0 = out + atomicAdd(cnt, (unsigned long long)k);
+    __syncthreads();
+    if (k > 0) {  // the same in every thread
+      if (threadIdx.x == 0) {
+        *pos0 = out + atomicAdd(cnt, (unsigned long long)k);
+        *nfound = 0;
+      }
       __syncthreads();
       for (int i = threadIdx.x; i < k; i += blockDim.x) store(*pos0 + i, found[i]);
-      __syncthreads();
-      if (threadIdx.x == 0) *nfound = 0;
       __syncthreads();
     }
   }
