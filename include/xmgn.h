@@ -73,7 +73,8 @@ xmgn_status xmgn_check_device(xmgn_stream stream);
  * (round half to even, s = lattice_scale, a power of two, default 2^21) and
  * compared by the int64 squared distance; ties go to the smaller index; a
  * point is never its own neighbour; coincident points are allowed.  |q| must
- * stay below 2^24 (|x| < 8 at the default scale), else XMGN_ERR_RANGE.
+ * stay below 2^24 (|x| < 8 at the default scale), else XMGN_ERR_RANGE with no
+ * output written.
  *
  * The kNN relation is then symmetrised (edge (i <- j) iff j in kNN(i) or
  * i in kNN(j), no duplicates) and emitted as receiver-major CSR with senders

@@ -104,9 +104,11 @@ inline unsigned grid_for(int64_t n, int threads, int64_t cap_blocks = 0) {
 
 // ---------------------------------------------------------------- scans
 // Exclusive prefix sum of n int32 values into int64 or int32 out[0..n]
-// (out[n] = total).  Uses `tmp` scratch of scan_tmp_elems(n) int64.
+// (out[n] = total).  Uses `tmp` scratch of scan_tmp_elems(n) int64.  When a
+// device flag `skip` is given and set (and n > 0), out is left as it is.
 size_t scan_tmp_elems(int64_t n);
-xmgn_status exclusive_scan_i32(const int32_t* in, int64_t* out, int64_t n, int64_t* tmp, cudaStream_t s);
+xmgn_status exclusive_scan_i32(const int32_t* in, int64_t* out, int64_t n, int64_t* tmp, cudaStream_t s,
+                               const int32_t* skip = nullptr);
 xmgn_status exclusive_scan_i32(const int32_t* in, int32_t* out, int64_t n, int64_t* tmp, cudaStream_t s);
 
 // ---------------------------------------------------------------- launches

@@ -18,6 +18,10 @@
 // The whole build runs on the stream with one host wait at its end: the grid
 // is laid out on the device from the bounding box, and the rows are emitted
 // only if they fit the caller's capacity, which the host reports afterwards.
+// A coordinate off the lattice ends the work at once all the same: it sets a
+// flag of the call (bbox[6]), and every later kernel leaves when it is set, so
+// that no time goes into a cloud whose points have fallen together and no
+// output array is touched.
 #include <math.h>
 
 #include "common.cuh"
@@ -27,6 +31,7 @@ namespace xmgn {
 namespace {
 constexpr int kMaxK = 32;
 
+// bbox: least and greatest lattice coordinate per axis, [6]: a coordinate is off the lattice.
 __global__ void quantize_kernel(const float* __restrict__ xyz, int64_t n, float scale,
                                 int32_t* __restrict__ q, int32_t* __restrict__ bbox,
                                 uint32_t* err) {
@@ -41,6 +46,7 @@ __global__ void quantize_kernel(const float* __restrict__ xyz, int64_t n, float 
       int32_t qi = 0;
       if (!(fabsf(v) < 16777216.0f)) {  // also catches NaN / inf
         dev_flag(err, DEV_ERR_RANGE);
+        bbox[6] = 1;
       } else {
         qi = int32_t(v);
       }
@@ -73,6 +79,8 @@ __global__ void bbox_init_kernel(int32_t* bbox) {
   if (threadIdx.x < 3) {
     bbox[threadIdx.x] = INT32_MAX;
     bbox[3 + threadIdx.x] = INT32_MIN;
+  } else if (threadIdx.x == 3) {
+    bbox[6] = 0;
   }
 }
 
@@ -81,6 +89,7 @@ struct Grid {
   int32_t lo[3];
   int32_t c;     // cell edge in lattice units
   int32_t g[3];  // cells per axis
+  int32_t bad;   // bbox[6]
 };
 constexpr int kMaxLevels = 16;
 struct LevelSizes {
@@ -103,11 +112,16 @@ __host__ __device__ inline int64_t cell_budget(int64_t n) {
 
 // The grid of every level (thread l: the first sizes.n[l] points) over the box
 // of all points: at most cell_budget cells.
-__global__ void grid_layout_kernel(const int32_t* __restrict__ bbox, LevelSizes sizes, int levels, Grid* __restrict__ out) {
+// A range error that the device's error word holds already counts as this
+// call's, as the host reports it.
+__global__ void grid_layout_kernel(int32_t* bbox, LevelSizes sizes, int levels, const uint32_t* __restrict__ err,
+                                   Grid* __restrict__ out) {
   pdl_wait();
   pdl_trigger();
   const int l = threadIdx.x;
   if (l >= levels) return;
+  const int32_t bad = (bbox[6] != 0 || (*err & DEV_ERR_RANGE)) ? 1 : 0;
+  if (l == 0) bbox[6] = bad;
   const int64_t budget = cell_budget(sizes.n[l]);
   double vol = 1.0;
   Grid G;
@@ -129,6 +143,7 @@ __global__ void grid_layout_kernel(const int32_t* __restrict__ bbox, LevelSizes 
     e = e + e / 4 + 1;
   }
   G.c = int32_t(e);
+  G.bad = bad;
   out[l] = G;
 }
 
@@ -140,6 +155,7 @@ __global__ void cell_count_kernel(const int32_t* __restrict__ q, int64_t n, cons
   pdl_wait();
   pdl_trigger();
   const Grid G = *grid;
+  if (G.bad) return;
   for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n;
        i += int64_t(gridDim.x) * blockDim.x) {
     const int cx = cell_coord(q[3 * i], G.lo[0], G.c);
@@ -153,9 +169,10 @@ __global__ void cell_count_kernel(const int32_t* __restrict__ q, int64_t n, cons
 
 __global__ void cell_scatter_kernel(const int32_t* __restrict__ q, const int32_t* __restrict__ cell_of,
                                     const int32_t* __restrict__ at, int64_t n, const int32_t* __restrict__ start,
-                                    int4* __restrict__ pts) {
+                                    const Grid* __restrict__ grid, int4* __restrict__ pts) {
   pdl_wait();
   pdl_trigger();
+  if (grid->bad) return;
   for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n;
        i += int64_t(gridDim.x) * blockDim.x)
     pts[start[cell_of[i]] + at[i]] = make_int4(q[3 * i], q[3 * i + 1], q[3 * i + 2], int32_t(i));
@@ -225,6 +242,7 @@ __global__ void __launch_bounds__(128) knn_kernel(const int32_t* __restrict__ q,
   pdl_wait();
   pdl_trigger();
   const Grid gr = *grid;
+  if (gr.bad) return;
   const int lane = threadIdx.x & 31, gl = lane % G;
   const uint32_t mask = G == 1 ? 0u : ((G == 32 ? 0xffffffffu : ((1u << G) - 1u)) << (lane - gl));
   for (int64_t t = q0 + (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) / G; t < q1;
@@ -364,14 +382,24 @@ xmgn_status knn_launch(const int32_t* q, const int4* pts, const int32_t* start, 
   return XMGN_OK;
 }
 
+__global__ void empty_slots_kernel(int32_t* __restrict__ nbr, int64_t slots, const int32_t* __restrict__ bad) {
+  pdl_wait();
+  pdl_trigger();
+  if (*bad) return;
+  for (int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; t < slots; t += int64_t(gridDim.x) * blockDim.x)
+    nbr[t] = -1;
+}
+
 // ---- symmetrisation
 // Row i of the undirected graph = its own K slots and every j that lists i.
 // Reverse entries: slot t of point i names j = nbr[t]; i goes to place rank[t]
 // of j's list.
 __global__ void sym_rev_kernel(const int32_t* __restrict__ nbr, int64_t n, int k, const int64_t* __restrict__ rstart,
-                               const int32_t* __restrict__ rank, int32_t* __restrict__ rev) {
+                               const int32_t* __restrict__ rank, const int32_t* __restrict__ bad,
+                               int32_t* __restrict__ rev) {
   pdl_wait();
   pdl_trigger();
+  if (*bad) return;
   for (int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; t < n * k;
        t += int64_t(gridDim.x) * blockDim.x) {
     const int32_t j = nbr[t];
@@ -392,10 +420,12 @@ __global__ void sym_rev_kernel(const int32_t* __restrict__ nbr, int64_t n, int k
 constexpr int kRow = 64;
 __global__ void __launch_bounds__(256, 6) sym_sort_kernel(const int32_t* __restrict__ nbr, int64_t n, int k,
                                                        const int64_t* __restrict__ rstart,
-                                                       const int32_t* __restrict__ rev, int32_t* __restrict__ out,
+                                                       const int32_t* __restrict__ rev,
+                                                       const int32_t* __restrict__ bad, int32_t* __restrict__ out,
                                                        int32_t* __restrict__ deg) {
   pdl_wait();
   pdl_trigger();
+  if (*bad) return;
   __shared__ __align__(16) int32_t raw[16][kRow], srt[16][kRow];
   const int lane = threadIdx.x & 31, l = lane & 15, gi = threadIdx.x >> 4, hs = lane & 16;
   constexpr uint32_t kAll = 0xffffffffu;
@@ -481,18 +511,20 @@ __global__ void __launch_bounds__(256, 6) sym_sort_kernel(const int32_t* __restr
 }
 
 // Copies the sorted rows to their CSR places, 8 lanes per row; nothing is
-// written when the edges exceed the caller's capacity.
+// written when the edges exceed the caller's capacity or a coordinate is bad.
 __global__ void sym_emit_kernel(const int32_t* __restrict__ rows, const int64_t* __restrict__ rstart, int k,
                                 const int64_t* __restrict__ row_ptr, int64_t n, int64_t cap,
                                 int32_t* __restrict__ col, int32_t* __restrict__ recv,
-                                const uint32_t* __restrict__ err, int64_t* __restrict__ info) {
+                                const uint32_t* __restrict__ err, const int32_t* __restrict__ bad,
+                                int64_t* __restrict__ info) {
   pdl_wait();
   pdl_trigger();
+  const bool stop = *bad != 0;
   if (blockIdx.x == 0 && threadIdx.x == 0) {  // what the host reads at the end, in one copy
-    info[0] = row_ptr[n];
-    info[1] = int64_t(*err);
+    info[0] = stop ? 0 : row_ptr[n];
+    info[1] = int64_t(*err) | (stop ? int64_t(DEV_ERR_RANGE) : 0);
   }
-  if (row_ptr[n] > cap) return;
+  if (stop || row_ptr[n] > cap) return;
   const int l = threadIdx.x & 7;
   for (int64_t i = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 3; i < n;
        i += (int64_t(gridDim.x) * blockDim.x) >> 3) {
@@ -522,16 +554,19 @@ xmgn_status quantize_launch(const float* xyz, int64_t n, double scale, int32_t* 
 // keeps four edges in flight and reads rows of up to 8 edges whole; longer
 // rows are searched by key (their senders' ids, or global ids, ascend).  17.2M
 // edges of a 2M-point batch: 123 us (a binary search by key per thread) -> 98 us.
-// e < 0: the edge count is row_ptr[n], and nothing is written if it exceeds cap.
+// e < 0: the edge count is row_ptr[n], and nothing is written if it exceeds cap
+// or *bad is set.
 constexpr int kPermEdges = 4;
 __global__ void __launch_bounds__(256) csc_perm_kernel(const int64_t* __restrict__ row_ptr,
                                                        const int32_t* __restrict__ col,
                                                        const int32_t* __restrict__ recv,
                                                        const int32_t* __restrict__ key, int64_t n, int64_t e,
-                                                       int64_t cap, int32_t* __restrict__ perm, uint32_t* err) {
+                                                       int64_t cap, const int32_t* __restrict__ bad,
+                                                       int32_t* __restrict__ perm, uint32_t* err) {
   pdl_wait();
   pdl_trigger();
   if (e < 0) {
+    if (*bad) return;
     e = row_ptr[n];
     if (e > cap) return;
   }
@@ -618,7 +653,7 @@ static void knn_layout(int64_t N, int32_t K, Arena& A, KnnWs& w) {
 static xmgn_status quantize_all(const float* xyz, int64_t N, double scale, const LevelSizes& sizes, int levels,
                                 KnnWs& w, uint32_t* err, cudaStream_t s) {
   XMGN_TRY(quantize_launch(xyz, N, scale, w.q, w.bbox, err, s));
-  launch_pdl(grid_layout_kernel, 1, 32, 0, s, w.bbox, sizes, levels, w.grid);
+  launch_pdl(grid_layout_kernel, 1, 32, 0, s, w.bbox, sizes, levels, err, w.grid);
   XMGN_LAUNCH_CHECK();
   XMGN_CUDA(cudaMemsetAsync(w.rcnt, 0, sizeof(int32_t) * size_t(N), s));
   return XMGN_OK;
@@ -631,7 +666,8 @@ static xmgn_status grid_sort(int64_t n_ref, const Grid* grid, KnnWs& w, cudaStre
   launch_pdl(cell_count_kernel, grid_for(n_ref, 256), 256, 0, s, w.q, n_ref, grid, w.cell_of, w.at, w.cnt);
   XMGN_LAUNCH_CHECK();
   XMGN_TRY(exclusive_scan_i32(w.cnt, w.cstart, cells, w.scan_tmp, s));
-  launch_pdl(cell_scatter_kernel, grid_for(n_ref, 256), 256, 0, s, w.q, w.cell_of, w.at, n_ref, w.cstart, w.pts);
+  launch_pdl(cell_scatter_kernel, grid_for(n_ref, 256), 256, 0, s, w.q, w.cell_of, w.at, n_ref, w.cstart, grid,
+             w.pts);
   XMGN_LAUNCH_CHECK();
   return XMGN_OK;
 }
@@ -642,18 +678,21 @@ static xmgn_status grid_sort(int64_t n_ref, const Grid* grid, KnnWs& w, cudaStre
 static xmgn_status symmetrise_slots(int64_t N, int32_t K, KnnWs& w, int64_t* row_ptr, int32_t* col,
                                     int32_t* recv, int32_t* csc_perm, int64_t E_cap, int64_t* E_out,
                                     uint32_t* err, cudaStream_t s) {
+  const int32_t* bad = w.bbox + 6;
   XMGN_TRY(exclusive_scan_i32(w.rcnt, w.rstart, N, w.scan_tmp, s));
-  launch_pdl(sym_rev_kernel, grid_for(N * K, 256), 256, 0, s, w.nbr, N, K, w.rstart, w.rank, w.rev);
+  launch_pdl(sym_rev_kernel, grid_for(N * K, 256), 256, 0, s, w.nbr, N, K, w.rstart, w.rank, bad, w.rev);
   XMGN_LAUNCH_CHECK();
-  launch_pdl(sym_sort_kernel, grid_for(N * 16, 256), 256, 0, s, w.nbr, N, K, w.rstart, w.rev, w.rows, w.deg);
+  launch_pdl(sym_sort_kernel, grid_for(N * 16, 256), 256, 0, s, w.nbr, N, K, w.rstart, w.rev, bad, w.rows,
+             w.deg);
   XMGN_LAUNCH_CHECK();
-  XMGN_TRY(exclusive_scan_i32(w.deg, row_ptr, N, w.scan_tmp, s));
-  launch_pdl(sym_emit_kernel, grid_for(N * 8, 256), 256, 0, s, w.rows, w.rstart, K, row_ptr, N, E_cap, col, recv, err, w.info);
+  XMGN_TRY(exclusive_scan_i32(w.deg, row_ptr, N, w.scan_tmp, s, bad));
+  launch_pdl(sym_emit_kernel, grid_for(N * 8, 256), 256, 0, s, w.rows, w.rstart, K, row_ptr, N, E_cap, col, recv, err,
+             bad, w.info);
   XMGN_LAUNCH_CHECK();
   if (csc_perm) {
     const int64_t most = 2 * N * K < E_cap ? 2 * N * K : E_cap;
-    launch_pdl(csc_perm_kernel, grid_for((most + kPermEdges - 1) / kPermEdges, 256), 256, 0, s, row_ptr, col, recv, nullptr, N,
-                                                                                        -1, E_cap, csc_perm, err);
+    launch_pdl(csc_perm_kernel, grid_for((most + kPermEdges - 1) / kPermEdges, 256), 256, 0, s, row_ptr, col, recv,
+               nullptr, N, -1, E_cap, bad, csc_perm, err);
     XMGN_LAUNCH_CHECK();
   }
   int64_t info[2];
@@ -757,7 +796,8 @@ xmgn_status build_multiscale(const float* xyz, int64_t N, const int64_t* sizes, 
   LevelSizes ls{};
   for (int l = 0; l < n_levels; ++l) ls.n[l] = sizes[l];
   XMGN_TRY(quantize_all(xyz, N, scale, ls, n_levels, w, err, s));
-  XMGN_CUDA(cudaMemsetAsync(w.nbr, 0xff, sizeof(int32_t) * size_t(N) * K, s));  // all slots empty (-1)
+  launch_pdl(empty_slots_kernel, grid_for(N * K, 256, int64_t(num_sms()) * 8), 256, 0, s, w.nbr, N * K, w.bbox + 6);
+  XMGN_LAUNCH_CHECK();
   for (int l = 0; l < n_levels; ++l) {
     // kNN within level l (the first sizes[l] points): slots [l*k, l*k + k)
     XMGN_TRY(grid_sort(sizes[l], w.grid + l, w, s));

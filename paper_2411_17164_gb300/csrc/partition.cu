@@ -32,7 +32,8 @@ namespace xmgn {
 
 __global__ void csc_perm_kernel(const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
                                 const int32_t* __restrict__ recv, const int32_t* __restrict__ key,
-                                int64_t n, int64_t e, int64_t cap, int32_t* __restrict__ perm, uint32_t* err);
+                                int64_t n, int64_t e, int64_t cap, const int32_t* __restrict__ bad,
+                                int32_t* __restrict__ perm, uint32_t* err);
 xmgn_status quantize_launch(const float* xyz, int64_t n, double scale, int32_t* q, int32_t* bbox,
                             uint32_t* err, cudaStream_t s);
 
@@ -630,7 +631,7 @@ __global__ void __launch_bounds__(256) batch_edges_kernel(const uint64_t* __rest
 struct PartLayout {
   int32_t* q;
   int32_t* bbox;
-  int32_t* part;       // part ids when the caller gives no part array
+  int32_t* part;       // part ids of the bisection
   int32_t* seg;        // bisection segment of each node
   int32_t* ext[2];     // 6 per segment, of this level and the next
   RcbSeg* plan;        // all levels
@@ -816,7 +817,7 @@ xmgn_status partition_halo(const int64_t* row_ptr, const int32_t* col, int64_t N
   part_layout(A, N, P, w);
   if (!A.ok()) return fail(XMGN_ERR_WORKSPACE, "partition workspace too small: need %zu", A.used);
   uint32_t* err = device_error_word();
-  int32_t* part = part_out ? part_out : w.part;
+  const int32_t* part = part_in ? part_in : w.part;
   const int64_t words = (N + 31) / 32;
   // edges and the CSC permutation, once ids and row offsets are in place
   auto emit_edges = [&](int64_t nb, int64_t eb) -> xmgn_status {
@@ -826,7 +827,8 @@ xmgn_status partition_halo(const int64_t* row_ptr, const int32_t* col, int64_t N
       XMGN_LAUNCH_CHECK();
     }
     if (b_csc_perm && eb > 0) {
-      launch_pdl(csc_perm_kernel, grid_for((eb + 3) / 4, 256), 256, 0, s, b_row_ptr, b_col, b_recv, gid, nb, eb, eb, b_csc_perm, err);
+      launch_pdl(csc_perm_kernel, grid_for((eb + 3) / 4, 256), 256, 0, s, b_row_ptr, b_col, b_recv, gid, nb, eb, eb,
+                 nullptr, b_csc_perm, err);
       XMGN_LAUNCH_CHECK();
     }
     XMGN_CUDA(cudaMemsetAsync(w.stamp, 0, sizeof(int64_t) * 8, s));  // one emit per sizing pass
@@ -854,12 +856,7 @@ xmgn_status partition_halo(const int64_t* row_ptr, const int32_t* col, int64_t N
 
   XMGN_CUDA(cudaMemsetAsync(w.stamp, 0, sizeof(int64_t) * 8, s));  // this pass replaces what an earlier one left
   // ---------------- parts
-  if (part_in) {
-    if (part != part_in)
-      XMGN_CUDA(cudaMemcpyAsync(part, part_in, sizeof(int32_t) * size_t(N), cudaMemcpyDeviceToDevice, s));
-  } else {
-    XMGN_TRY(bisect(xyz, N, scale, P, w, part, err, s));
-  }
+  if (!part_in) XMGN_TRY(bisect(xyz, N, scale, P, w, w.part, err, s));
 
   // ---------------- halo BFS
   XMGN_CUDA(cudaMemsetAsync(w.bits, 0, sizeof(uint32_t) * size_t(int64_t(P) * words), s));
@@ -896,6 +893,8 @@ xmgn_status partition_halo(const int64_t* row_ptr, const int32_t* col, int64_t N
     if (herr & DEV_ERR_GRAPH) return fail(XMGN_ERR_GRAPH, "part id or sender id out of range");
     return fail(XMGN_ERR_WORKSPACE, "halo members exceed the workspace capacity (%lld)", (long long)w.cap);
   }
+  if (part_out && part_out != part)  // only now: bad coordinates or ids leave it alone
+    XMGN_CUDA(cudaMemcpyAsync(part_out, part, sizeof(int32_t) * size_t(N), cudaMemcpyDeviceToDevice, s));
   if (emit && cap_nodes < nb) return fail(XMGN_ERR_WORKSPACE, "cap_nodes %lld < %lld", (long long)cap_nodes, (long long)nb);
   for (int p = 0; p <= P; ++p) node_ptr[p] = info[2 + p];
   for (int p = 0; p < P; ++p) inner_cnt[p] = info[3 + P + p];

@@ -56,13 +56,15 @@ __global__ void __launch_bounds__(kScanThreads) tile_sum_kernel(const T* __restr
 }
 
 // Scan of tile blockIdx.x.  sums: null (a single tile), the tile sums, or
-// (scanned) their exclusive prefix.  The last tile also writes out[n].
+// (scanned) their exclusive prefix.  The last tile also writes out[n].  Nothing
+// is written when `skip` is given and set.
 template <class T, class O>
 __global__ void __launch_bounds__(kScanThreads) tile_scan_kernel(const T* __restrict__ in, O* __restrict__ out,
                                                                  int64_t n, const int64_t* __restrict__ sums,
-                                                                 int scanned) {
+                                                                 int scanned, const int32_t* __restrict__ skip) {
   pdl_wait();
   pdl_trigger();
+  if (skip && *skip) return;
   __shared__ int64_t red[kScanThreads / 32];
   __shared__ int64_t tile[kScanTile + kScanTile / kScanItems];
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
@@ -110,7 +112,7 @@ __global__ void __launch_bounds__(kScanThreads) tile_scan_kernel(const T* __rest
 }
 
 template <class T, class O>
-xmgn_status scan_impl(const T* in, O* out, int64_t n, int64_t* tmp, cudaStream_t s) {
+xmgn_status scan_impl(const T* in, O* out, int64_t n, int64_t* tmp, cudaStream_t s, const int32_t* skip = nullptr) {
   if (n <= 0) {
     XMGN_CUDA(cudaMemsetAsync(out, 0, sizeof(O), s));
     return XMGN_OK;
@@ -126,7 +128,8 @@ xmgn_status scan_impl(const T* in, O* out, int64_t n, int64_t* tmp, cudaStream_t
       sums = tmp + nt;
     }
   }
-  launch_pdl(tile_scan_kernel<T, O>, unsigned(nt), kScanThreads, 0, s, in, out, n, sums, nt > kDirectTiles ? 1 : 0);
+  launch_pdl(tile_scan_kernel<T, O>, unsigned(nt), kScanThreads, 0, s, in, out, n, sums, nt > kDirectTiles ? 1 : 0,
+             skip);
   XMGN_LAUNCH_CHECK();
   return XMGN_OK;
 }
@@ -138,8 +141,9 @@ size_t scan_tmp_elems(int64_t n) {
   return size_t(2 * nt + 1) + scan_tmp_elems(nt);
 }
 
-xmgn_status exclusive_scan_i32(const int32_t* in, int64_t* out, int64_t n, int64_t* tmp, cudaStream_t s) {
-  return scan_impl<int32_t, int64_t>(in, out, n, tmp, s);
+xmgn_status exclusive_scan_i32(const int32_t* in, int64_t* out, int64_t n, int64_t* tmp, cudaStream_t s,
+                               const int32_t* skip) {
+  return scan_impl<int32_t, int64_t>(in, out, n, tmp, s, skip);
 }
 xmgn_status exclusive_scan_i32(const int32_t* in, int32_t* out, int64_t n, int64_t* tmp, cudaStream_t s) {
   return scan_impl<int32_t, int32_t>(in, out, n, tmp, s);
