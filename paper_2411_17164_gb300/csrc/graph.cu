@@ -211,6 +211,42 @@ struct Best {
   }
 };
 
+// The (y, z) rows of ring r >= 2 around a cell that lie in the grid and can hold
+// cells of it: all rows of the clamped square, or, once both x faces are outside
+// the grid, those on its rim only (an inner row has no cell but its two ends).
+// So a point looks at no more rows than the grid has cells, also where the grid
+// is thin and a far point needs many rings: with all (2r + 1)^2 rows of every
+// ring, a point 2700 cells off a flat cloud would step through 2.6e10.
+__device__ __forceinline__ int ring_rows(const Grid& g, int cx, int cy, int cz, int r) {
+  const int ny = min(cy + r, g.g[1] - 1) - max(cy - r, 0) + 1, nz = min(cz + r, g.g[2] - 1) - max(cz - r, 0) + 1;
+  if (cx - r >= 0 || cx + r < g.g[0]) return ny * nz;
+  const int fy = (cy - r >= 0) + (cy + r < g.g[1]), fz = (cz - r >= 0) + (cz + r < g.g[2]);  // faces inside the grid
+  return fz * ny + fy * (nz - fz);  // the rows of the z faces, then the two ends of the others
+}
+// Row `id` of them.  Called, not inlined, and with nothing kept between rows: most
+// points need no such ring, and the registers would cost the search resident warps
+// (three levels up to 1.25M points 1938 us, inlined 1953; 200k points on a
+// line 55 -> 2.6 ms against all rows of every ring).
+__device__ __noinline__ int2 ring_row(const Grid* grid, int cx, int cy, int cz, int r, int id) {
+  const Grid g = *grid;
+  int y, z;
+  const int ylo = cy - r, yhi = cy + r, zlo = cz - r, zhi = cz + r;
+  const int y0 = max(ylo, 0), z0 = max(zlo, 0), ny = min(yhi, g.g[1] - 1) - y0 + 1;
+  y = y0 + id % ny;
+  z = z0 + id / ny;
+  if (cx - r >= 0 || cx + r < g.g[0]) return make_int2(y, z);
+  const int fz = (zlo >= 0) + (zhi < g.g[2]);
+  const int i = id - fz * ny;
+  if (i < 0) {
+    z = id < ny && zlo >= 0 ? zlo : zhi;
+  } else {
+    const int m = min(zhi, g.g[2] - 1) - z0 + 1 - fz;
+    y = i < m && ylo >= 0 ? ylo : yhi;
+    z = (zlo >= 0 ? z0 + 1 : z0) + i % m;
+  }
+  return make_int2(y, z);
+}
+
 template <int G>
 __device__ __forceinline__ int group_get(uint32_t mask, int v, int l) {
   if constexpr (G == 1) return v;
@@ -234,11 +270,10 @@ __device__ __forceinline__ int group_get(uint32_t mask, int v, int l) {
 // to 1.25M points.  Rows are read from the middle of the block out and left out
 // when they are farther away than the k-th best so far (93 -> 85 us, 0.77 -> 0.64).
 template <int KC, int G, bool QUERY>
-__global__ void __launch_bounds__(128) knn_kernel(const int32_t* __restrict__ q, const int4* __restrict__ pts,
-                                                  const int32_t* __restrict__ start, int64_t q0, int64_t q1, int k,
-                                                  const Grid* __restrict__ grid, int32_t* __restrict__ nbr,
-                                                  int64_t stride, int off, int32_t* __restrict__ rcnt,
-                                                  int32_t* __restrict__ rank) {
+__global__ void __launch_bounds__(128, KC <= 6 ? 8 : KC == 8 ? 6 : 0)
+    knn_kernel(const int32_t* __restrict__ q, const int4* __restrict__ pts, const int32_t* __restrict__ start,
+               int64_t q0, int64_t q1, int k, const Grid* __restrict__ grid, int32_t* __restrict__ nbr, int64_t stride,
+               int off, int32_t* __restrict__ rcnt, int32_t* __restrict__ rank) {
   pdl_wait();
   pdl_trigger();
   const Grid gr = *grid;
@@ -266,17 +301,23 @@ __global__ void __launch_bounds__(128) knn_kernel(const int32_t* __restrict__ q,
       }
     };
     for (int r = 1;; ++r) {
-      const int side = 2 * r + 1, rows = side * side;
       const int x0 = max(cx - r, 0), x1 = min(cx + r, gr.g[0] - 1);
+      const int rows = r == 1 ? 9 : ring_rows(gr, cx, cy, cz, r);
       // This lane's row of the G rows from `base` on (the 3 x 3 rows of the first block from the middle out):
       // one range, or the two end cells of an inner row; far2: no point of the row is nearer than its root.
       int64_t far2 = 0;
       auto ranges = [&](int base) {
         int4 v = make_int4(0, 0, 0, 0);
         const int id = base + gl;
-        const int dy = r == 1 ? int((0x22161u >> (2 * id)) & 3u) - 1 : id % side - r;
-        const int dz = r == 1 ? int((0x28215u >> (2 * id)) & 3u) - 1 : id / side - r;
-        const int y = cy + dy, z = cz + dz;
+        int y, z;
+        if (r == 1) {
+          y = cy + int((0x22161u >> (2 * id)) & 3u) - 1;
+          z = cz + int((0x28215u >> (2 * id)) & 3u) - 1;
+        } else {
+          const int2 w = ring_row(grid, cx, cy, cz, r, id);
+          y = w.x, z = w.y;
+        }
+        const int dy = y - cy, dz = z - cz;
         if (id < rows && y >= 0 && y < gr.g[1] && z >= 0 && z < gr.g[2]) {
           const int64_t my = dy == 0 ? 0 : dy < 0 ? ry - int64_t(y + 1) * gr.c + 1 : int64_t(y) * gr.c - ry;
           const int64_t mz = dz == 0 ? 0 : dz < 0 ? rz - int64_t(z + 1) * gr.c + 1 : int64_t(z) * gr.c - rz;
