@@ -695,16 +695,30 @@ struct Seg {
   int32_t parts, base;
 };
 
+// The host side of a bisection's plan.  The copies of it are asynchronous, and
+// where the GPU reads pageable memory itself nothing stages them: the arrays live
+// until the stream has been waited for.
+struct HostPlan {
+  std::vector<RcbSeg> plan;
+  std::vector<int32_t> base;
+  cudaStream_t s = nullptr;
+  bool pending = false;
+  ~HostPlan() {
+    if (pending) cudaStreamSynchronize(s);  // an error on the way to the caller's wait
+  }
+};
+
 // Parts by recursive coordinate bisection: part ids of all nodes into `part`,
-// no host synchronisation (a coordinate off the lattice is flagged in err).
+// no host synchronisation (a coordinate off the lattice is flagged in err).  The
+// caller keeps `host` and clears its `pending` once it has waited for the stream.
 xmgn_status bisect(const float* xyz, int64_t N, double scale, int32_t P, PartLayout& w, int32_t* part, uint32_t* err,
-                   cudaStream_t s) {
+                   HostPlan& host, cudaStream_t s) {
   XMGN_TRY(quantize_launch(xyz, N, scale, w.q, w.bbox, err, s));
   if (P == 1) {
     XMGN_CUDA(cudaMemsetAsync(part, 0, sizeof(int32_t) * size_t(N), s));
     return XMGN_OK;
   }
-  std::vector<RcbSeg> plan;
+  std::vector<RcbSeg>& plan = host.plan;
   std::vector<int> level;  // first plan entry of each level
   std::vector<Seg> segs{{N, P, 0}};
   for (bool any = true; any;) {
@@ -727,9 +741,11 @@ xmgn_status bisect(const float* xyz, int64_t N, double scale, int32_t P, PartLay
     for (const Seg& g : segs) any |= g.parts > 1;
   }
   level.push_back(int(plan.size()));
-  std::vector<int32_t> base(segs.size());
+  std::vector<int32_t>& base = host.base;
+  base.resize(segs.size());
   for (size_t i = 0; i < segs.size(); ++i) base[i] = segs[i].base;
-  // pageable sources: staged before the calls return
+  host.s = s;
+  host.pending = true;
   XMGN_CUDA(cudaMemcpyAsync(w.plan, plan.data(), sizeof(RcbSeg) * plan.size(), cudaMemcpyHostToDevice, s));
   XMGN_CUDA(cudaMemcpyAsync(w.base, base.data(), sizeof(int32_t) * base.size(), cudaMemcpyHostToDevice, s));
   XMGN_CUDA(cudaMemsetAsync(w.hist, 0, sizeof(uint32_t) * size_t(P) * kMaxBins, s));
@@ -856,7 +872,8 @@ xmgn_status partition_halo(const int64_t* row_ptr, const int32_t* col, int64_t N
 
   XMGN_CUDA(cudaMemsetAsync(w.stamp, 0, sizeof(int64_t) * 8, s));  // this pass replaces what an earlier one left
   // ---------------- parts
-  if (!part_in) XMGN_TRY(bisect(xyz, N, scale, P, w, w.part, err, s));
+  HostPlan host;
+  if (!part_in) XMGN_TRY(bisect(xyz, N, scale, P, w, w.part, err, host, s));
 
   // ---------------- halo BFS
   XMGN_CUDA(cudaMemsetAsync(w.bits, 0, sizeof(uint32_t) * size_t(int64_t(P) * words), s));
@@ -885,6 +902,7 @@ xmgn_status partition_halo(const int64_t* row_ptr, const int32_t* col, int64_t N
   std::vector<int64_t> info(size_t(2) * P + 3);
   XMGN_CUDA(cudaMemcpyAsync(info.data(), w.info, sizeof(int64_t) * info.size(), cudaMemcpyDeviceToHost, s));
   XMGN_CUDA(cudaStreamSynchronize(s));
+  host.pending = false;
   const int64_t nb = info[0];
   const uint32_t herr = uint32_t(info[1]) & (DEV_ERR_CAP | DEV_ERR_GRAPH | (part_in ? 0u : DEV_ERR_RANGE));
   if (herr || nb > w.cap) {
