@@ -2,6 +2,7 @@
 // helpers).  Everything here is internal; the public surface is include/xmgn.h.
 #pragma once
 
+#include <atomic>
 #include <utility>
 
 #include <cuda_runtime.h>
@@ -92,6 +93,20 @@ inline int num_sms() {
     cached[dev] = n > 0 ? n : 1;
   }
   return cached[dev];
+}
+
+// Runs set() when a launch site is first reached on the current device: what it
+// sets (the limit of a kernel's dynamic shared memory) belongs to the device.
+// `done`, a bit per device, belongs to the site.
+template <class F>
+inline xmgn_status once_per_device(std::atomic<uint64_t>& done, F set) {
+  int dev = 0;
+  XMGN_CUDA(cudaGetDevice(&dev));
+  const uint64_t bit = dev < 64 ? uint64_t(1) << dev : 0;
+  if (done.load(std::memory_order_acquire) & bit) return XMGN_OK;
+  XMGN_TRY(set());
+  done.fetch_or(bit, std::memory_order_release);
+  return XMGN_OK;
 }
 
 inline unsigned grid_for(int64_t n, int threads, int64_t cap_blocks = 0) {

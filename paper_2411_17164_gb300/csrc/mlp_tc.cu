@@ -2454,12 +2454,9 @@ template <int MODE>
 xmgn_status launch_fwd(const FwdArgs& a, cudaStream_t s) {
   if (!a.w.w1lo || !a.w.w2lo) return fail(XMGN_ERR_ARG, "missing low weight images");
   const int probe = MODE == M_EDGE ? PROBE_EDGE_FWD : (MODE == M_NODE ? PROBE_NODE_FWD : -1);
-  static bool attr = false;
+  static std::atomic<uint64_t> attr{0};  // devices
   if constexpr (MODE == M_EDGE) {
-    if (!attr) {
-      XMGN_TRY(allow_max_smem(edge_fwd_kernel));
-      attr = true;
-    }
+    XMGN_TRY(once_per_device(attr, [] { return allow_max_smem(edge_fwd_kernel); }));
     const uint32_t sm = carve_edge_fwd(a.w, nullptr, nullptr) + 1024u;
     XMGN_TRY(check_smem<MODE>(sm));
     FwdArgs b = a;
@@ -2471,19 +2468,13 @@ xmgn_status launch_fwd(const FwdArgs& a, cudaStream_t s) {
     launch_pdl(edge_fwd_kernel, mlp_grid(a.rows), kThreads, sm, s, b, me);
     tune_end(TUNE_EDGE_FWD_ORDER, s);
   } else if constexpr (MODE == M_NODE) {
-    if (!attr) {
-      XMGN_TRY(allow_max_smem(node_fwd_kernel));
-      attr = true;
-    }
+    XMGN_TRY(once_per_device(attr, [] { return allow_max_smem(node_fwd_kernel); }));
     const uint32_t sm = carve_node_fwd(a.w, nullptr, nullptr) + 1024u;
     XMGN_TRY(check_smem<MODE>(sm));
     probe_begin(probe, s);
     launch_pdl(node_fwd_kernel, mlp_grid(a.rows), kThreads, sm, s, a);
   } else {
-    if (!attr) {
-      XMGN_TRY(allow_max_smem(mlp_fwd_kernel<MODE>));
-      attr = true;
-    }
+    XMGN_TRY(once_per_device(attr, [] { return allow_max_smem(mlp_fwd_kernel<MODE>); }));
     const uint32_t sm = smem_bytes<MODE>(a.w, false);
     XMGN_TRY(check_smem<MODE>(sm));
     probe_begin(probe, s);
@@ -2496,8 +2487,8 @@ xmgn_status launch_fwd(const FwdArgs& a, cudaStream_t s) {
 
 template <int MODE>
 xmgn_status launch_bwd(const BwdArgs& a, cudaStream_t s) {
-  static bool attr = false;
-  if (!attr) {
+  static std::atomic<uint64_t> attr{0};  // devices
+  XMGN_TRY(once_per_device(attr, [] {
     if constexpr (MODE == M_EDGE) {
       XMGN_TRY(allow_max_smem(edge_bwd_kernel));
       XMGN_TRY(allow_max_smem(edge_bwd2_kernel));
@@ -2505,8 +2496,8 @@ xmgn_status launch_bwd(const BwdArgs& a, cudaStream_t s) {
     } else {
       XMGN_TRY(allow_max_smem(mlp_bwd_kernel<MODE>));
     }
-    attr = true;
-  }
+    return XMGN_OK;
+  }));
   if (MODE != M_EDGE && Shape<MODE>::SPLIT && (!a.w.w1lo || !a.w.w2lo))
     return fail(XMGN_ERR_ARG, "missing low weight images");
   const int variant = MODE == M_EDGE ? tune_choice(TUNE_EDGE_BWD_TILES, a.rows) : 0;

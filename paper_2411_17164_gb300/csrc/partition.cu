@@ -749,11 +749,11 @@ xmgn_status bisect(const float* xyz, int64_t N, double scale, int32_t P, PartLay
   XMGN_CUDA(cudaMemcpyAsync(w.plan, plan.data(), sizeof(RcbSeg) * plan.size(), cudaMemcpyHostToDevice, s));
   XMGN_CUDA(cudaMemcpyAsync(w.base, base.data(), sizeof(int32_t) * base.size(), cudaMemcpyHostToDevice, s));
   XMGN_CUDA(cudaMemsetAsync(w.hist, 0, sizeof(uint32_t) * size_t(P) * kMaxBins, s));
-  static bool attr = false;
-  if (!attr) {
+  static std::atomic<uint64_t> attr{0};  // devices
+  XMGN_TRY(once_per_device(attr, [] {
     XMGN_CUDA(cudaFuncSetAttribute(rcb_hist_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kHistSmem * 4));
-    attr = true;
-  }
+    return XMGN_OK;
+  }));
   // digits of the 53-bit key, high to low: 25 coordinate bits, then as many id bits as N needs
   struct Digit {
     int on_id, shift, bits;

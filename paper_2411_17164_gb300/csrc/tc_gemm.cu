@@ -471,11 +471,8 @@ xmgn_status tc_gemm(const Bf16Rows& A, int64_t M, const uint8_t* img_base, const
   memset(&td, 0, sizeof(td));
   if (a.staged) XMGN_TRY(f32_map(&td, D, M, N, ldd));
   const size_t smem = 1024 + ((a.img_bytes + 1023) & ~1023u) + 2 * size_t(128) * a.K * 2;
-  static bool attr = false;
-  if (!attr) {
-    XMGN_TRY(allow_max_smem(tc_gemm_kernel));
-    attr = true;
-  }
+  static std::atomic<uint64_t> attr{0};  // devices
+  XMGN_TRY(once_per_device(attr, [] { return allow_max_smem(tc_gemm_kernel); }));
   launch_pdl(tc_gemm_kernel, tc_grid((M + 127) / 128), kThreads, smem, s, a, td);
   XMGN_LAUNCH_CHECK();
   return XMGN_OK;
@@ -512,11 +509,8 @@ xmgn_status tc_gemm_tn(const std::vector<TnJob>& jobs, int64_t M, float* part, s
     red.push_back({part, grid, len, 0, len, j.out, K1, N, j.kvalid, j.nvalid, j.nsplit});
     part += tc_gemm_tn_part_elems(K1, N);
   }
-  static bool attr = false;
-  if (!attr) {
-    XMGN_TRY(allow_max_smem(tc_gemm_tn_kernel));
-    attr = true;
-  }
+  static std::atomic<uint64_t> attr{0};  // devices
+  XMGN_TRY(once_per_device(attr, [] { return allow_max_smem(tc_gemm_tn_kernel); }));
   tune_begin(TUNE_TN_GRID, s);
   launch_pdl(tc_gemm_tn_kernel, dim3(unsigned(grid), unsigned(jobs.size())), kThreads, smem, s, L);
   XMGN_LAUNCH_CHECK();

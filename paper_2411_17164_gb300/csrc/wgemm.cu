@@ -404,11 +404,11 @@ uint32_t smem_of(int BN) { return kStages * (kAStage + uint32_t(BN) * kBK * 2u) 
 
 xmgn_status launch(WgArgs& a, const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap& td, cudaStream_t s,
                    const CUtensorMap* tp = nullptr) {
-  static bool attr = false;
-  if (!attr) {
+  static std::atomic<uint64_t> attr{0};  // devices
+  XMGN_TRY(once_per_device(attr, [] {
     XMGN_CUDA(cudaFuncSetAttribute(wg_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem_of(256))));
-    attr = true;
-  }
+    return XMGN_OK;
+  }));
   a.err = device_error_word();
   const int64_t tiles = int64_t(a.tiles_m) * a.tiles_n * a.splits;
   const int grid = int(tiles < num_sms() ? tiles : num_sms());

@@ -26,3 +26,10 @@ def test_sources_of_copies_live_until_the_stream_is_waited_for(run):
     got = dict(run("copies"))
     assert got.pop("changed") == "0"
     assert set(got.values()) == {"0"}  # and the calls succeed
+
+
+def test_every_path_launches_on_a_second_device(run):
+    """Limits of dynamic shared memory belong to a device, not to the process."""
+    got = dict(run("devices"))
+    assert got.pop("refused") == "0" and len(got) == 12
+    assert set(got.values()) == {"0"}
