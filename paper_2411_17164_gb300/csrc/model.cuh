@@ -117,10 +117,12 @@ xmgn_status gemm_nt_f32(const RowSrc& A, int64_t M, const float* B, int N, float
                         int epi, const float* aux, cudaStream_t s);
 // G[K1,N] = A^T B over M rows, written (not added) into G (row-major, ld N);
 // deterministic two-level reduction through `part` scratch (its size covers
-// every product of at most K1 x N).
+// every product of at most K1 x N over at most M rows).  terms > M: B's rows are
+// sums of that many rows in all (of a node's edges), and the product is split
+// over as many chunks as if they were summed here.
 size_t gemm_tn_part_elems(int64_t M, int K1, int N);
 xmgn_status gemm_tn_f32(const RowSrc& A, int64_t M, const float* B, int64_t ldb, int N, float* G,
-                        float* part, cudaStream_t s);
+                        float* part, cudaStream_t s, int64_t terms = 0);
 // Column sums in two levels: colsum_chunk_count(M) row chunks, each written as
 // one partial row, then out[c] = the sum of the nb partial rows (fixed order).
 int colsum_chunk_count(int64_t M);

@@ -81,7 +81,7 @@ void f32_ws_layout(Arena& A, const ParamPlan& p, int64_t n, int64_t E, F32Ws& w,
   w.P = tc ? nullptr : A.take<float>(size_t(n) * 2 * H);
   w.S = tc ? nullptr : A.take<float>(size_t(n) * 2 * H);
   w.grad = A.take<float>(size_t(p.total));
-  size_t tn = gemm_tn_part_elems(R, wide_kmax(p), H);
+  const size_t tn = gemm_tn_part_elems(R, p.in_enc > 2 * H ? p.in_enc : 2 * H, H);  // the widest operand: [h, a]
   w.tnpart = A.take<float>(tn);
   w.cspart = A.take<float>(colsum_part_elems(R, H));
   w.lnpart = A.take<float>(ln_bwd_part_elems(H));
@@ -364,7 +364,7 @@ xmgn_status f32_backward(const ParamPlan& p, const float* P, const xmgn_graph& g
       for (int b = 0; b < 2; ++b) {
         const int64_t wb = oe.W1 + int64_t(b) * H * H;
         XMGN_TRY(gemm_nt_f32(rows1(w.S + b * H, 2 * H, H), n, P + wb, H, w.dh, H, EPI_ACCUM, nullptr, s));
-        XMGN_TRY(gemm_tn_f32(rows1(hl, H, H), n, w.S + b * H, 2 * H, H, G + wb, w.tnpart, s));
+        XMGN_TRY(gemm_tn_f32(rows1(hl, H, H), n, w.S + b * H, 2 * H, H, G + wb, w.tnpart, s, E));
       }
       XMGN_TRY(colsum_f32(w.S, n, H, 2 * H, G + oe.b1, w.cspart, s));
       XMGN_TRY(gemm_nt_f32(rows1(w.dZ1, H, H), E, P + oe.W1 + 2 * int64_t(H) * H, H, w.de, H, EPI_ACCUM, nullptr,

@@ -33,3 +33,22 @@ def test_every_path_launches_on_a_second_device(run):
     got = dict(run("devices"))
     assert got.pop("refused") == "0" and len(got) == 12
     assert set(got.values()) == {"0"}
+
+
+@pytest.mark.parametrize("H", [32, 128, 256, 512])
+@pytest.mark.parametrize("rows", [300, 5000, 60000, 354000, 1500000])
+def test_fp32_weight_gradient_chains_are_bounded(run, H, rows):
+    """No weight gradient of the FP32 path sums more than max(4096, M / 128) rows in one running sum (a graph with as
+    many nodes as edges, so that M is one number), and the partial sums of different buffers do not meet."""
+    out = run("products", H, rows)
+    assert out[0] == ["status", "0"]
+    chunks = [int(v[1]) for v in out if v[0] == "chunks"]
+    assert len(chunks) >= 10
+    for c in chunks:
+        assert 16 * -(--(-rows // c) // 16) <= max(4096, 16 * -(--(-rows // 128) // 16)), (c, rows)
+    room = {}
+    for _, base, nb, ln in (v for v in out if v[0] == "parts"):
+        room[int(base)] = max(room.get(int(base), 0), 4 * int(nb) * int(ln))
+    at = sorted(room)
+    for a, b in zip(at, at[1:]):
+        assert a + room[a] <= b
