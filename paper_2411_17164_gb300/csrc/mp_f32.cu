@@ -67,10 +67,11 @@ void f32_ws_layout(Arena& A, const ParamPlan& p, int64_t n, int64_t E, F32Ws& w,
   w.nfeat = p.fourier ? A.take<float>(size_t(n) * p.in_enc) : nullptr;
   w.feat = A.take<float>(size_t(E) * kInEdge);
   w.Z1 = A.take<float>(size_t(R) * H);
-  w.A1 = A.take<float>(size_t(R) * H);
-  w.Z2 = A.take<float>(size_t(R) * H);
-  w.dZ2 = A.take<float>(size_t(R) * H);
-  w.dZ1 = A.take<float>(size_t(R) * H);
+  // the wide path keeps these in bf16 (WideScratch)
+  w.A1 = tc ? nullptr : A.take<float>(size_t(R) * H);
+  w.Z2 = tc ? nullptr : A.take<float>(size_t(R) * H);
+  w.dZ2 = tc ? nullptr : A.take<float>(size_t(R) * H);
+  w.dZ1 = tc ? nullptr : A.take<float>(size_t(R) * H);
   w.elast = A.take<float>(size_t(E) * H);
   w.dy = A.take<float>(size_t(n) * p.out);
   w.dh = A.take<float>(size_t(n) * H);
@@ -81,8 +82,8 @@ void f32_ws_layout(Arena& A, const ParamPlan& p, int64_t n, int64_t E, F32Ws& w,
   w.P = tc ? nullptr : A.take<float>(size_t(n) * 2 * H);
   w.S = tc ? nullptr : A.take<float>(size_t(n) * 2 * H);
   w.grad = A.take<float>(size_t(p.total));
-  const size_t tn = gemm_tn_part_elems(R, p.in_enc > 2 * H ? p.in_enc : 2 * H, H);  // the widest operand: [h, a]
-  w.tnpart = A.take<float>(tn);
+  const int k1 = p.in_enc > 2 * H ? p.in_enc : 2 * H;  // the widest operand of a weight gradient: [h, a]
+  w.tnpart = tc ? nullptr : A.take<float>(gemm_tn_part_elems(R, k1, H));
   w.cspart = A.take<float>(colsum_part_elems(R, H));
   w.lnpart = A.take<float>(ln_bwd_part_elems(H));
   w.losspart = A.take<float>(loss_part_elems(n));

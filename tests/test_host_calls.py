@@ -1,4 +1,5 @@
 """The library's host side on a stand-in CUDA runtime (host_runtime.cpp), without a GPU."""
+import ctypes as C
 import glob
 import os
 import subprocess
@@ -52,3 +53,20 @@ def test_fp32_weight_gradient_chains_are_bounded(run, H, rows):
     at = sorted(room)
     for a, b in zip(at, at[1:]):
         assert a + room[a] <= b
+
+
+@pytest.mark.parametrize("H", [256, 512])
+def test_wide_workspace_holds_what_the_path_reads(H):
+    """Per edge: five fp32 rows (pre-activation, last edge state, its gradient, receiver and sender parts), the gathered
+    bf16 operand of 3H, three bf16 rows, one fp32 product, the four edge inputs."""
+    from paper_2411_17164_gb300 import build, xmgn
+    build.build()
+
+    def ws(E):
+        w, c = C.c_size_t(), C.c_size_t()
+        d = xmgn.ModelDesc(H, 3, 6, 4, xmgn.XMGN_BF16)
+        assert xmgn.lib().xmgn_model_ws(C.byref(d), 50_000, E, C.byref(w), C.byref(c)) == 0
+        return w.value
+
+    need = 5 * 4 * H + 2 * 3 * H + 3 * 2 * H + 4 * H + 16
+    assert ws(400_000) - ws(300_000) <= 100_000 * need + 100_000  # and the block partials of the column sums
