@@ -21,7 +21,10 @@ struct MlpImgs {
   const uint8_t* w1lo;  // bf16(W1 - bf16(W1)) (all modes but the node MLP)
   const uint8_t* w2lo;  // bf16(W2 - bf16(W2))
   uint32_t w1_bytes, w2_bytes;
-  int late;  // the images are written by the kernel launched just before
+  // Whether the kernel waits for the one launched before it before it reads the
+  // images and the MLP's parameters.  0 only where another kernel stands between
+  // whatever wrote them and this one (kernels begin early, launch_pdl).
+  int late;
 };
 
 struct MlpParams {

@@ -351,8 +351,8 @@ void col_jobs(std::vector<RedJob>& j, const float* cpart, int nparts, int H, con
   }
 }
 
-MlpImgs imgs_of(const uint8_t* base, const Img& a, const Img& b, const Img* al = nullptr,
-                const Img* bl = nullptr) {
+// As the first kernel behind the packing must read them.
+MlpImgs fresh_imgs(const uint8_t* base, const Img& a, const Img& b, const Img* al = nullptr, const Img* bl = nullptr) {
   MlpImgs m;
   m.w1 = base + a.off;
   m.w2 = base + b.off;
@@ -360,6 +360,12 @@ MlpImgs imgs_of(const uint8_t* base, const Img& a, const Img& b, const Img* al =
   m.w2lo = bl ? base + bl->off : nullptr;
   m.w1_bytes = a.bytes();
   m.w2_bytes = b.bytes();
+  m.late = 1;
+  return m;
+}
+// As the kernels after that one may: the images (and parameters) are older than the kernel before.
+MlpImgs imgs_of(const uint8_t* base, const Img& a, const Img& b, const Img* al = nullptr, const Img* bl = nullptr) {
+  MlpImgs m = fresh_imgs(base, a, b, al, bl);
   m.late = 0;
   return m;
 }
@@ -494,8 +500,7 @@ xmgn_status bf16_forward(const ParamPlan& p, const float* P, const xmgn_graph& g
   f.fin_w = p.in_node;
   f.xyz = xyz;
   f.fourier = p.fourier;
-  f.w = imgs_of(c.img, ip.new1, ip.new2, &ip.new1l, &ip.new2l);
-  f.w.late = 1;
+  f.w = fresh_imgs(c.img, ip.new1, ip.new2, &ip.new1l, &ip.new2l);
   f.p = params_of(P, p.ne);
   f.o32 = c.h32;
   f.o16 = c.h16;

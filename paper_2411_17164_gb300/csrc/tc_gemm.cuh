@@ -55,6 +55,9 @@ struct Bf16Rows {
 // D[M, N] (=|+=) A[M, K] * B  where B is the image `img` used K-major
 // (img.R = N, img.C = K) or, if b_mn, MN-major (img.R = K, img.C = N).
 // With D null the product is rounded to bf16 and written to D16 instead.
+// The kernel loads the image before it waits for the kernel launched before it
+// (launch_pdl): the image must be older than that kernel.  Not straight after
+// pack_images, in other words: one more kernel has to stand between.
 xmgn_status tc_gemm(const Bf16Rows& A, int64_t M, const uint8_t* img_base, const Img& img, bool b_mn,
                     int N, float* D, int64_t ldd, bool accumulate, cudaStream_t s, bf16* D16 = nullptr);
 
