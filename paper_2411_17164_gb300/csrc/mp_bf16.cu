@@ -351,6 +351,21 @@ void col_jobs(std::vector<RedJob>& j, const float* cpart, int nparts, int H, con
   }
 }
 
+// The products of `tn` over n rows, then the sums of their partials and of `red`:
+// one unit for the tuner, as the choice of the grid weighs the product against
+// the partials that it leaves to be summed.  The products' sums, by far the most
+// blocks, stand first (a block looks for its job from the front).
+xmgn_status products_and_sums(const std::vector<TnJob>& tn, int64_t n, float* part, const std::vector<RedJob>& red,
+                              cudaStream_t s) {
+  std::vector<RedJob> all;
+  tune_begin(TUNE_TN_GRID, s);
+  XMGN_TRY(tc_gemm_tn(tn, n, part, all, s));
+  all.insert(all.end(), red.begin(), red.end());
+  XMGN_TRY(reduce_batch(all, s));
+  tune_end(TUNE_TN_GRID, s);
+  return XMGN_OK;
+}
+
 // As the first kernel behind the packing must read them.
 MlpImgs fresh_imgs(const uint8_t* base, const Img& a, const Img& b, const Img* al = nullptr, const Img* bl = nullptr) {
   MlpImgs m;
@@ -642,10 +657,10 @@ xmgn_status bf16_backward(const ParamPlan& p, const float* P, const xmgn_graph& 
   XMGN_TRY(mlp_bwd_tc(M_DEC, bd, s));
   {
     std::vector<RedJob> red;
-    XMGN_TRY(tc_gemm_tn({{rows_of(hL, H), w.dZ1n, H, H, G + p.dec.W1, H, H, H},
-                         {rows_of(w.A1g, H), w.dZ2g, 64, 64, G + p.dec.W2, H, p.out, p.out}}, n, w.tnpart, red, s));
     col_jobs(red, w.cpartn, gn, H, p.dec, G);
-    XMGN_TRY(reduce_batch(red, s));
+    XMGN_TRY(products_and_sums({{rows_of(hL, H), w.dZ1n, H, H, G + p.dec.W1, H, H, H},
+                                {rows_of(w.A1g, H), w.dZ2g, 64, 64, G + p.dec.W2, H, p.out, p.out}},
+                               n, w.tnpart, red, s));
   }
 
   // Weight-gradient products of the node MLP: with the layer's other one in a
@@ -681,8 +696,7 @@ xmgn_status bf16_backward(const ParamPlan& p, const float* P, const xmgn_graph& 
     std::vector<RedJob> red;
     col_jobs(red, w.cpartn, gn, H, on, G);
     if (node_products_now) {
-      XMGN_TRY(tc_gemm_tn(tn, n, w.tnpart, red, s));
-      XMGN_TRY(reduce_batch(red, s));
+      XMGN_TRY(products_and_sums(tn, n, w.tnpart, red, s));
       tn.clear();
       red.clear();
     }
@@ -719,7 +733,6 @@ xmgn_status bf16_backward(const ParamPlan& p, const float* P, const xmgn_graph& 
     XMGN_TRY(tc_gemm(rows_of(w.S16, 2 * H), n, c.img, li.ewrs, true, H, w.dh, H, true, s));
     {
       tn.push_back({rows_of(h16, H), w.S16, 2 * H, 2 * H, G + oe.W1, H, 2 * H, H});
-      XMGN_TRY(tc_gemm_tn(tn, n, w.tnpart, red, s));
       // db1 and T_l (seg_sums partials); dW1_e, dW2, db2, dgamma (per-CTA partials of the edge kernel)
       const int64_t cs = 4 * int64_t(H), ps = 2 * int64_t(H);
       red.push_back({w.colp, int(sg), ps, 0, H, G + oe.b1});
@@ -730,7 +743,7 @@ xmgn_status bf16_backward(const ParamPlan& p, const float* P, const xmgn_graph& 
         red.push_back({w.cpart, ge, cs, H, H, G + oe.b2});
         red.push_back({w.cpart, ge, cs, 2 * int64_t(H), H, G + oe.g});
       }
-      XMGN_TRY(reduce_batch(red, s));
+      XMGN_TRY(products_and_sums(tn, n, w.tnpart, red, s));
     }
   }
   {  // dbeta of the edge MLPs from db1 and T_l (the edge kernel does not sum it)
@@ -776,10 +789,10 @@ xmgn_status bf16_backward(const ParamPlan& p, const float* P, const xmgn_graph& 
   XMGN_TRY(mlp_bwd_tc(M_NENC, bne, s));
   {
     std::vector<RedJob> red;
-    XMGN_TRY(tc_gemm_tn({{rows_of(w.X16, 128), w.dZ1n, H, H, G + p.ne.W1, p.in_enc, H, H},
-                         {rows_of(w.A1g, H), w.dZ2g, H, H, G + p.ne.W2, H, H, H}}, n, w.tnpart, red, s));
     col_jobs(red, w.cpartn, gn, H, p.ne, G);
-    XMGN_TRY(reduce_batch(red, s));
+    XMGN_TRY(products_and_sums({{rows_of(w.X16, 128), w.dZ1n, H, H, G + p.ne.W1, p.in_enc, H, H},
+                                {rows_of(w.A1g, H), w.dZ2g, H, H, G + p.ne.W2, H, H, H}},
+                               n, w.tnpart, red, s));
   }
   if (off) {  // join the copy stream
     XMGN_CUDA(cudaEventRecord(oc->sync[1], oc->copy));

@@ -511,10 +511,8 @@ xmgn_status tc_gemm_tn(const std::vector<TnJob>& jobs, int64_t M, float* part, s
   }
   static std::atomic<uint64_t> attr{0};  // devices
   XMGN_TRY(once_per_device(attr, [] { return allow_max_smem(tc_gemm_tn_kernel); }));
-  tune_begin(TUNE_TN_GRID, s);
   launch_pdl(tc_gemm_tn_kernel, dim3(unsigned(grid), unsigned(jobs.size())), kThreads, smem, s, L);
   XMGN_LAUNCH_CHECK();
-  tune_end(TUNE_TN_GRID, s);
   return XMGN_OK;
 }
 

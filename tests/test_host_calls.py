@@ -70,3 +70,16 @@ def test_wide_workspace_holds_what_the_path_reads(H):
 
     need = 5 * 4 * H + 2 * 3 * H + 3 * 2 * H + 4 * H + 16
     assert ws(400_000) - ws(300_000) <= 100_000 * need + 100_000  # and the block partials of the column sums
+
+
+@pytest.mark.parametrize("n", [2000, 200_000])
+def test_tuner_times_the_products_with_their_sums(run, n):
+    """The grid of the node-level products trades their time for the partials to be summed: both are inside the events."""
+    out = run("timed", 3, n)
+    assert out[0] == ["status", "0"]
+    names = [v[1] for v in out if v[0] == "launch"]
+    at = [i for i, v in enumerate(names) if v == "event"]
+    assert len(at) >= 8 and len(at) % 2 == 0
+    for a, b in zip(at[::2], at[1::2]):
+        inside = names[a + 1:b]
+        assert any("tc_gemm_tn_kernel" in v for v in inside) and any("reduce_parts_kernel" in v for v in inside)
