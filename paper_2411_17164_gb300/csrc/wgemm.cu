@@ -315,8 +315,10 @@ __global__ void __launch_bounds__(kWgThreads, 1) wg_kernel(WgArgs a, const __gri
     }
   }
   if (tid == 64 || tid == 192) bulk_wait0();  // every output store is complete
-  // Only now: a row kernel started beside this one would run with the little L1
-  // that this one's shared memory leaves.
+  // A CTA counts as triggered with its first thread here, a producer that has
+  // issued its last load: the next kernel may begin while the last tiles are still
+  // multiplied and stored (its own wait orders the results).  A trigger right
+  // behind pdl_wait measured the same.
   pdl_trigger();
   tc_fence_before();
   __syncthreads();
