@@ -664,11 +664,14 @@ xmgn_status bf16_backward(const ParamPlan& p, const float* P, const xmgn_graph& 
   }
 
   // Weight-gradient products of the node MLP: with the layer's other one in a
-  // single launch after the edge kernel, or, where their five operands (10 H
-  // bytes a node) and partials take longer to read again after the edge kernel
-  // has streamed through L2 than two launches cost, right behind the node kernel
-  // (2k nodes: 1.93 -> 1.63 ms a step in one; 200k nodes: 31.12 ms, 32.0 in one).
-  const bool node_products_now = size_t(n) * H * 10 > (size_t(32) << 20);
+  // single launch after the edge kernel, or right behind the node kernel, whose
+  // outputs (10 H bytes a node) are then read before the edge kernel has streamed
+  // through L2.  One launch saves two kernels a layer, but from 6.5k nodes on its
+  // three products are more CTAs than SMs.  Training steps of 15 layers, one launch
+  // against behind: 2k nodes 1.57 / 1.71 ms, 6k 2.24 / 2.38, 8k 2.47 / 2.49, 8.5k
+  // 2.69 / 2.71, 9k 2.76 / 2.75, 12k 3.25 / 3.20, 20k 5.20 / 5.08, 26k 5.90 / 5.77,
+  // 32k 6.58 / 6.51; equal within 0.2 % from 40k to 200k.
+  const bool node_products_now = size_t(n) * H * 10 > 11'200'000;  // 8750 nodes
   for (int l = p.L - 1; l >= 0; --l) {
     const LayerImgs& li = ip.layer[l];
     const bf16* h16 = c.h16 + size_t(l) * n * H;
