@@ -2572,7 +2572,8 @@ __global__ void edge_inputs_bf16_kernel(const float* __restrict__ xyz, const int
 xmgn_status edge_inputs_bf16(const float* xyz, const int32_t* gid, const int32_t* recv, const int32_t* col,
                              int64_t E, bf16* out, cudaStream_t s) {
   if (E <= 0) return XMGN_OK;
-  launch_pdl(edge_inputs_bf16_kernel, grid_for(E, 256, int64_t(num_sms()) * 16), 256, 0, s, xyz, gid, recv, col, E, out);
+  launch_pdl(edge_inputs_bf16_kernel, grid_for(E, 256, int64_t(num_sms()) * 16), 256, 0, s, xyz, gid, recv, col, E,
+             out);
   XMGN_LAUNCH_CHECK();
   return XMGN_OK;
 }

@@ -756,7 +756,7 @@ xmgn_status bf16_backward(const ParamPlan& p, const float* P, const xmgn_graph& 
           p.edge[l].be != p.edge[0].be + l * stride)
         return fail(XMGN_ERR_ARG, "edge MLP parameters are not laid out with a fixed stride per layer");
     launch_pdl(edge_beta_mv_kernel, p.L, 256, 0, s, P, p.edge[0].W1 + 2 * int64_t(H) * H, p.edge[0].b1, stride, G,
-                                            w.vbeta);
+               w.vbeta);
     XMGN_LAUNCH_CHECK();
     launch_pdl(edge_beta_kernel, 1, 128, 0, s, p.L, p.edge[0].be, stride, w.tsum, w.vbeta, G);
     XMGN_LAUNCH_CHECK();

@@ -686,9 +686,15 @@ xmgn_status layernorm_fwd_f32(const float* Z, int64_t M, int N, const float* gam
   if (M <= 0) return XMGN_OK;
   const unsigned grid = grid_for(M * 32, 256, int64_t(num_sms()) * 16);
   if (rows_vec4(N, {Z, Y, resid_in, resid_out})) {
-    if (N == 128) launch_pdl_if(rows_early(M, N), ln_fwd_v4_kernel<1>, grid, 256, 0, s, Z, bias, M, gamma, beta, Y, resid_in, resid_out);
-    if (N == 256) launch_pdl_if(rows_early(M, N), ln_fwd_v4_kernel<2>, grid, 256, 0, s, Z, bias, M, gamma, beta, Y, resid_in, resid_out);
-    if (N == 512) launch_pdl_if(rows_early(M, N), ln_fwd_v4_kernel<4>, grid, 256, 0, s, Z, bias, M, gamma, beta, Y, resid_in, resid_out);
+    if (N == 128)
+      launch_pdl_if(rows_early(M, N), ln_fwd_v4_kernel<1>, grid, 256, 0, s, Z, bias, M, gamma, beta, Y, resid_in,
+                    resid_out);
+    if (N == 256)
+      launch_pdl_if(rows_early(M, N), ln_fwd_v4_kernel<2>, grid, 256, 0, s, Z, bias, M, gamma, beta, Y, resid_in,
+                    resid_out);
+    if (N == 512)
+      launch_pdl_if(rows_early(M, N), ln_fwd_v4_kernel<4>, grid, 256, 0, s, Z, bias, M, gamma, beta, Y, resid_in,
+                    resid_out);
     XMGN_LAUNCH_CHECK();
     return XMGN_OK;
   }
@@ -704,13 +710,20 @@ xmgn_status layernorm_fwd_agg_f32(const float* Z, const float* bias, const int64
   if (n <= 0) return XMGN_OK;
   const unsigned grid = grid_for(n * 32, 256, int64_t(num_sms()) * 16);
   if (rows_vec4(N, {Z, resid_in, resid_out, agg})) {
-    if (N == 128) launch_pdl_if(rows_early(8 * n, N), ln_fwd_agg_v4_kernel<1>, grid, 256, 0, s, Z, bias, row_ptr, n, gamma, beta, resid_in, resid_out, agg);
-    if (N == 256) launch_pdl_if(rows_early(8 * n, N), ln_fwd_agg_v4_kernel<2>, grid, 256, 0, s, Z, bias, row_ptr, n, gamma, beta, resid_in, resid_out, agg);
-    if (N == 512) launch_pdl_if(rows_early(8 * n, N), ln_fwd_agg_v4_kernel<4>, grid, 256, 0, s, Z, bias, row_ptr, n, gamma, beta, resid_in, resid_out, agg);
+    if (N == 128)
+      launch_pdl_if(rows_early(8 * n, N), ln_fwd_agg_v4_kernel<1>, grid, 256, 0, s, Z, bias, row_ptr, n, gamma, beta,
+                    resid_in, resid_out, agg);
+    if (N == 256)
+      launch_pdl_if(rows_early(8 * n, N), ln_fwd_agg_v4_kernel<2>, grid, 256, 0, s, Z, bias, row_ptr, n, gamma, beta,
+                    resid_in, resid_out, agg);
+    if (N == 512)
+      launch_pdl_if(rows_early(8 * n, N), ln_fwd_agg_v4_kernel<4>, grid, 256, 0, s, Z, bias, row_ptr, n, gamma, beta,
+                    resid_in, resid_out, agg);
     XMGN_LAUNCH_CHECK();
     return XMGN_OK;
   }
-  launch_pdl_if(rows_early(8 * n, N), ln_fwd_agg_kernel, grid, 256, 0, s, Z, bias, row_ptr, n, N, gamma, beta, resid_in, resid_out, agg);
+  launch_pdl_if(rows_early(8 * n, N), ln_fwd_agg_kernel, grid, 256, 0, s, Z, bias, row_ptr, n, N, gamma, beta, resid_in,
+                resid_out, agg);
   XMGN_LAUNCH_CHECK();
   return XMGN_OK;
 }
@@ -738,11 +751,18 @@ xmgn_status layernorm_bwd_f32(const float* Z, int64_t M, int N, const float* gam
   if (nb < 1) nb = 1;
   const size_t sh = size_t(8) * 3 * N * sizeof(float);
   if (rows_vec4(N, {Z, dY1, dY2, dZ, reinterpret_cast<const float*>(dZ16)})) {
-    if (N == 128) launch_pdl_if(rows_early(M, N), ln_bwd_v4_kernel<1>, unsigned(nb), 256, sh, s, Z, bias, M, gamma, dY1, dY2, idx2, dZ, dZ16, part);
-    if (N == 256) launch_pdl_if(rows_early(M, N), ln_bwd_v4_kernel<2>, unsigned(nb), 256, sh, s, Z, bias, M, gamma, dY1, dY2, idx2, dZ, dZ16, part);
-    if (N == 512) launch_pdl_if(rows_early(M, N), ln_bwd_v4_kernel<4>, unsigned(nb), 256, sh, s, Z, bias, M, gamma, dY1, dY2, idx2, dZ, dZ16, part);
+    if (N == 128)
+      launch_pdl_if(rows_early(M, N), ln_bwd_v4_kernel<1>, unsigned(nb), 256, sh, s, Z, bias, M, gamma, dY1, dY2, idx2,
+                    dZ, dZ16, part);
+    if (N == 256)
+      launch_pdl_if(rows_early(M, N), ln_bwd_v4_kernel<2>, unsigned(nb), 256, sh, s, Z, bias, M, gamma, dY1, dY2, idx2,
+                    dZ, dZ16, part);
+    if (N == 512)
+      launch_pdl_if(rows_early(M, N), ln_bwd_v4_kernel<4>, unsigned(nb), 256, sh, s, Z, bias, M, gamma, dY1, dY2, idx2,
+                    dZ, dZ16, part);
   } else {
-    launch_pdl_if(rows_early(M, N), ln_bwd_kernel, unsigned(nb), 256, sh, s, Z, bias, M, N, gamma, dY1, dY2, idx2, dZ, dZ16, part);
+    launch_pdl_if(rows_early(M, N), ln_bwd_kernel, unsigned(nb), 256, sh, s, Z, bias, M, N, gamma, dY1, dY2, idx2, dZ,
+                  dZ16, part);
   }
   XMGN_LAUNCH_CHECK();
   launch_pdl(sum_parts_kernel, (3 * N + 31) / 32, 256, 0, s, part, int(nb), 3 * N, dgamma, N, dbeta, db);
@@ -761,9 +781,11 @@ xmgn_status seg_sum_rows_f32(const float* v, int64_t ldv, const int64_t* row_ptr
   if (n <= 0) return XMGN_OK;
   const unsigned grid = grid_for(n * 32, 256, int64_t(num_sms()) * 16);
   if (seg_vec4(v, ldv, H, out, ldo))
-    launch_pdl_if(rows_early(8 * n, H), seg_sum_v4_kernel<false>, grid, 256, 0, s, v, ldv, row_ptr, nullptr, n, H, out, ldo, accumulate ? 1 : 0);
+    launch_pdl_if(rows_early(8 * n, H), seg_sum_v4_kernel<false>, grid, 256, 0, s, v, ldv, row_ptr, nullptr, n, H, out,
+                  ldo, accumulate ? 1 : 0);
   else
-    launch_pdl_if(rows_early(8 * n, H), seg_rows_kernel, grid, 256, 0, s, v, ldv, row_ptr, n, H, out, ldo, accumulate ? 1 : 0);
+    launch_pdl_if(rows_early(8 * n, H), seg_rows_kernel, grid, 256, 0, s, v, ldv, row_ptr, n, H, out, ldo,
+                  accumulate ? 1 : 0);
   XMGN_LAUNCH_CHECK();
   return XMGN_OK;
 }
@@ -774,9 +796,11 @@ xmgn_status seg_sum_cols_f32(const float* v, int64_t ldv, const int64_t* row_ptr
   if (n <= 0) return XMGN_OK;
   const unsigned grid = grid_for(n * 32, 256, int64_t(num_sms()) * 16);
   if (seg_vec4(v, ldv, H, out, ldo))
-    launch_pdl_if(rows_early(8 * n, H), seg_sum_v4_kernel<true>, grid, 256, 0, s, v, ldv, row_ptr, perm, n, H, out, ldo, accumulate ? 1 : 0);
+    launch_pdl_if(rows_early(8 * n, H), seg_sum_v4_kernel<true>, grid, 256, 0, s, v, ldv, row_ptr, perm, n, H, out, ldo,
+                  accumulate ? 1 : 0);
   else
-    launch_pdl_if(rows_early(8 * n, H), seg_cols_kernel, grid, 256, 0, s, v, ldv, row_ptr, perm, n, H, out, ldo, accumulate ? 1 : 0);
+    launch_pdl_if(rows_early(8 * n, H), seg_cols_kernel, grid, 256, 0, s, v, ldv, row_ptr, perm, n, H, out, ldo,
+                  accumulate ? 1 : 0);
   XMGN_LAUNCH_CHECK();
   return XMGN_OK;
 }

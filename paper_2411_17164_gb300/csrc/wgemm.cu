@@ -25,8 +25,7 @@
 // the epilogue and stores bf16 blocks of 64 columns (optionally also the fp32
 // pre-activation), so the fp32 product never goes to memory.  Two sets because
 // with four warps the epilogue of a K = 512 product is as long as the product
-// it hides behind (H = 512, 50k nodes: 16.56 -> 16.44 ms a
-// step).
+// it hides behind (H = 512, 50k nodes: 16.56 -> 16.44 ms a step).
 // Every wait is bounded: a wait that gives up flags the device error word and
 // the roles wind down.
 #include <cuda.h>
@@ -402,7 +401,8 @@ namespace {
 
 int tile_width(int N) { return N > 128 ? 256 : (N > 64 ? 128 : 64); }
 
-uint32_t smem_of(int BN) { return kStages * (kAStage + uint32_t(BN) * kBK * 2u) + 2u * kStage + 1024u; }  // a staging buffer per epilogue set
+// The ring of operand stages and a staging buffer per epilogue set.
+uint32_t smem_of(int BN) { return kStages * (kAStage + uint32_t(BN) * kBK * 2u) + 2u * kStage + 1024u; }
 
 xmgn_status launch(WgArgs& a, const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap& td, cudaStream_t s,
                    const CUtensorMap* tp = nullptr) {
@@ -514,8 +514,8 @@ xmgn_status wg_gemm_tn(const bf16* A, int64_t lda, const bf16* B, int64_t ldb, i
   XMGN_TRY(f32_map(&td, part, int64_t(a.splits) * tiles * kBM, a.BN, a.BN));  // [split][tile] blocks of 128 x BN
   XMGN_TRY(launch(a, ta, tb, td, s));
   const int64_t total = int64_t(K1) * N;
-  launch_pdl(wg_reduce_kernel, grid_for(total, 256, int64_t(num_sms()) * 8), 256, 0, s, part, a.splits, a.tiles_m, a.tiles_n,
-                                                                               a.BN, K1, N, G);
+  launch_pdl(wg_reduce_kernel, grid_for(total, 256, int64_t(num_sms()) * 8), 256, 0, s, part, a.splits, a.tiles_m,
+             a.tiles_n, a.BN, K1, N, G);
   XMGN_LAUNCH_CHECK();
   return XMGN_OK;
 }
