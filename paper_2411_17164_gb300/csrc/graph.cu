@@ -147,7 +147,9 @@ __global__ void grid_layout_kernel(int32_t* bbox, LevelSizes sizes, int levels, 
   out[l] = G;
 }
 
-__device__ __forceinline__ int cell_coord(int32_t q, int32_t lo, int32_t c) { return int(uint32_t(q - lo) / uint32_t(c)); }
+__device__ __forceinline__ int cell_coord(int32_t q, int32_t lo, int32_t c) {
+  return int(uint32_t(q - lo) / uint32_t(c));
+}
 
 // Cell of every reference point, and its place among the cell's points.
 __global__ void cell_count_kernel(const int32_t* __restrict__ q, int64_t n, const Grid* __restrict__ grid,
@@ -266,9 +268,9 @@ __device__ __forceinline__ int group_get(uint32_t mask, int v, int l) {
 // Bound by the latency of the dependent reads (range, then points).  Against a
 // thread per point with its candidate list in local memory, the cell ids read
 // first and the coordinates gathered: 114 -> 23 us at 2k points (eight lanes
-// per point), 185 -> 85 us at 200k, and 1.43 -> 0.64 ms for the three levels up
+// per point), 185 -> 86 us at 200k, and 1.43 -> 0.66 ms for the three levels up
 // to 1.25M points.  Rows are read from the middle of the block out and left out
-// when they are farther away than the k-th best so far (93 -> 85 us, 0.77 -> 0.64).
+// when they are farther away than the k-th best so far (93 -> 85 us, 0.77 -> 0.64 ms).
 template <int KC, int G, bool QUERY>
 __global__ void __launch_bounds__(128, KC <= 6 ? 8 : KC == 8 ? 6 : 0)
     knn_kernel(const int32_t* __restrict__ q, const int4* __restrict__ pts, const int32_t* __restrict__ start,
@@ -403,7 +405,8 @@ void knn_launch_g(unsigned grid, cudaStream_t s, const int32_t* q, const int4* p
   else if (k <= 16)
     launch_pdl(knn_kernel<16, G, QUERY>, grid, 128, 0, s, q, pts, start, q0, q1, k, gr, nbr, stride, off, rcnt, rank);
   else
-    launch_pdl(knn_kernel<kMaxK, G, QUERY>, grid, 128, 0, s, q, pts, start, q0, q1, k, gr, nbr, stride, off, rcnt, rank);
+    launch_pdl(knn_kernel<kMaxK, G, QUERY>, grid, 128, 0, s, q, pts, start, q0, q1, k, gr, nbr, stride, off, rcnt,
+               rank);
 }
 
 // Lanes per point: eight while that still leaves at most one wave of resident
@@ -416,7 +419,8 @@ xmgn_status knn_launch(const int32_t* q, const int4* pts, const int32_t* start, 
                        cudaStream_t s) {
   const int64_t n = q1 - q0;
   if (n * 8 <= int64_t(num_sms()) * 2048)
-    knn_launch_g<QUERY, 8>(grid_for(n * 8, 128, 1 << 30), s, q, pts, start, q0, q1, k, gr, nbr, stride, off, rcnt, rank);
+    knn_launch_g<QUERY, 8>(grid_for(n * 8, 128, 1 << 30), s, q, pts, start, q0, q1, k, gr, nbr, stride, off, rcnt,
+                           rank);
   else
     knn_launch_g<QUERY, 1>(grid_for(n, 128, 1 << 30), s, q, pts, start, q0, q1, k, gr, nbr, stride, off, rcnt, rank);
   XMGN_LAUNCH_CHECK();

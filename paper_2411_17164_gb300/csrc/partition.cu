@@ -16,11 +16,11 @@
 // hop: per-block hop counts, one scan in (part, hop, block) order, and each
 // set bit knows its place.
 //
-// Measured, 2M points in 16 parts with 15 hops, both calls: 28.9 -> 1.21 ms
+// Measured, 2M points in 16 parts with 15 hops, both calls: 28.9 -> 1.01 ms
 // (bisection by sorting all keys per level, with six extent atomics per node,
-// was 27 ms of it); 64 given regions of a 1M-point cloud: 2.45 -> 0.78 ms
+// was 27 ms of it); 64 given regions of a 1M-point cloud: 2.48 -> 0.72 ms
 // (the bitonic member sort was 0.8 ms of it).  What is left is bound by the L2
-// traffic of the edge pass (146 us) and of the reverse-edge search (98 us),
+// traffic of the edge pass (147 us) and of the reverse-edge search (99 us),
 // and by the launches of the levels and hops.
 #include <math.h>
 
@@ -118,7 +118,8 @@ __global__ void __launch_bounds__(1024) rcb_hist_kernel(const int32_t* __restric
     if (bin >= 0) {
       const uint32_t at = uint32_t(s) * uint32_t(nb) + uint32_t(bin);
       const unsigned same = __match_any_sync(__activemask(), at);
-      if ((threadIdx.x & 31) == unsigned(__ffs(same) - 1)) atomicAdd(SMEM ? &sh[at] : &hist[at], uint32_t(__popc(same)));
+      if ((threadIdx.x & 31) == unsigned(__ffs(same) - 1))
+        atomicAdd(SMEM ? &sh[at] : &hist[at], uint32_t(__popc(same)));
     }
   }
   if (SMEM) {
@@ -781,17 +782,17 @@ xmgn_status bisect(const float* xyz, int64_t N, double scale, int32_t P, PartLay
       // one histogram per block in shared memory while all segments' fit; with more segments the
       // atomics spread over that many more addresses and go to memory
       if (words <= kHistSmem)
-        launch_pdl(rcb_hist_kernel<true>, grid_for(N, 1024, int64_t(num_sms()) * 2), 1024, size_t(words) * 4, s, 
-            seg, N, w.q, w.state, nseg, d.on_id, d.shift, d.bits, w.hist);
+        launch_pdl(rcb_hist_kernel<true>, grid_for(N, 1024, int64_t(num_sms()) * 2), 1024, size_t(words) * 4, s, seg, N,
+                   w.q, w.state, nseg, d.on_id, d.shift, d.bits, w.hist);
       else
-        launch_pdl(rcb_hist_kernel<false>, grid_for(N, 1024, int64_t(num_sms()) * 2), 1024, 0, s, 
-            seg, N, w.q, w.state, nseg, d.on_id, d.shift, d.bits, w.hist);
+        launch_pdl(rcb_hist_kernel<false>, grid_for(N, 1024, int64_t(num_sms()) * 2), 1024, 0, s, seg, N, w.q, w.state,
+                   nseg, d.on_id, d.shift, d.bits, w.hist);
       XMGN_LAUNCH_CHECK();
       launch_pdl(rcb_find_kernel, unsigned(nseg), 256, 0, s, w.state, d.on_id, d.shift, d.bits, w.hist);
       XMGN_LAUNCH_CHECK();
     }
-    launch_pdl(rcb_split_kernel, grid_for(N, 512, int64_t(num_sms()) * 4), 512, 0, s, 
-        w.seg, l == 0 ? 1 : 0, N, w.q, w.state, pl, nnext, w.ext[(l + 1) & 1], w.base, last ? part : nullptr);
+    launch_pdl(rcb_split_kernel, grid_for(N, 512, int64_t(num_sms()) * 4), 512, 0, s, w.seg, l == 0 ? 1 : 0, N, w.q,
+               w.state, pl, nnext, w.ext[(l + 1) & 1], w.base, last ? part : nullptr);
     XMGN_LAUNCH_CHECK();
   }
   return XMGN_OK;
@@ -838,8 +839,8 @@ xmgn_status partition_halo(const int64_t* row_ptr, const int32_t* col, int64_t N
   // edges and the CSC permutation, once ids and row offsets are in place
   auto emit_edges = [&](int64_t nb, int64_t eb) -> xmgn_status {
     if (nb > 0) {
-      launch_pdl(batch_edges_kernel, grid_for(nb * 4, 256), 256, 0, s, w.members, nb, N, row_ptr, col, w.map, w.bits, words, L,
-                                                               b_row_ptr, b_col, b_recv, err);
+      launch_pdl(batch_edges_kernel, grid_for(nb * 4, 256), 256, 0, s, w.members, nb, N, row_ptr, col, w.map, w.bits,
+                 words, L, b_row_ptr, b_col, b_recv, err);
       XMGN_LAUNCH_CHECK();
     }
     if (b_csc_perm && eb > 0) {
@@ -881,13 +882,13 @@ xmgn_status partition_halo(const int64_t* row_ptr, const int32_t* col, int64_t N
   launch_pdl(bfs_seed_kernel, grid_for(N, 256), 256, 0, s, part, N, P, w.bits, words, w.map, err);
   XMGN_LAUNCH_CHECK();
   if (L > 0) {
-    launch_pdl(bfs_first_kernel, grid_for(N, 256, int64_t(num_sms()) * 8), 256, 0, s, row_ptr, col, N, part, P, w.bits, words,
-                                                                              w.map, w.members, w.counters, w.cap, err);
+    launch_pdl(bfs_first_kernel, grid_for(N, 256, int64_t(num_sms()) * 8), 256, 0, s, row_ptr, col, N, part, P, w.bits,
+               words, w.map, w.members, w.counters, w.cap, err);
     XMGN_LAUNCH_CHECK();
   }
   for (int h = 2; h <= L; ++h) {
-    launch_pdl(bfs_round_kernel, grid_for(N * 8, 256, int64_t(num_sms()) * 8), 256, 0, s, 
-        row_ptr, col, N, w.bits, words, w.map, w.members, w.counters, h, w.cap, err);
+    launch_pdl(bfs_round_kernel, grid_for(N * 8, 256, int64_t(num_sms()) * 8), 256, 0, s, row_ptr, col, N, w.bits,
+               words, w.map, w.members, w.counters, h, w.cap, err);
     XMGN_LAUNCH_CHECK();
   }
 
@@ -919,10 +920,11 @@ xmgn_status partition_halo(const int64_t* row_ptr, const int32_t* col, int64_t N
 
   // ---------------- batch nodes and degrees
   launch_pdl(hop_place_kernel, hgrid, 256, 0, s, w.bits, w.map, words, N, L, w.hbase, w.members, emit ? gid : nullptr,
-                                         emit ? hop : nullptr);
+             emit ? hop : nullptr);
   XMGN_LAUNCH_CHECK();
   if (nb > 0) {
-    launch_pdl(batch_deg_kernel, grid_for(nb, 256), 256, 0, s, w.members, nb, N, L, row_ptr, col, w.bits, words, w.deg, err);
+    launch_pdl(batch_deg_kernel, grid_for(nb, 256), 256, 0, s, w.members, nb, N, L, row_ptr, col, w.bits, words, w.deg,
+               err);
     XMGN_LAUNCH_CHECK();
   }
   int64_t* brp = emit ? b_row_ptr : w.brp;

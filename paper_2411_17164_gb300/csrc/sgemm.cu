@@ -12,8 +12,12 @@
 // packed pairs so that one fma.rn.f32x2 does two multiply-adds per issue slot.
 // The FMA pipe is what bounds it: per slice and thread 16 x 64 multiply-adds
 // stand against 64 shared-memory loads of 16 bytes, all free of bank conflicts
-// (a warp reads 64 + 128 consecutive bytes per step).  212k x 128 x 128: 110 us,
-// 63 TFLOP/s; the 64 x 64 scalar tiles before took 4 times as long.
+// (a warp reads 64 + 128 consecutive bytes per step), and at K = 128 the first
+// loads and the epilogue beside it, which nothing hides.  Launch list of a
+// 15-layer step, 212k x 128 x 128: NN 160 us (43 TFLOP/s), with the gathered rows
+// 203 (34), NT 204 (34), TN 135 (51); over all products of the step 36 TFLOP/s of
+// 80.5 at 2070 MHz.  The 64 x 64 scalar tiles before: 142 against 36.5 ms a step,
+// the split first edge layer included.
 // general_nnt_kernel / general_tn_kernel take what the 16-byte loads cannot:
 // widths, leading dimensions or bases that are not multiples of four floats
 // (the node encoder's six inputs, parameter vectors at odd addresses).
